@@ -291,6 +291,8 @@ def prepare(case, seed):
         arena.K.zero_()
         arena.V.zero_()
         state["arena"] = arena
+        state["out"] = {"K": arena.K.view(torch.int16), "V": arena.V.view(torch.int16), "acc": arena.acc(),
+                        "pos": arena.pos(), "count": arena.count(), "evicted": arena.evicted(), "lens": arena.lens()}
         if c["graph"]:
             _generate(state)  # the plan's first use sets up its device state, which a capture cannot
             torch.cuda.synchronize()
@@ -308,27 +310,25 @@ def prepare(case, seed):
         pre, _ = _route(c)
         state["scores"] = [_supplied_scores(c, seed, l) if pre[l] in (SNAPKV, H2O) else None for l in range(c["L"])]
         state["Q"] = None
+    bufs = state["bufs"]
+    state["out"] = {"K": bufs["out_K"].view(torch.int16), "V": bufs["out_V"].view(torch.int16),
+                    "idx": bufs["out_idx"], "count": bufs["out_count"], "h2o_state": bufs["h2o_state"]}
+    if c["kind"] != "scored":
+        state["out"]["scores"] = [plan.scores(bufs, c["B"], c["S_cap"], l) if state["Q"][l] is not None else None
+                                  for l in range(c["L"])]
     return state
 
 
 def run(state):
-    c, plan, bufs = state["case"], state["plan"], state["bufs"]
-    if c["kind"].startswith("decode"):
-        arena = state["arena"]
-        if c["graph"]:
-            state["graph"].replay()
-        else:
-            _generate(state)
-        return {"K": arena.K.view(torch.int16), "V": arena.V.view(torch.int16), "acc": arena.acc(), "pos": arena.pos(),
-                "count": arena.count(), "evicted": arena.evicted(), "lens": arena.lens()}
-    plan.evict_prefill(state["K"], state["V"], state["Q"], state["lens"], c["B"], c["S_cap"], bufs,
-                       scores=state.get("scores"), lse=state.get("lse"))
-    out = {"K": bufs["out_K"].view(torch.int16), "V": bufs["out_V"].view(torch.int16), "idx": bufs["out_idx"],
-           "count": bufs["out_count"], "h2o_state": bufs["h2o_state"]}
-    if c["kind"] != "scored":
-        out["scores"] = [plan.scores(bufs, c["B"], c["S_cap"], l) if state["Q"][l] is not None else None
-                         for l in range(c["L"])]
-    return out
+    c, plan = state["case"], state["plan"]
+    if not c["kind"].startswith("decode"):
+        plan.evict_prefill(state["K"], state["V"], state["Q"], state["lens"], c["B"], c["S_cap"], state["bufs"],
+                           scores=state.get("scores"), lse=state.get("lse"))
+    elif c["graph"]:
+        state["graph"].replay()
+    else:
+        _generate(state)
+    return state["out"]  # the caller's own buffers, which the call fills
 
 
 def work(case):
