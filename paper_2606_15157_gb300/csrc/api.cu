@@ -25,7 +25,8 @@ struct DevCtx {
   int device = -1;
   int num_sms = 0;
   int smem_optin = 0;
-  size_t score_smem_set = 0, h2o_full_smem_set = 0;
+  // dynamic shared memory each compiled variant was last set to
+  size_t score_smem_set[kScoreVariants] = {}, h2o_full_smem_set[2] = {};
   int* status = nullptr;
 };
 
@@ -162,7 +163,8 @@ int query_device(DevCtx& c, int dev) {
     return KVEV_ECUDA;
   if (major < 10) return KVEV_ENOTSUP;
   c.device = dev;
-  c.score_smem_set = c.h2o_full_smem_set = 0;
+  for (size_t& b : c.score_smem_set) b = 0;
+  for (size_t& b : c.h2o_full_smem_set) b = 0;
   return KVEV_OK;
 }
 
@@ -621,14 +623,15 @@ extern "C" int kvev_evict_prefill_lse(kvev_plan* plan, const void* const* K, con
 
 namespace {
 
-// 1 when the compiled score kernel for head size d is launched with enough
-// registers for its setmaxnreg split, 0 when not, -1 when the query failed.
-int score_regs_ok(int d) {
-  static std::once_flag once[2];
-  static int ok[2] = {-1, -1};
-  const int i = d == 64 ? 0 : 1;
+// 1 when the compiled score kernel for head size d and R_pad rows is launched
+// with enough registers for its setmaxnreg split, 0 when not, -1 when the
+// query failed.
+int score_regs_ok(int d, int R_pad) {
+  static std::once_flag once[kScoreVariants];
+  static int ok[kScoreVariants] = {-1, -1, -1, -1};
+  const int i = score_variant(d, R_pad);
   std::call_once(once[i], [&] {
-    const int regs = score_kernel_regs(d);
+    const int regs = score_kernel_regs(d, R_pad);
     ok[i] = regs < 0 ? -1 : (regs * kScoreThreads >= kRegsNeeded ? 1 : 0);
   });
   return ok[i];
@@ -743,14 +746,15 @@ int evict_impl(kvev_plan& P, DevCtx& D, const void* const* K, const void* const*
     // drawing on the registers the CTA was launched with; refuse to launch a
     // build whose allocation could not cover that (the raise would never
     // complete).
-    if (score_regs_ok(P.d) != 1) return KVEV_ENOTSUP;
+    if (score_regs_ok(P.d, ws.R_pad) != 1) return KVEV_ENOTSUP;
     // Request more than half of the SM's shared memory so exactly one CTA is
     // resident per SM: its TMEM allocation then never waits on another CTA.
     const size_t smem = std::max<size_t>(score_smem_bytes(P.d, q_rows, q_bufs, ws.R_pad, stages),
                                          static_cast<size_t>(D.smem_optin) / 2 + 1024);
-    if (D.score_smem_set != smem) {
-      if (score_set_smem(P.d, smem) != cudaSuccess) return KVEV_ECUDA;
-      D.score_smem_set = smem;
+    size_t& smem_set = D.score_smem_set[score_variant(P.d, ws.R_pad)];
+    if (smem_set != smem) {
+      if (score_set_smem(P.d, ws.R_pad, smem) != cudaSuccess) return KVEV_ECUDA;
+      smem_set = smem;
     }
     sp.n_units = ws.n_units;
     sp.B = B;
@@ -832,9 +836,10 @@ int evict_impl(kvev_plan& P, DevCtx& D, const void* const* K, const void* const*
     const size_t fsmem = std::max<size_t>(static_cast<size_t>(h2o_full_smem_bytes(P.d)),
                                           static_cast<size_t>(D.smem_optin) / 2 + 1024);
     if (fsmem + 1024 > static_cast<size_t>(D.smem_optin)) return KVEV_ENOTSUP;
-    if (D.h2o_full_smem_set != fsmem) {
+    size_t& fsmem_set = D.h2o_full_smem_set[P.d == 64 ? 0 : 1];
+    if (fsmem_set != fsmem) {
       if (h2o_full_set_smem(P.d, fsmem) != cudaSuccess) return KVEV_ECUDA;
-      D.h2o_full_smem_set = fsmem;
+      fsmem_set = fsmem;
     }
     if (lse_win) {  // the caller's every-row normalisers replace the row pass
       for (int j = 0; j < fp.n_h2o; ++j) fp.lse_src[j] = lse_win[P.score_layers[fp.h2o_slot[j]]];

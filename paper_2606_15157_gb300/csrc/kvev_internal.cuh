@@ -41,6 +41,10 @@ constexpr int kSlotCols = 128;        // fp32 columns per slot (4 x 128 = all 51
 constexpr int kRegsControl = 64;
 constexpr int kRegsSoftmax = 104;
 constexpr int kRegsNeeded = 128 * kRegsControl + 128 * kSoftmaxWGs * kRegsSoftmax;
+// The score kernel is compiled per head size (64, 128) and per number of
+// 128-row groups of the window rows (1, 2).
+constexpr int kScoreVariants = 4;
+constexpr int score_variant(int d, int R_pad) { return (d == 64 ? 0 : 1) + (R_pad > 128 ? 2 : 0); }
 constexpr int kSelectThreads = 256;    // one selection CTA per unit
 constexpr int kSelectCtasPerSm = 4;    // resident selection CTAs an SM should hold
 constexpr int kWsAlign = 256;
@@ -588,8 +592,8 @@ int score_smem_bytes(int d, int q_rows, int q_bufs, int R_pad, int stages);
 bool decode_supported(int d, int G);
 cudaError_t launch_decode_init(const DecodeParams& p, cudaStream_t s);
 cudaError_t launch_decode_step(const DecodeParams& p, size_t smem, cudaStream_t s);
-int score_kernel_regs(int d);
-cudaError_t score_set_smem(int d, size_t smem);
+int score_kernel_regs(int d, int R_pad);
+cudaError_t score_set_smem(int d, int R_pad, size_t smem);
 int h2o_full_smem_bytes(int d);
 int h2o_full_kernel_regs(int d);
 cudaError_t h2o_full_set_smem(int d, size_t smem);

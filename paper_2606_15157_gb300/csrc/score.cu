@@ -30,7 +30,7 @@
 // stages -lse2 for sweep 2; warpgroups 1-4 are softmax warpgroups.  The tensor
 // core fills 256-column TMEM units (two adjacent 128-column slots) in a ring
 // of two: sweep 1 one unit per (super-tile, 128-row group), sweep 2 one unit
-// per 128-key tile.  All four softmax warpgroups consume every unit, 64
+// per 128-key tile, or per two tiles when the rows fit 128 columns.  All four softmax warpgroups consume every unit, 64
 // columns each, copying them with one tcgen05.ld and releasing the unit
 // before any arithmetic.  setmaxnreg moves registers from warpgroup 0 to the
 // softmax warpgroups.
@@ -258,11 +258,10 @@ __device__ __forceinline__ void producer(const ScoreParams& p, const Smem& sm, i
 // MMA issuer (one warp; an elected lane issues): sweep 1 -> S = Q K^T,
 // sweep 2 -> S^T = K Q^T.
 // ---------------------------------------------------------------------------
-template <int D>
+template <int D, int NH>
 __device__ __forceinline__ void mma_issuer(const ScoreParams& p, const Smem& sm, uint32_t tmem_base, int first,
                            int stride, int J) {
   constexpr uint32_t kStageBytes = kSuperKeys * D * 2;
-  const int nh = p.R_pad > 128 ? 2 : 1;
   // sweep 1: S[128 rows of a group][256 keys of a super-tile]
   const uint32_t idesc1 = idesc_bf16_f32(128, kSuperKeys);
   // sweep 2: S^T[128 keys][every window row] (up to 256)
@@ -295,8 +294,10 @@ __device__ __forceinline__ void mma_issuer(const ScoreParams& p, const Smem& sm,
       // Work units of one super-tile, each a 256-column TMEM unit (two
       // slots) with one full and one empty barrier (those of its first
       // slot): sweep 1 -> one unit per 128-row group of Q, N = 256 keys;
-      // sweep 2 -> one unit per 128-key half, N = every window row.
-      const int nu = s1 ? nh : min(2, it.ntiles - 2 * j);
+      // sweep 2 -> one unit per 128-key half, N = every window row, or, when
+      // the rows fit one slot (NH = 1), one unit for both halves, a slot each.
+      const int halves = min(2, it.ntiles - 2 * j);
+      const int nu = s1 ? NH : NH == 2 ? halves : 1;
       for (int u = 0; u < nu; ++u) {
         if (!wait_bar_warp(&sm.tempty[sl], tph ^ 1, p)) { ok = false; break; }
         tc_fence_after();
@@ -309,11 +310,13 @@ __device__ __forceinline__ void mma_issuer(const ScoreParams& p, const Smem& sm,
             umma_bf16_elect(dcol, qdesc + a, kdesc + b, idesc1, k > 0);
           }
         } else {
-          const uint64_t adesc = kdesc + static_cast<uint64_t>(u * khalf);
+          for (int t2 = 0; t2 < (NH == 2 ? 1 : halves); ++t2) {
+            const uint64_t adesc = kdesc + static_cast<uint64_t>((NH == 2 ? u : t2) * khalf);
 #pragma unroll
-          for (int k = 0; k < D / 16; ++k) {
-            const uint32_t a = (k >> 2) * kcol_step + (k & 3) * 2, b = (k >> 2) * qcol_step + (k & 3) * 2;
-            umma_bf16_elect(dcol, adesc + a, qdesc0 + b, idesc2, k > 0);
+            for (int k = 0; k < D / 16; ++k) {
+              const uint32_t a = (k >> 2) * kcol_step + (k & 3) * 2, b = (k >> 2) * qcol_step + (k & 3) * 2;
+              umma_bf16_elect(dcol + t2 * kSlotCols, adesc + a, qdesc0 + b, idesc2, k > 0);
+            }
           }
         }
         umma_commit_elect(&sm.tfull[sl]);
@@ -340,64 +343,136 @@ __device__ __forceinline__ int row_pos(const ScoreParams& p, int r, int n) {
 }
 
 
-__device__ __forceinline__ void s2_chunk(const ScoreParams& p, const uint32_t (&rr)[32], bool full,
-                                         const float* nl, int r0, int k, int n, float2 (&a)[4]) {
-  const float c = p.scale_log2;
-  if (full) {
-    s2_chunk_full(rr, c, nl, a);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      const int r = r0 + i;
-      if (r < p.R && k <= row_pos(p, r, n)) {
-        const float e = ex2_approx(fmaf(__uint_as_float(rr[i]), c, lds1(nl + i)));
-        if (i & 1) a[(i >> 1) & 3].y += e; else a[(i >> 1) & 3].x += e;
-      }
-    }
-  }
-}
-
 // ---- TMEM unit hand-off ----------------------------------------------------
-// Every 256-column unit is consumed by all four softmax warpgroups:
-// warpgroup w copies its 64 columns and releases the unit at once (the
-// unit's empty barrier counts the 16 softmax warps: one elected lane arrives
-// for its warp, as a shared-memory barrier takes its arrivals one at a time),
-// so the tensor core refills it as soon as the last slice is copied and no
-// warpgroup holds TMEM while it computes.
+// Every 256-column unit is consumed by all four softmax warpgroups: a warp
+// copies its columns to registers and releases the unit at once (the unit's
+// empty barrier counts the 16 softmax warps: one elected lane arrives for its
+// warp, as a shared-memory barrier takes its arrivals one at a time), so the
+// tensor core refills it as soon as the last slice is copied and no warpgroup
+// holds TMEM while it computes.
 
 __device__ __forceinline__ bool slot_wait(const ScoreParams& p, const Smem& sm, uint32_t g, bool ok) {
   if (ok && !wait_bar(&sm.tfull[g & (kSlots - 1)], (g / kSlots) & 1, p)) ok = false;
   return ok;
 }
 
-
-// This warpgroup's 64 columns of a unit (the unit's two slots are 256
-// adjacent columns; warpgroup w takes [64w, 64w + 64)) in one load, released
-// (through the first slot's barrier) before any arithmetic.
-__device__ __forceinline__ void unit_take(const Smem& sm, uint32_t lane_base, uint32_t g, uint32_t (&r0)[32],
-                                          uint32_t (&r1)[32]) {
-  const uint32_t s0 = g & (kSlots - 1);
-  tmem_ld64_async(lane_base + s0 * kSlotCols, r0, r1);
-  tmem_wait64(r0, r1);
+__device__ __forceinline__ void unit_release(const Smem& sm, uint32_t g) {
   tc_fence_before();
   __syncwarp();
-  mbar_arrive_elect(&sm.tempty[s0]);
+  mbar_arrive_elect(&sm.tempty[g & (kSlots - 1)]);
 }
 
+// The units whose every key is visible to every row (all but the last few of a
+// prompt) run in loops of their own, without a branch per unit; the units at
+// the edges take masked versions.  Measured together with s2_unit_edge's
+// counted row index and the two-tile units of softmax_wg<1>, per launch, before
+// and after: one 8,192-token prompt, 32 rows x 4 heads 239 and 173 us (4.5 and
+// 6.2 TB/s of K for the two sweeps); one 30,011-token prompt, 64 x 4 627 and
+// 576 us; eight of 16K-32K 4.25 and 4.01 ms; with the normalisers supplied,
+// four of them 1.02 and 0.90 ms (6.1 TB/s, 0.91 of the measured copy rate).
+
+// Sweep 1: the thread's row of one 128-row group against this warpgroup's 64
+// keys k0 .. k0 + 63; with kMask only the keys its position tr can see.
+template <bool kMask>
+__device__ __forceinline__ void s1_unit(const ScoreParams& p, const Smem& sm, uint32_t taddr, uint32_t g, int k0,
+                                        int tr, float& m, float& z) {
+  uint32_t r0[32], r1[32];
+  tmem_ld64_async(taddr + (g & (kSlots - 1)) * kSlotCols, r0, r1);
+  tmem_wait64(r0, r1);
+  unit_release(sm, g);
+  float v0[32], v1[32];
+#pragma unroll
+  for (int q = 0; q < 32; ++q) {
+    v0[q] = __uint_as_float(r0[q]);
+    v1[q] = __uint_as_float(r1[q]);
+  }
+  if (kMask) {
+    mask_chunk(v0, k0, tr);
+    mask_chunk(v1, k0 + 32, tr);
+  }
+  s1_chunk64(v0, v1, p.scale_log2, m, z);
+}
+
+// Sweep 2: this thread's key against 64 (or 32) rows that all exist and all
+// see it; nl = -lse2 of the rows.
+__device__ __forceinline__ float s2_unit64(const ScoreParams& p, const Smem& sm, uint32_t taddr, uint32_t g,
+                                           const float* nl) {
+  uint32_t ra[32], rb[32];
+  tmem_ld64_async(taddr + (g & (kSlots - 1)) * kSlotCols, ra, rb);
+  tmem_wait64(ra, rb);
+  unit_release(sm, g);
+  float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  s2_chunk_full(ra, p.scale_log2, nl, a);
+  s2_chunk_full(rb, p.scale_log2, nl + 32, a);
+  return sum4x2(a);
+}
+
+__device__ __forceinline__ float s2_unit32(const ScoreParams& p, const Smem& sm, uint32_t taddr, uint32_t g,
+                                           const float* nl) {
+  uint32_t ra[32];
+  tmem_ld32_async(taddr + (g & (kSlots - 1)) * kSlotCols, ra);
+  tmem_wait32(ra);
+  unit_release(sm, g);
+  float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  s2_chunk_full(ra, p.scale_log2, nl, a);
+  return sum4x2(a);
+}
+
+// Sweep 2 at the edges: rows [r0, r0 + nrows) (nrows 64 or 32), of which only
+// those below R exist, against key k (k < n), which only rows at or past its
+// position see: row r sits at n - W + r % W.  A row that does not count gets
+// the exponent -inf.  r % W is counted up, not divided: with a division per
+// element the tiles at a prompt's end added 5 us to a 30 us chunk, and with
+// four chunks per unit and 152 CTAs a quarter of the CTAs are dealt every
+// unit's last chunk (they finished at 232 us, the others at 195 us).
+__device__ __forceinline__ float s2_unit_edge(const ScoreParams& p, const Smem& sm, uint32_t taddr, uint32_t g,
+                                              const float* nl, int r0, int nrows, int k, int n) {
+  float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  const int th = k < n ? k - (n - p.W) : p.W;  // rows with r % W >= th see the key
+  int i = r0 % p.W;
+#pragma unroll 1
+  for (int h = 0; h < nrows && r0 + h < p.R_pad; h += 32) {
+    uint32_t rr[32];
+    tmem_ld32_async(taddr + (g & (kSlots - 1)) * kSlotCols + h, rr);
+    tmem_wait32(rr);
+    const int exist = p.R - (r0 + h);  // rows of the chunk that exist
+#pragma unroll
+    for (int q = 0; q < 32; ++q) {
+      const float x = fmaf(__uint_as_float(rr[q]), p.scale_log2, lds1(nl + h + q));
+      const float e = ex2_approx(i >= th && q < exist ? x : -INFINITY);
+      if (q & 1) a[(q >> 1) & 3].y += e; else a[(q >> 1) & 3].x += e;
+      i = i + 1 == p.W ? 0 : i + 1;
+    }
+  }
+  unit_release(sm, g);
+  return sum4x2(a);
+}
+
+// NH: 128-row groups of the window rows (R_pad <= 128 NH).  Sweep 2 units hold
+// one 128-key tile x up to 256 rows (NH = 2), of which warpgroup w takes rows
+// [64w, 64w + 64), or two tiles x up to 128 rows (NH = 1), of which warpgroup
+// w takes tile w / 2 and half w % 2 of the rows.  (With one tile per unit at
+// NH = 1, half of the warpgroups would have no rows.)
+template <int NH>
 __device__ __forceinline__ void softmax_wg(const ScoreParams& p, const Smem& sm, uint32_t tmem_base,
                                            int wg, int first, int stride, int J) {
+  constexpr int kPack = NH == 2 ? 1 : 2;                // key tiles per sweep-2 unit
+  constexpr int kParts = kSoftmaxWGs / kPack;           // partial sums per key
+  constexpr int kBatch = kRedTiles * kPack;             // tiles whose partials sm.red holds
   const int warp = threadIdx.x >> 5;
   const int quarter = warp & 3;                        // TMEM lane quarter of this warp
   const int lrow = quarter * 32 + (threadIdx.x & 31);  // TMEM lane: row (sweep 1) / key (sweep 2)
   const int stid = threadIdx.x - 128;                  // 0..511 over the softmax warpgroups
-  const int nh = p.R_pad > 128 ? 2 : 1;                // 128-row groups (slots) per tile
-  // this warpgroup's 64 columns of every 256-column unit
-  const uint32_t lane_base =
-      tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(64 * wg);
-  // sweep 2: this warpgroup's rows [64wg, 64wg + 32) and [64wg + 32, 64wg + 64)
-  const int r0a = 64 * wg, r0b = 64 * wg + 32;
-  const bool has_a = r0a < p.R_pad;
-  const bool has_b = r0b < p.R_pad;
+  const uint32_t lanes = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
+  const uint32_t t1 = lanes + static_cast<uint32_t>(64 * wg);  // sweep 1: 64 of the unit's 256 keys
+  // whether any of the warp's lanes holds a row of the last 128-row group
+  const bool live = (NH - 1) * 128 + quarter * 32 < p.R_pad;
+  const int tsub = NH == 2 ? 0 : wg >> 1;              // sweep 2: tile of the unit
+  const int part = NH == 2 ? wg : wg & 1;              // and part of its rows
+  const int nrows = NH == 2 || p.R_pad > 64 ? 64 : 32;
+  const int r0 = part * nrows;
+  const uint32_t t2 = lanes + static_cast<uint32_t>(tsub * kSlotCols + r0);
+  const bool rows_full = r0 + nrows <= p.R, rows_none = r0 >= p.R_pad;
   uint32_t g = 0;     // slot stream position (advances 2 per 256-column unit)
   uint32_t q1 = 0, q2 = 0;  // sweep-1 / sweep-2 entries done
   bool ok = true;
@@ -412,35 +487,35 @@ __device__ __forceinline__ void softmax_wg(const ScoreParams& p, const Smem& sm,
       const ItemInfo it = decode_item(p, t, load_item(p, t));
       float m0 = -INFINITY, z0 = 0.f, m1 = -INFINITY, z1 = 0.f;
       const int tr0 = lrow < p.R ? row_pos(p, lrow, it.n) : -1;
-      const int tr1 = 128 + lrow < p.R ? row_pos(p, 128 + lrow, it.n) : -1;
-      // One unit per (256-key super-tile, 128-row group): this warpgroup's 32
-      // keys of each 128-key half, for the thread's row of the group.  Rows
-      // that do not exist (tr < 0) are computed like the others and dropped
-      // when the warpgroup publishes.
+      const int tr1 = NH == 2 && 128 + lrow < p.R ? row_pos(p, 128 + lrow, it.n) : -1;
+      // One unit per (256-key super-tile, 128-row group): this warpgroup's 64
+      // keys of the super-tile, for the thread's row of the group.  Rows that
+      // do not exist (tr < 0) are computed like the others and dropped when
+      // the warpgroup publishes; a warp without rows only releases the unit.
       const int nst = (it.ntiles + 1) / 2;
-      for (int j = 0; j < nst; ++j) {
-        const int kb = it.key0 + j * kSuperKeys;
-        const int k0 = kb + 64 * wg;                       // keys k0 .. k0 + 63
-        const bool full = kb + kSuperKeys - 1 <= it.n - p.W;  // every key visible to every row
-        for (int h = 0; h < nh; ++h) {
+      // the super-tiles whose every key is visible to every row come first
+      const int nfull = min(nst, max(0, it.n - p.W + 1 - it.key0) / kSuperKeys);
+      int k0 = it.key0 + 64 * wg;
+      for (int j = 0; j < nfull; ++j, k0 += kSuperKeys) {
+        ok = slot_wait(p, sm, g, ok);
+        if (NH == 2 || live) s1_unit<false>(p, sm, t1, g, k0, tr0, m0, z0);
+        else unit_release(sm, g);
+        g += 2;
+        if (NH == 2) {
           ok = slot_wait(p, sm, g, ok);
-          uint32_t r0[32], r1[32];
-          unit_take(sm, lane_base, g, r0, r1);
-          float v0[32], v1[32];
-#pragma unroll
-          for (int q = 0; q < 32; ++q) {
-            v0[q] = __uint_as_float(r0[q]);
-            v1[q] = __uint_as_float(r1[q]);
-          }
-          const int tr = h == 0 ? tr0 : tr1;
-          if (!full) {
-            mask_chunk(v0, k0, tr);
-            mask_chunk(v1, k0 + 32, tr);
-          }
-          if (h == 0)
-            s1_chunk64(v0, v1, p.scale_log2, m0, z0);
-          else
-            s1_chunk64(v0, v1, p.scale_log2, m1, z1);
+          if (live) s1_unit<false>(p, sm, t1, g, k0, tr1, m1, z1);
+          else unit_release(sm, g);
+          g += 2;
+        }
+      }
+#pragma unroll 1
+      for (int j = nfull; j < nst; ++j, k0 += kSuperKeys) {
+#pragma unroll 1
+        for (int h = 0; h < NH; ++h) {
+          ok = slot_wait(p, sm, g, ok);
+          float m = h == 0 ? m0 : m1, z = h == 0 ? z0 : z1;
+          s1_unit<true>(p, sm, t1, g, k0, h == 0 ? tr0 : tr1, m, z);
+          if (h == 0) { m0 = m; z0 = z; } else { m1 = m; z1 = z; }
           g += 2;
         }
       }
@@ -448,7 +523,7 @@ __device__ __forceinline__ void softmax_wg(const ScoreParams& p, const Smem& sm,
       if (!wait_bar(&sm.pempty[0], (q1 & 1) ^ 1, p)) ok = false;
       const float2 none = make_float2(-INFINITY, 0.f);
       if (lrow < p.R_pad) sm.pc[wg * p.R_pad + lrow] = tr0 >= 0 && ok ? make_float2(m0, z0) : none;
-      if (nh == 2 && 128 + lrow < p.R_pad)
+      if (NH == 2 && 128 + lrow < p.R_pad)
         sm.pc[wg * p.R_pad + 128 + lrow] = tr1 >= 0 && ok ? make_float2(m1, z1) : none;
       __syncwarp();
       mbar_arrive_elect(&sm.pfull[0]);
@@ -461,48 +536,55 @@ __device__ __forceinline__ void softmax_wg(const ScoreParams& p, const Smem& sm,
       // -lse2 of the unit, loaded ahead by the normaliser warp
       const uint32_t lb = q2 & 1;
       if (!wait_bar(&sm.lfull[lb], (q2 >> 1) & 1, p)) ok = false;
-      const float* lam = sm.lam + lb * p.R_pad;
-      float* out = p.raw + static_cast<size_t>(it.u) * p.S_cap;
-      for (int i = 0; i < it.ntiles; ++i) {
-        const int kb = it.key0 + i * kTileKeys;
-        const int k = kb + lrow;
-        const bool key_full = kb + kTileKeys - 1 <= it.n - p.W;
-        float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f),
-                       make_float2(0.f, 0.f)};
-        ok = slot_wait(p, sm, g, ok);
-        {
-          uint32_t ra[32], rb[32];
-          unit_take(sm, lane_base, g, ra, rb);
-          if (ok && key_full && r0b + 32 <= p.R) {  // the common case: every key and row counts
-            s2_chunk_full(ra, p.scale_log2, lam + r0a, a);
-            s2_chunk_full(rb, p.scale_log2, lam + r0b, a);
-          } else {
-            if (ok && has_a && k < it.n)
-              s2_chunk(p, ra, key_full && r0a + 32 <= p.R, lam + r0a, r0a, k, it.n, a);
-            if (ok && has_b && k < it.n)
-              s2_chunk(p, rb, key_full && r0b + 32 <= p.R, lam + r0b, r0b, k, it.n, a);
+      const float* lam = sm.lam + lb * p.R_pad + r0;
+      float* out = p.raw + static_cast<size_t>(it.u) * p.S_cap + it.key0;
+      const int nkeys = it.n - it.key0;  // keys of the unit from the item's first on
+      // units whose every key is visible to every row come first
+      const int nfull = max(0, nkeys - p.W + 1) / (kTileKeys * kPack);
+      const int nunits = (it.ntiles + kPack - 1) / kPack;
+      // Each warpgroup keeps its partial sum of every key of a batch of kBatch
+      // tiles in its own shared-memory rows; at the end of the batch the
+      // kParts partials are added (in row order) and stored, with one barrier
+      // on either side instead of a hand-off per tile.
+      for (int u0 = 0; u0 < nunits; u0 += kRedTiles) {
+        const int u1 = min(u0 + kRedTiles, nunits);
+        const int uf = rows_full ? min(u1, nfull) : u0;  // units of the common case: every key and row counts
+        float* red = sm.red + (part * kBatch + tsub) * 128 + lrow;
+        int u = u0;
+        if (NH == 2 || nrows == 64) {
+          for (; u < uf; ++u, g += 2, red += 128 * kPack) {
+            ok = slot_wait(p, sm, g, ok);
+            *red = s2_unit64(p, sm, t2, g, lam);
+          }
+        } else {
+          for (; u < uf; ++u, g += 2, red += 128 * kPack) {
+            ok = slot_wait(p, sm, g, ok);
+            *red = s2_unit32(p, sm, t2, g, lam);
           }
         }
-        g += 2;
-        // Each warpgroup keeps its partial sum of every key of a batch of
-        // kRedTiles tiles in its own shared-memory rows; at the end of the
-        // batch all four are added (in warpgroup order) and stored, with one
-        // barrier on either side instead of a hand-off per tile.
-        const int bt = i % kRedTiles;
-        sm.red[(wg * kRedTiles + bt) * 128 + lrow] = sum4x2(a);
-        if (bt == kRedTiles - 1 || i == it.ntiles - 1) {
-          named_bar_sync(1, 128 * kSoftmaxWGs);
-          const int key0 = it.key0 + (i - bt) * kTileKeys;
-          for (int q = stid; q < (bt + 1) * 128; q += 128 * kSoftmaxWGs) {
-            float sum = 0.f;
+#pragma unroll 1
+        for (; u < u1; ++u, g += 2, red += 128 * kPack) {
+          ok = slot_wait(p, sm, g, ok);
+          const int k = (u * kPack + tsub) * kTileKeys + lrow;  // this thread's key, from the item's first
+          float sum = 0.f;
+          if (rows_none || k - lrow >= nkeys)
+            unit_release(sm, g);
+          else
+            sum = s2_unit_edge(p, sm, t2, g, lam, r0, nrows, it.key0 + k, it.n);
+          *red = sum;
+        }
+        named_bar_sync(1, 128 * kSoftmaxWGs);
+        const int kb = u0 * kPack * kTileKeys;
+        const int nk = min(nkeys - kb, (u1 - u0) * kPack * kTileKeys);
+        for (int q = stid; q < nk; q += 128 * kSoftmaxWGs) {
+          float total = 0.f;
 #pragma unroll
-            for (int w = 0; w < kSoftmaxWGs; ++w) sum += sm.red[w * kRedTiles * 128 + q];
-            if (ok && key0 + q < it.n) out[key0 + q] = sum * p.inv_G;
-          }
-          // the batch's rows may be overwritten, and after the entry's last
-          // batch every warpgroup is done reading lam
-          named_bar_sync(1, 128 * kSoftmaxWGs);
+          for (int w = 0; w < kParts; ++w) total += sm.red[w * kBatch * 128 + q];
+          if (ok) out[kb + q] = total * p.inv_G;
         }
+        // the batch's rows may be overwritten, and after the entry's last
+        // batch every warpgroup is done reading lam
+        named_bar_sync(1, 128 * kSoftmaxWGs);
       }
       if (stid == 0) mbar_arrive(&sm.lempty[lb]);
       ++q2;
@@ -645,7 +727,7 @@ __device__ __forceinline__ void lam_loader(const ScoreParams& p, const Smem& sm,
   }
 }
 
-template <int D>
+template <int D, int NH>
 __global__ void __launch_bounds__(kScoreThreads, 1) score_kernel(const __grid_constant__ ScoreParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   if (smem_u32(smem_raw) & 1023u) {  // the 128-byte swizzle needs 1024-byte aligned tiles
@@ -694,12 +776,12 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_kernel(const __grid_co
   if (warp < 4) {
     regs_dealloc<kRegsControl>();
     if (warp == 0 && (threadIdx.x & 31) == 0) producer<D>(p, sm, first, stride, J);
-    if (warp == 1) mma_issuer<D>(p, sm, tmem_base, first, stride, J);  // whole warp
+    if (warp == 1) mma_issuer<D, NH>(p, sm, tmem_base, first, stride, J);  // whole warp
     if (warp == 2) publisher(p, sm, first, stride, J);                 // whole warp
     if (warp == 3) lam_loader(p, sm, first, stride, J);                // whole warp
   } else {
     regs_alloc<kRegsSoftmax>();
-    softmax_wg(p, sm, tmem_base, (warp - 4) >> 2, first, stride, J);  // warpgroups 0..3
+    softmax_wg<NH>(p, sm, tmem_base, (warp - 4) >> 2, first, stride, J);  // warpgroups 0..3
   }
   tc_fence_before();
   __syncthreads();
@@ -842,18 +924,22 @@ int score_smem_bytes(int d, int q_rows, int q_bufs, int R_pad, int stages) {
   return static_cast<int>((off + 127) & ~size_t(127));
 }
 
-int score_kernel_regs(int d) {
+namespace {
+using ScoreFn = void (*)(const ScoreParams);
+// The score kernel of head size d (64 or 128) and R_pad window rows.
+ScoreFn score_fn(int d, int R_pad) {
+  if (d == 64) return R_pad > 128 ? score_kernel<64, 2> : score_kernel<64, 1>;
+  return R_pad > 128 ? score_kernel<128, 2> : score_kernel<128, 1>;
+}
+}  // namespace
+
+int score_kernel_regs(int d, int R_pad) {
   cudaFuncAttributes a = {};
-  const cudaError_t e = d == 64 ? cudaFuncGetAttributes(&a, score_kernel<64>)
-                                : cudaFuncGetAttributes(&a, score_kernel<128>);
-  return e == cudaSuccess ? a.numRegs : -1;
+  return cudaFuncGetAttributes(&a, score_fn(d, R_pad)) == cudaSuccess ? a.numRegs : -1;
 }
 
-cudaError_t score_set_smem(int d, size_t smem) {
-  if (d == 64)
-    return cudaFuncSetAttribute(score_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(smem));
-  return cudaFuncSetAttribute(score_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+cudaError_t score_set_smem(int d, int R_pad, size_t smem) {
+  return cudaFuncSetAttribute(score_fn(d, R_pad), cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(smem));
 }
 
@@ -876,8 +962,7 @@ cudaError_t launch_score(const ScoreParams& p, int d, int grid, size_t smem, cud
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (d == 64) return cudaLaunchKernelEx(&cfg, score_kernel<64>, p);
-  return cudaLaunchKernelEx(&cfg, score_kernel<128>, p);
+  return cudaLaunchKernelEx(&cfg, score_fn(d, p.R_pad), p);
 }
 
 }  // namespace kvev

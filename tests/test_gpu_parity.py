@@ -277,6 +277,20 @@ def test_edge_window_and_groups(torch, orc):
         parity.check_workload(wl, dev, wl.lens)
 
 
+@pytest.mark.parametrize("H_q,H_kv,W,d", [(2, 2, 8, 64), (4, 2, 16, 128), (6, 2, 16, 128), (4, 2, 32, 64),
+                                          (6, 2, 32, 128), (4, 1, 33, 64), (4, 1, 40, 128), (8, 2, 63, 128)])
+def test_score_tile_edges(torch, orc, H_q, H_kv, W, d):
+    # R = G*W = 8, 32, 48, 64, 96 (two key tiles per sweep-2 unit), 132, 160 and
+    # 252 rows (one), with prompts that end around the edges of the window, a
+    # 128-key tile, a 256-key super-tile and a chunk: an odd last tile, the
+    # last tile all past the window's first key, and none of it.
+    lens = [1, W - 1, W, W + 1, 127, 128 + W - 1, 128 + W, 256 + W - 2, 256 + W - 1, 256 + W, 383, 2048, 2049,
+            2048 + W, 2176 + W]
+    wl = _custom([gen.SNAPKV, gen.H2O], [W + 9, 20], lens, W=W, d=d, H_q=H_q, H_kv=H_kv, pool=(7, gen.POOL_AVG),
+                 S_cap=2304)
+    parity.check_workload(wl, device_workload(wl), wl.lens)
+
+
 def test_h2o_recent_override_and_ties(torch, orc):
     # h2o_recent = 0 (pure heavy hitters) and = b (pure recency); plus all-zero
     # queries so every score in a row ties and the lower-position rule decides.
