@@ -1108,6 +1108,11 @@ extern "C" int kvev_decode_init(kvev_plan* plan, int B, int growth, const void* 
   dp.pre_count = pre_count;
   dp.h2o_state = h2o_state;
   dp.lens_in = lens_dev;
+  // eight CTAs per SM keep enough of the copy in flight: few units are split
+  // over several, each of at least 64 slots
+  int cap = 0;
+  for (int l = 0; l < P.L; ++l) cap = std::max(cap, d.cap[l]);
+  dp.init_split = std::max(1, std::min((8 * P.ctx.num_sms + d.units - 1) / d.units, cap / 64));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   P.last_stream = s;
   return launch_decode_init(dp, s) == cudaSuccess ? KVEV_OK : KVEV_ECUDA;

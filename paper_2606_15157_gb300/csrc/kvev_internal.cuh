@@ -174,6 +174,7 @@ struct DecodeParams {
   const float* attn[kMaxLayers];  // [B][H_kv][cap + 1] caller-supplied attention, or null
   int L, B, H_kv, H_q, G, d, units;
   int n_att, n_cheap; // attending units; StreamingLLM and append-only units
+  int init_split;     // CTAs per unit of the initialisation
   float scale_log2;   // log2(e) / sqrt(d)
   void* K;            // arena rows [rows][d] bf16
   void* V;
