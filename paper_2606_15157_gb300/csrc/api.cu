@@ -986,6 +986,7 @@ int dec_params(const kvev_plan& P, int B, const DecLayout& d, DecodeParams& dp) 
   dp.units = d.units;
   dp.scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(P.d)));
   int64_t pre_off = 0;
+  int n_att_layers = 0, n_cheap_layers = 0;
   for (int l = 0; l < P.L; ++l) {
     DecLayer& y = dp.layer[l];
     const int md = P.route_dec[l], b = P.budget[l];
@@ -998,13 +999,14 @@ int dec_params(const kvev_plan& P, int B, const DecLayout& d, DecodeParams& dp) 
     y.pre_slots = P.slots[l];
     y.pre_row_off = pre_off;
     pre_off += rows_per_layer(P, B, l);
-    if (y.cap > 0 && (md == KVEV_H2O || md == KVEV_TOVA))
-      dp.n_att += B * P.H_kv;
-    else if (y.cap > 0)
-      dp.n_cheap += B * P.H_kv;
-    y.att_end = dp.n_att;
-    y.cheap_end = dp.n_cheap;
     if (y.cap == 0) continue;
+    if (md == KVEV_H2O || md == KVEV_TOVA) {
+      dp.att_layer[n_att_layers++] = static_cast<uint8_t>(l);
+      dp.n_att += B * P.H_kv;
+    } else {
+      dp.cheap_layer[n_cheap_layers++] = static_cast<uint8_t>(l);
+      dp.n_cheap += B * P.H_kv;
+    }
     if (md == KVEV_H2O || md == KVEV_TOVA) {
       y.r = md == KVEV_TOVA ? 0 : (P.h2o_recent < 0 ? b / 2 : P.h2o_recent);
       if (b < 1 || y.r >= b) return KVEV_EINVAL;  // at least one slot must be evictable
@@ -1017,16 +1019,30 @@ int dec_params(const kvev_plan& P, int B, const DecLayout& d, DecodeParams& dp) 
   return KVEV_OK;
 }
 
-// Shared memory of the step kernel: the logits of the largest H2O/TOVA unit.
-// Dynamic shared memory of a decode step: G rows of logits per slot, or one
-// row (the new keys) when the attention is supplied.
-size_t dec_smem(const kvev_plan& P, const DecLayout& d, bool supplied_attention = false) {
+// Slots of the largest H2O / TOVA unit (0: the route has none).
+int dec_att_cap(const kvev_plan& P, const DecLayout& d) {
   int cap = 0;
   for (int l = 0; l < P.L; ++l)
     if (d.cap[l] > 0 && (P.route_dec[l] == KVEV_H2O || P.route_dec[l] == KVEV_TOVA))
       cap = std::max(cap, d.cap[l]);
-  const size_t rows = supplied_attention ? 1 : static_cast<size_t>(P.G);
-  return cap == 0 ? 0 : sizeof(float) * rows * (cap + 1);
+  return cap;
+}
+
+// CTAs per H2O / TOVA unit (a cluster): a unit's K rows are a serial chain of
+// load round trips for one CTA (16 slots per warp and trip), so while the units
+// leave CTA slots of the GPU empty each is split, as long as every warp still
+// has a tile of 16 slots.  At most three CTAs per SM, of the four that fit:
+// with more, the last clusters of eight found no GPC with eight free slots and
+// ran as a second wave (18.8 against 13.6 us at batch 1).  Not with the
+// attention supplied: a unit is then a few loads per thread, and the cluster's
+// barriers cost what the split gains (batch 1: 6.4 against 5.8 us at 512
+// slots).  Measured per step, 32 layers of which 7 are H2O with 2,048 slots, 8
+// KV heads, one CTA per unit and split: batch 1 24.5 and 13.7 us (eight CTAs),
+// batch 2 26.4 and 19.3 (four), batch 4 31.6 and 29.0 (two).
+int dec_cluster(int n_att, int cap, int num_sms) {
+  int c = kMaxDecCluster;
+  while (c > 1 && (static_cast<int64_t>(n_att) * c > 3 * static_cast<int64_t>(num_sms) || cap < 16 * 8 * c)) c >>= 1;
+  return c;
 }
 
 void set_state_ptrs(DecodeParams& dp, const DecLayout& d, void* dec_K, void* dec_V, void* state) {
@@ -1147,18 +1163,24 @@ int decode_step_impl(kvev_plan* plan, int B, int growth, void* dec_K, void* dec_
     const bool attends = P.route_dec[l] == KVEV_H2O || P.route_dec[l] == KVEV_TOVA;
     if (attends && attn) {
       if (!attn[l] || (reinterpret_cast<uintptr_t>(attn[l]) & 3u)) return KVEV_EINVAL;
-      dp.attn[l] = attn[l];
+      dp.layer[l].attn = attn[l];
     } else if (attends && (!q_new[l] || !aligned16(q_new[l]))) {
       return KVEV_EINVAL;
     }
-    dp.k_new[l] = k_new[l];
-    dp.v_new[l] = v_new[l];
-    dp.q_new[l] = q_new ? q_new[l] : nullptr;
+    dp.layer[l].k_new = k_new[l];
+    dp.layer[l].v_new = v_new[l];
+    dp.layer[l].q_new = q_new ? q_new[l] : nullptr;
   }
   rc = ensure_device(plan);
   if (rc != KVEV_OK) return rc;
-  const size_t smem = dec_smem(P, d, attn != nullptr);
-  if (smem + 1024 > static_cast<size_t>(P.ctx.smem_optin)) return KVEV_ENOTSUP;
+  // logits of a unit: G rows per slot, or one row (the new keys) when the
+  // attention is supplied; a unit must fit one CTA, however it is split
+  const int cap = dec_att_cap(P, d), rows = attn ? 1 : P.G;
+  if (cap > 0 && sizeof(float) * static_cast<size_t>(rows) * (cap + 1) + 1024 >
+                     static_cast<size_t>(P.ctx.smem_optin))
+    return KVEV_ENOTSUP;
+  dp.cluster = cap > 0 && !attn ? dec_cluster(dp.n_att, cap, P.ctx.num_sms) : 1;
+  const size_t smem = cap > 0 ? decode_logit_bytes(cap, rows, dp.cluster) : 0;
   set_state_ptrs(dp, d, dec_K, dec_V, dec_state);
   dp.status = P.ctx.status;
   cudaStream_t s = static_cast<cudaStream_t>(stream);

@@ -12,8 +12,10 @@
 // the last step's attention).  Slot order carries no meaning: an evicted
 // slot is overwritten by the new token.
 //
-// One CTA per H2O / TOVA unit, and one warp per StreamingLLM or append-only
-// unit (eight per CTA).  H2O / TOVA: the G query rows of the new token attend to
+// One CTA per H2O / TOVA unit, or a cluster of up to eight when there are few
+// units (each CTA takes a run of 16-slot tiles; the softmax normalisers and the
+// eviction candidates cross the cluster through distributed shared memory),
+// and one warp per StreamingLLM or append-only unit (eight per CTA).  H2O / TOVA: the G query rows of the new token attend to
 // every retained slot and to the new token, p_j = (1/G) sum_g softmax_j(q_g .
 // k_j / sqrt(d)); acc += p (H2O) or acc = p (TOVA).  When the unit already
 // holds b slots, the slot with the smallest acc among positions older than
@@ -43,33 +45,73 @@ __device__ __forceinline__ int find_dec_layer(const DecodeParams& p, int u) {
   return lo;
 }
 
-struct DecShared {
-  float f[kDecodeThreads / 32];
-  int i[2 * (kDecodeThreads / 32)];
-  float g[8][kDecodeThreads / 32];  // per-head partials of the G <= 8 query heads
+// A CTA's eviction candidate (slot -1: none) and, from the CTA that holds the
+// new token's index, the new token's key.
+struct __align__(16) DecCandidate {
+  float key;
+  int pos, slot;
+  float new_key;
 };
 
-// Block-wide max (kMax) or sum of G values per thread, all heads in one
-// exchange: warp shuffles, then one shared-memory round.
-template <int G, bool kMax>
-__device__ __forceinline__ void block_reduce_heads(float (&v)[G], DecShared& sh) {
-#pragma unroll
-  for (int g = 0; g < G; ++g)
-    for (int o = 16; o > 0; o >>= 1) {
-      const float y = __shfl_xor_sync(0xffffffffu, v[g], o);
-      v[g] = kMax ? fmaxf(v[g], y) : v[g] + y;
-    }
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0)
-#pragma unroll
-    for (int g = 0; g < G; ++g) sh.g[g][threadIdx.x >> 5] = v[g];
-  __syncthreads();
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    float r = sh.g[g][0];
-    for (int w = 1; w < kDecodeThreads / 32; ++w) r = kMax ? fmaxf(r, sh.g[g][w]) : r + sh.g[g][w];
-    v[g] = r;
-  }
+constexpr int kDecodeWarps = kDecodeThreads / 32;
+
+// Every array is written once per step and read after one barrier.
+template <bool kSplit>
+struct DecShared {
+  static constexpr int kC = kSplit ? kMaxDecCluster : 1;
+  DecCandidate cand[kC];        // of every CTA of the cluster
+  float cm[kC][8], cz[kC][8];   // their per-head (max, sum)
+  __align__(16) float wmax[8][kDecodeWarps];  // per-head maxima of this CTA's warps (G <= 8 heads)
+  __align__(16) float wsum[8][kDecodeWarps];  // and sums
+  DecCandidate wcand[kDecodeWarps];           // their eviction candidates
+};
+static_assert(sizeof(DecShared<false>) <= 1024, "the host leaves 1 KiB beside the logits");
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+
+// Every thread of the cluster: what was stored to shared memory (its own or
+// another CTA's) before is visible after.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// A CTA may store into another one only once that one has started: every
+// thread arrives when its unit's step begins and waits before the first store.
+__device__ __forceinline__ void cluster_started_arrive() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_started_wait() {
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
+
+// The address of this CTA's shared-memory object in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+
+__device__ __forceinline__ void st_cluster(uint32_t addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+
+__device__ __forceinline__ void st_cluster(uint32_t addr, const DecCandidate& c) {
+  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(__float_as_int(c.key)),
+               "r"(c.pos), "r"(c.slot), "r"(__float_as_int(c.new_key))
+               : "memory");
+}
+
+// The maximum (kMax) or sum, over the warps, of one head's per-warp values.
+template <bool kMax>
+__device__ __forceinline__ float over_warps(const float (&w)[kDecodeWarps]) {
+  static_assert(kDecodeWarps == 8, "two 16-byte loads");
+  const float4 a = lds4(w), b = lds4(w + 4);
+  return kMax ? fmaxf(fmaxf(fmaxf(a.x, a.y), fmaxf(a.z, a.w)), fmaxf(fmaxf(b.x, b.y), fmaxf(b.z, b.w)))
+              : ((((((a.x + a.y) + a.z) + a.w) + b.x) + b.y) + b.z) + b.w;
 }
 
 // Eviction order: smaller key first, then higher position first.
@@ -77,10 +119,10 @@ __device__ __forceinline__ bool evict_before(float a, int pa, float b, int pb) {
   return a < b || (a == b && pa > pb);
 }
 
-// Block-wide first candidate in eviction order (candidates have pos >= 0);
-// returns its slot, -1 if there is none.
-__device__ __forceinline__ int block_evict_choice(float a, int pos, int slot, DecShared& sh) {
-  for (int o = 16; o > 0; o >>= 1) {
+// The first candidate in eviction order (candidates have pos >= 0) over lanes
+// that differ in the bits of `lanes` (a power of two, exclusive), in each.
+__device__ __forceinline__ void warp_evict_choice(float& a, int& pos, int& slot, int lanes) {
+  for (int o = lanes >> 1; o > 0; o >>= 1) {
     const float a2 = __shfl_xor_sync(0xffffffffu, a, o);
     const int p2 = __shfl_xor_sync(0xffffffffu, pos, o);
     const int s2 = __shfl_xor_sync(0xffffffffu, slot, o);
@@ -90,25 +132,20 @@ __device__ __forceinline__ int block_evict_choice(float a, int pos, int slot, De
       slot = s2;
     }
   }
+}
+
+// Block-wide first candidate, in every thread; slot -1 if there is none.
+__device__ __forceinline__ void block_evict_choice(float& a, int& pos, int& slot, DecCandidate (&wcand)[kDecodeWarps]) {
+  const int lane = threadIdx.x & 31;
+  warp_evict_choice(a, pos, slot, 32);
+  if (lane == 0) wcand[threadIdx.x >> 5] = DecCandidate{a, pos, slot, 0.f};
   __syncthreads();
-  if ((threadIdx.x & 31) == 0) {
-    const int w = threadIdx.x >> 5;
-    sh.f[w] = a;
-    sh.i[2 * w] = pos;
-    sh.i[2 * w + 1] = slot;
-  }
-  __syncthreads();
-  float ba = sh.f[0];
-  int bp = sh.i[0], bs = sh.i[1];
-  for (int i = 1; i < kDecodeThreads / 32; ++i) {
-    const int pi = sh.i[2 * i];
-    if (pi >= 0 && (bp < 0 || evict_before(sh.f[i], pi, ba, bp))) {
-      ba = sh.f[i];
-      bp = pi;
-      bs = sh.i[2 * i + 1];
-    }
-  }
-  return bp < 0 ? -1 : bs;
+  const DecCandidate d = wcand[lane & (kDecodeWarps - 1)];
+  a = d.key;
+  pos = d.pos;
+  slot = d.slot;
+  warp_evict_choice(a, pos, slot, kDecodeWarps);
+  if (pos < 0) slot = -1;
 }
 
 // Copy one d-wide bf16 row (16-byte vectors) with the whole block.
@@ -122,24 +159,16 @@ struct UnitRef {
   size_t rows0;  // first slot row of the unit
 };
 
-// Put the new token into slot dst (its K/V row, position n, key acc_new) and
-// finish the unit's bookkeeping.  Called by the whole block.
-__device__ __forceinline__ void place_new(const DecodeParams& p, const UnitRef& r, int D, int dst, int n,
-                                          float acc_new, int new_count, int evicted_pos) {
-  if (dst >= 0) {
-    const size_t src = static_cast<size_t>(r.s) * p.H_kv + r.h;
-    copy_row(static_cast<uint16_t*>(p.K) + (r.rows0 + dst) * D,
-             static_cast<const uint16_t*>(p.k_new[r.l]) + src * D, D);
-    copy_row(static_cast<uint16_t*>(p.V) + (r.rows0 + dst) * D,
-             static_cast<const uint16_t*>(p.v_new[r.l]) + src * D, D);
-  }
+// Put the new token into slot dst: its K/V row, position n and key.  Called by
+// the whole block.
+__device__ __forceinline__ void place_new(const DecodeParams& p, const DecLayer& ly, const UnitRef& r, int D, int dst,
+                                          int n, float new_key) {
+  const size_t src = static_cast<size_t>(r.s) * p.H_kv + r.h;
+  copy_row(static_cast<uint16_t*>(p.K) + (r.rows0 + dst) * D, static_cast<const uint16_t*>(ly.k_new) + src * D, D);
+  copy_row(static_cast<uint16_t*>(p.V) + (r.rows0 + dst) * D, static_cast<const uint16_t*>(ly.v_new) + src * D, D);
   if (threadIdx.x == 0) {
-    if (dst >= 0) {
-      p.pos[r.rows0 + dst] = n;
-      p.acc[r.rows0 + dst] = acc_new;
-    }
-    p.count[r.u] = new_count;
-    p.evicted[r.u] = evicted_pos;
+    p.pos[r.rows0 + dst] = n;
+    p.acc[r.rows0 + dst] = new_key;
   }
 }
 
@@ -154,10 +183,12 @@ __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4],
 }
 
 // Logits (base 2) of the G query rows against slots 0..c-1 and the new token
-// (index c) into lg[head][j].
+// (index c), tiles [tile0, tile1) of 16 indices, into lg[head][index - 16 tile0],
+// and each warp's maximum per head into wmax.
 template <int D, int G>
 __device__ __forceinline__ void unit_logits(const DecodeParams& p, const uint16_t* Kb, const uint16_t* qn,
-                                            const uint16_t* kn, int c, int ld, float* lg) {
+                                            const uint16_t* kn, int c, int tile0, int tile1, int ld, float* lg,
+                                            float (&wmax)[8][kDecodeWarps]) {
   constexpr int KP = D / 32;  // k-step pairs
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int gid = lane >> 2, tig = lane & 3;
@@ -176,8 +207,9 @@ __device__ __forceinline__ void unit_logits(const DecodeParams& p, const uint16_
   // Slots 0..c-1 from the arena and the new token (index c) from its own k
   // row, 16 per tile; tiles are dealt to the warps in turn.
   const int cnt = c + 1;
-  const int ntiles = (cnt + 15) / 16;
-  for (int t = warp; t < ntiles; t += kDecodeThreads / 32) {
+  lg -= 16 * tile0;
+  float mx0 = -INFINITY, mx1 = -INFINITY;  // this lane's heads 2tig, 2tig + 1
+  for (int t = tile0 + warp; t < tile1; t += kDecodeThreads / 32) {
     const int j0 = t * 16 + gid, j1 = j0 + 8;  // this lane's two slot rows
     uint4 X[KP], Y[KP];
 #pragma unroll
@@ -201,13 +233,24 @@ __device__ __forceinline__ void unit_logits(const DecodeParams& p, const uint16_
     // acc: (slot j0, heads 2tig, 2tig+1) and (slot j1, same heads)
     const int h0 = 2 * tig;
     if (h0 < G) {
-      if (j0 < cnt) lg[h0 * ld + j0] = acc[0] * p.scale_log2;
-      if (j1 < cnt) lg[h0 * ld + j1] = acc[2] * p.scale_log2;
+      if (j0 < cnt) { lg[h0 * ld + j0] = acc[0] * p.scale_log2; mx0 = fmaxf(mx0, acc[0]); }
+      if (j1 < cnt) { lg[h0 * ld + j1] = acc[2] * p.scale_log2; mx0 = fmaxf(mx0, acc[2]); }
     }
     if (h0 + 1 < G) {
-      if (j0 < cnt) lg[(h0 + 1) * ld + j0] = acc[1] * p.scale_log2;
-      if (j1 < cnt) lg[(h0 + 1) * ld + j1] = acc[3] * p.scale_log2;
+      if (j0 < cnt) { lg[(h0 + 1) * ld + j0] = acc[1] * p.scale_log2; mx1 = fmaxf(mx1, acc[1]); }
+      if (j1 < cnt) { lg[(h0 + 1) * ld + j1] = acc[3] * p.scale_log2; mx1 = fmaxf(mx1, acc[3]); }
     }
+  }
+  mx0 *= p.scale_log2;
+  mx1 *= p.scale_log2;
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) {
+    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, o));
+    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, o));
+  }
+  if (gid == 0) {
+    if (2 * tig < G) wmax[2 * tig][warp] = mx0;
+    if (2 * tig + 1 < G) wmax[2 * tig + 1][warp] = mx1;
   }
 }
 
@@ -221,72 +264,117 @@ __device__ __forceinline__ void unit_logits(const DecodeParams& p, const uint16_
 // rows; k-step 2kp + w takes elements 4w .. 4w + 3 of that slice (the low two
 // as fragment columns 2t, 2t+1, the high two as 2t+8, 2t+9), and Q's B
 // fragment is loaded in the same order.
-template <int D, int G>
+//
+// The CTA of rank `rank` of the unit's `p.cluster` CTAs takes a run of the
+// tiles (kSplit; without it the one CTA takes all).  Each CTA softmaxes its
+// run against its own maximum; the (max, sum) pairs of all CTAs give the scale
+// of each, and their best eviction candidates the slot to evict.
+template <int D, int G, bool kSplit>
 __device__ void attend_unit(const DecodeParams& p, const DecLayer& ly, const UnitRef& r, int n, int c,
-                            float* lg, DecShared& sh) {
-  const int ld = ly.cap + 1;  // row stride of lg
+                            float* lg, DecShared<kSplit>& sh) {
+  if (kSplit) cluster_started_arrive();
+  const int C = kSplit ? p.cluster : 1;
+  const uint32_t rank = kSplit ? cluster_rank() : 0;
+  const int cnt = c + 1;                          // indices: slots 0..c-1, then the new token
+  const int ntiles = (cnt + 15) / 16;
+  const int per = kSplit ? (ntiles + C - 1) / C : ntiles;
+  const int tile0 = kSplit ? min(static_cast<int>(rank) * per, ntiles) : 0;
+  const int tile1 = kSplit ? min(tile0 + per, ntiles) : ntiles;
+  const int base = 16 * tile0;                    // first index of this CTA
+  const int m = kSplit ? max(0, min(cnt, 16 * tile1) - base) : cnt;  // and how many it has
+  const int ld = kSplit ? 16 * ((ly.cap + 16) / 16 / C + 1) : ly.cap + 1;  // row stride of lg, >= 16 per
   const uint16_t* Kb = static_cast<const uint16_t*>(p.K) + r.rows0 * D;
-  const uint16_t* kn = static_cast<const uint16_t*>(p.k_new[r.l]) + (static_cast<size_t>(r.s) * p.H_kv + r.h) * D;
-  const uint16_t* qn = p.q_new[r.l] == nullptr
+  const uint16_t* kn = static_cast<const uint16_t*>(ly.k_new) + (static_cast<size_t>(r.s) * p.H_kv + r.h) * D;
+  const uint16_t* qn = ly.q_new == nullptr
                            ? nullptr
-                           : static_cast<const uint16_t*>(p.q_new[r.l]) +
-                                 (static_cast<size_t>(r.s) * p.H_q + r.h * G) * D;
+                           : static_cast<const uint16_t*>(ly.q_new) + (static_cast<size_t>(r.s) * p.H_q + r.h * G) * D;
 
   // attention supplied by the caller's own decode attention: slots 0..c-1, then the new token
-  const float* at = p.attn[r.l] == nullptr
+  // (never with a split unit)
+  const float* at = kSplit || ly.attn == nullptr
                         ? nullptr
-                        : p.attn[r.l] + (static_cast<size_t>(r.s) * p.H_kv + r.h) * static_cast<size_t>(ld);
-  if (at == nullptr) unit_logits<D, G>(p, Kb, qn, kn, c, ld, lg);
-  const int cnt = c + 1;
-  __syncthreads();
-  // per-head softmax statistics (not needed when the attention is supplied)
-  float mg[G], zg[G];
+                        : ly.attn + (static_cast<size_t>(r.s) * p.H_kv + r.h) * static_cast<size_t>(ly.cap + 1);
+  float zg[G];  // 1 / (G z) of every head's softmax (not needed when the attention is supplied)
 #pragma unroll
-  for (int g = 0; g < G; ++g) {
-    mg[g] = 0.f;
-    zg[g] = 1.f;
-  }
+  for (int g = 0; g < G; ++g) zg[g] = 1.f;
   if (at == nullptr) {
+    unit_logits<D, G>(p, Kb, qn, kn, c, tile0, tile1, ld, lg, sh.wmax);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float mg[G], z[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-      mg[g] = -INFINITY;
-      for (int j = threadIdx.x; j < cnt; j += blockDim.x) mg[g] = fmaxf(mg[g], lg[g * ld + j]);
+      mg[g] = over_warps<true>(sh.wmax[g]);
+      z[g] = 0.f;
     }
-    block_reduce_heads<G, true>(mg, sh);
+    for (int j = threadIdx.x; j < m; j += blockDim.x) {  // each thread keeps its own exponentials
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-      zg[g] = 0.f;
-      for (int j = threadIdx.x; j < cnt; j += blockDim.x) {  // each thread keeps its own exponentials
+      for (int g = 0; g < G; ++g) {
         const float e = exp2f(lg[g * ld + j] - mg[g]);
         lg[g * ld + j] = e;
-        zg[g] += e;
+        z[g] += e;
       }
     }
-    block_reduce_heads<G, false>(zg, sh);
 #pragma unroll
-    for (int g = 0; g < G; ++g) zg[g] = 1.0f / (static_cast<float>(G) * zg[g]);
+    for (int g = 0; g < G; ++g) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) z[g] += __shfl_xor_sync(0xffffffffu, z[g], o);
+      if (lane == 0) sh.wsum[g][warp] = z[g];
+    }
+    __syncthreads();
+    if (kSplit) {
+      cluster_started_wait();
+      for (int i = threadIdx.x; i < C * G; i += kDecodeThreads) {  // head g's pair to CTA k
+        const int k = i / G, g = i - k * G;
+        st_cluster(cluster_addr(&sh.cm[rank][g], k), over_warps<true>(sh.wmax[g]));
+        st_cluster(cluster_addr(&sh.cz[rank][g], k), over_warps<false>(sh.wsum[g]));
+      }
+      __syncwarp();
+      cluster_sync();
+#pragma unroll
+      for (int g0 = 0; g0 < G; g0 += 4) {  // lanes: four heads x the pairs of up to eight CTAs
+        const int g = min(g0 + (lane >> 3), G - 1), k = lane & 7;
+        const float mk = k < C ? sh.cm[k][g] : -INFINITY, zk = k < C ? sh.cz[k][g] : 0.f;
+        float M = mk;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+        float Z = zk * exp2f(mk - M);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, o);
+        const float scale = exp2f(sh.cm[rank][g] - M) / (static_cast<float>(G) * Z);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (g0 + q < G) zg[g0 + q] = __shfl_sync(0xffffffffu, scale, 8 * q);
+      }
+    } else {
+#pragma unroll
+      for (int g = 0; g < G; ++g) zg[g] = 1.0f / (static_cast<float>(G) * over_warps<false>(sh.wsum[g]));
+    }
   }
   // group-mean attention -> new keys (each thread overwrites row 0 at its own j only)
-  const float* accr = p.acc + r.rows0;
-  const int32_t* posr = p.pos + r.rows0;
+  const float* accr = p.acc + r.rows0 + base;
+  const int32_t* posr = p.pos + r.rows0 + base;
+  if (at != nullptr) at += base;
   const int limit = n + 1 - ly.r;  // positions >= limit are protected
+  const int mc = c - base;         // the new token's local index
   float ba = INFINITY;
   int bp = -1, bs = -1;
   constexpr int kU = 4;  // slots per thread whose global loads are issued together
-  for (int j0 = threadIdx.x; j0 < cnt; j0 += kU * kDecodeThreads) {
+  for (int j0 = threadIdx.x; j0 < m; j0 += kU * kDecodeThreads) {
     float accv[kU], atv[kU];
     int posv[kU];
 #pragma unroll
     for (int q = 0; q < kU; ++q) {
       const int j = j0 + q * kDecodeThreads;
-      accv[q] = (ly.method == KVEV_H2O && j < c) ? accr[j] : 0.f;
-      posv[q] = j < c ? posr[j] : n;
-      atv[q] = (at != nullptr && j < cnt) ? at[j] : 0.f;
+      const bool slot = j < m && j < mc;
+      accv[q] = (ly.method == KVEV_H2O && slot) ? accr[j] : 0.f;
+      posv[q] = slot ? posr[j] : n;
+      atv[q] = (at != nullptr && j < m) ? at[j] : 0.f;
     }
 #pragma unroll
     for (int q = 0; q < kU; ++q) {
       const int j = j0 + q * kDecodeThreads;
-      if (j >= cnt) break;
+      if (j >= m) break;
       float pj = atv[q];
       if (at == nullptr) {  // group mean of the kept exponentials times 1 / (G z_g)
         pj = 0.f;
@@ -299,43 +387,61 @@ __device__ void attend_unit(const DecodeParams& p, const DecLayer& ly, const Uni
       if (pos >= 0 && pos < limit && (bp < 0 || evict_before(a, pos, ba, bp))) {
         ba = a;
         bp = pos;
-        bs = j;
+        bs = base + j;
       }
     }
   }
   const bool full = c >= ly.b;
-  const int ev = full ? block_evict_choice(ba, bp, bs, sh) : -1;  // c = the new token
-  __syncthreads();
-  const int evicted_pos = ev < 0 ? -1 : (ev < c ? posr[ev] : n);
-  __syncthreads();  // every thread has read posr[ev] before it is overwritten
-  for (int j = threadIdx.x; j < c; j += blockDim.x)
-    if (j != ev) p.acc[r.rows0 + j] = lg[j];
+  float new_key = 0.f;
+  if (full) {
+    block_evict_choice(ba, bp, bs, sh.wcand);  // bs = c: the new token; ends past a barrier: lg is complete
+    if (kSplit) {
+      if (static_cast<int>(threadIdx.x) < C)
+        st_cluster(cluster_addr(&sh.cand[rank], threadIdx.x),
+                   DecCandidate{ba, bp, bs, mc >= 0 && mc < m ? lg[mc] : 0.f});
+      __syncwarp();
+      cluster_sync();
+      const int k = threadIdx.x & 7;
+      bs = -1;
+      bp = -1;
+      if (k < C) {
+        const DecCandidate d = sh.cand[k];
+        ba = d.key;
+        bp = d.pos;
+        bs = d.slot;
+      }
+      warp_evict_choice(ba, bp, bs, 8);
+      new_key = sh.cand[(c / 16) / per].new_key;
+    } else {
+      new_key = lg[c];
+    }
+  } else {
+    bs = -1;
+    __syncthreads();
+    if (mc >= 0 && mc < m) new_key = lg[mc];
+  }
+  for (int j = threadIdx.x; j < m; j += blockDim.x)
+    if (j < mc && base + j != bs) p.acc[r.rows0 + base + j] = lg[j];
+  const bool lead = rank == 0 && threadIdx.x == 0;
   if (!full) {
     if (c >= ly.cap) {  // never for a consistent state: slots of an evicting layer stay <= b
-      if (threadIdx.x == 0) atomicOr(p.status, kStatusDevice);
+      if (lead) atomicOr(p.status, kStatusDevice);
       return;
     }
-    place_new(p, r, D, c, n, lg[c], c + 1, -1);
-  } else if (ev < 0) {  // no evictable slot (protected window covers the cache)
-    if (threadIdx.x == 0) atomicOr(p.status, kStatusDevice);
+    if (mc >= 0 && mc < m) place_new(p, ly, r, D, c, n, new_key);
+    if (lead) {
+      p.count[r.u] = c + 1;
+      p.evicted[r.u] = -1;
+    }
+  } else if (bs < 0) {  // no evictable slot (protected window covers the cache)
+    if (lead) atomicOr(p.status, kStatusDevice);
   } else {
-    place_new(p, r, D, ev < c ? ev : -1, n, lg[c], c, evicted_pos);
+    if (bs < c && bs >= base && bs < base + m) place_new(p, ly, r, D, bs, n, new_key);
+    if (lead) {
+      p.count[r.u] = c;
+      p.evicted[r.u] = bp;  // the new token's own position when it is the one evicted
+    }
   }
-}
-
-constexpr int kDecodeWarps = kDecodeThreads / 32;
-
-// The first layer whose prefix end (att_end or cheap_end) exceeds i: the
-// layer holding the i-th unit of that kind.
-template <bool kAttend>
-__device__ __forceinline__ int find_kind_layer(const DecodeParams& p, int i) {
-  int lo = 0, hi = p.L - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if ((kAttend ? p.layer[mid].att_end : p.layer[mid].cheap_end) > i) hi = mid;
-    else lo = mid + 1;
-  }
-  return lo;
 }
 
 __device__ __forceinline__ UnitRef unit_ref(const DecodeParams& p, int l, int rem) {
@@ -351,18 +457,19 @@ __device__ __forceinline__ UnitRef unit_ref(const DecodeParams& p, int l, int re
 
 // The step of the a-th H2O / TOVA unit (called by the whole block; returns
 // early on an inconsistent state, which it records in the status word).
-template <int D, int G>
-__device__ __forceinline__ void step_attend(const DecodeParams& p, int a, float* lg, DecShared& sh) {
-  const int l = find_kind_layer<true>(p, a);
+template <int D, int G, bool kSplit>
+__device__ __forceinline__ void step_attend(const DecodeParams& p, int a, float* lg, DecShared<kSplit>& sh) {
+  const int per_layer = p.B * p.H_kv;
+  const int l = p.att_layer[a / per_layer];
   const DecLayer& ly = p.layer[l];
-  const UnitRef r = unit_ref(p, l, a - (ly.att_end - p.B * p.H_kv));
+  const UnitRef r = unit_ref(p, l, a % per_layer);
   const int n = p.lens[r.s];
   const int c = p.count[r.u];
-  if (c < 0 || c > ly.cap) {
+  if (c < 0 || c > ly.cap) {  // the same for every CTA of the unit
     if (threadIdx.x == 0) atomicOr(p.status, kStatusDevice);
     return;
   }
-  attend_unit<D, G>(p, ly, r, n, c, lg, sh);
+  attend_unit<D, G, kSplit>(p, ly, r, n, c, lg, sh);
 }
 
 // place_new by one warp: the new token's K/V row (16-byte vectors over the
@@ -377,7 +484,7 @@ __device__ __forceinline__ void place_new_warp(const DecodeParams& p, const Unit
       const bool isv = i >= vec;
       const int e = isv ? i - vec : i;
       uint4* drow = reinterpret_cast<uint4*>(isv ? p.V : p.K) + (r.rows0 + dst) * vec + e;
-      const uint4* srow = reinterpret_cast<const uint4*>(isv ? p.v_new[r.l] : p.k_new[r.l]) + src * vec + e;
+      const uint4* srow = reinterpret_cast<const uint4*>(isv ? p.layer[r.l].v_new : p.layer[r.l].k_new) + src * vec + e;
       *drow = *srow;
     }
   }
@@ -396,9 +503,10 @@ __device__ __forceinline__ void place_new_warp(const DecodeParams& p, const Unit
 // sink + recent slots are held; an append-only unit takes the next slot.
 __device__ void step_cheap_warp(const DecodeParams& p, int i, int D) {
   const int lane = threadIdx.x & 31;
-  const int l = find_kind_layer<false>(p, i);
+  const int per_layer = p.B * p.H_kv;
+  const int l = p.cheap_layer[i / per_layer];
   const DecLayer& ly = p.layer[l];
-  const UnitRef r = unit_ref(p, l, i - (ly.cheap_end - p.B * p.H_kv));
+  const UnitRef r = unit_ref(p, l, i % per_layer);
   const int n = p.lens[r.s];
   const int c = p.count[r.u];
   const bool streaming = ly.method == KVEV_STREAMING;
@@ -411,13 +519,25 @@ __device__ void step_cheap_warp(const DecodeParams& p, int i, int D) {
     place_new_warp(p, r, D, c, n, 0.f, c + 1, -1);
     return;
   }
-  // smallest position >= sink among the slots and the new token (positions are distinct)
+  // smallest position >= sink among the slots and the new token (positions are
+  // distinct); 16 loads in flight per lane, as one warp scans the whole unit
   int bp = 0x7FFFFFFF, bs = -1;
-  for (int j = lane; j <= c; j += 32) {
-    const int pos = j < c ? p.pos[r.rows0 + j] : n;
-    if (pos >= ly.sink && pos < bp) {
-      bp = pos;
-      bs = j;
+  const int32_t* posr = p.pos + r.rows0;
+  if (lane == 0 && n >= ly.sink) {
+    bp = n;
+    bs = c;
+  }
+  constexpr int kU = 16;
+  for (int j0 = lane; j0 < c; j0 += 32 * kU) {
+    int v[kU];
+#pragma unroll
+    for (int q = 0; q < kU; ++q) v[q] = j0 + 32 * q < c ? posr[j0 + 32 * q] : -1;
+#pragma unroll
+    for (int q = 0; q < kU; ++q) {
+      if (v[q] >= ly.sink && v[q] < bp) {
+        bp = v[q];
+        bs = j0 + 32 * q;
+      }
     }
   }
 #pragma unroll
@@ -437,15 +557,19 @@ __device__ void step_cheap_warp(const DecodeParams& p, int i, int D) {
   place_new_warp(p, r, D, bs < c ? bs : -1, n, 0.f, c, bp);
 }
 
-template <int D, int G>
-__global__ void __launch_bounds__(kDecodeThreads) decode_step_kernel(const __grid_constant__ DecodeParams p) {
+template <int D, int G, bool kSplit>
+__global__ void __launch_bounds__(kDecodeThreads, kDecCtasPerSm) decode_step_kernel(const __grid_constant__ DecodeParams p) {
   extern __shared__ float lg[];
-  __shared__ DecShared sh;
-  // CTAs [0, n_att): one H2O / TOVA unit each; then eight cheap units per CTA
-  if (static_cast<int>(blockIdx.x) < p.n_att) {
-    step_attend<D, G>(p, blockIdx.x, lg, sh);
+  __shared__ DecShared<kSplit> sh;
+  // the H2O / TOVA units, and eight cheap units per CTA: after the others, or,
+  // split, before them (every CTA is resident at once, and those end first)
+  const int n_cheap_ctas = kSplit ? static_cast<int>(gridDim.x) - p.n_att * p.cluster : 0;
+  const int n_att_ctas = kSplit ? 0 : p.n_att;
+  const int b = static_cast<int>(blockIdx.x);
+  if (kSplit ? b >= n_cheap_ctas : b < n_att_ctas) {
+    step_attend<D, G, kSplit>(p, kSplit ? (b - n_cheap_ctas) / p.cluster : b, lg, sh);
   } else {
-    const int i = (blockIdx.x - p.n_att) * kDecodeWarps + (threadIdx.x >> 5);
+    const int i = (b - n_att_ctas) * kDecodeWarps + (threadIdx.x >> 5);
     if (i < p.n_cheap) step_cheap_warp(p, i, D);
   }
   // The last CTA of the step to finish advances every sequence by one token:
@@ -527,17 +651,34 @@ __global__ void __launch_bounds__(kDecodeThreads) decode_init_kernel(const __gri
     for (int i = threadIdx.x; i < p.B; i += blockDim.x) p.lens[i] = p.lens_in[i];
 }
 
-template <int D, int G>
-cudaError_t launch_step_dg(const DecodeParams& p, size_t smem, cudaStream_t st) {
+template <int D, int G, bool kSplit>
+cudaError_t launch_step_dgs(const DecodeParams& p, size_t smem, cudaStream_t st) {
   if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(decode_step_kernel<D, G>,
+    const cudaError_t e = cudaFuncSetAttribute(decode_step_kernel<D, G, kSplit>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                static_cast<int>(smem));
     if (e != cudaSuccess) return e;
   }
-  const int grid = p.n_att + (p.n_cheap + kDecodeWarps - 1) / kDecodeWarps;
-  decode_step_kernel<D, G><<<grid, kDecodeThreads, smem, st>>>(p);
-  return cudaGetLastError();
+  const int cheap = (p.n_cheap + kDecodeWarps - 1) / kDecodeWarps;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(p.n_att * p.cluster + (cheap + p.cluster - 1) / p.cluster * p.cluster);  // whole clusters
+  cfg.blockDim = dim3(kDecodeThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  if (kSplit) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = p.cluster;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+  }
+  return cudaLaunchKernelEx(&cfg, decode_step_kernel<D, G, kSplit>, p);
+}
+
+template <int D, int G>
+cudaError_t launch_step_dg(const DecodeParams& p, size_t smem, cudaStream_t st) {
+  return p.cluster > 1 ? launch_step_dgs<D, G, true>(p, smem, st) : launch_step_dgs<D, G, false>(p, smem, st);
 }
 
 template <int D>
@@ -555,6 +696,13 @@ cudaError_t launch_step_d(const DecodeParams& p, size_t smem, cudaStream_t st) {
 
 bool decode_supported(int d, int G) {
   return (d == 64 || d == 128) && (G == 1 || G == 2 || G == 4 || G == 8);
+}
+
+// Dynamic shared memory of a step: `rows` rows of logits over a CTA's share of
+// the unit's cap + 1 indices (cap slots and the new token).
+size_t decode_logit_bytes(int cap, int rows, int cluster) {
+  const size_t ld = cluster > 1 ? 16 * static_cast<size_t>((cap + 16) / 16 / cluster + 1) : static_cast<size_t>(cap) + 1;
+  return sizeof(float) * rows * ld;
 }
 
 cudaError_t launch_decode_init(const DecodeParams& p, cudaStream_t st) {

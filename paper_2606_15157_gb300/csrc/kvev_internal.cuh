@@ -150,7 +150,8 @@ struct SelectParams {
   void* out_V;
 };
 
-// Per-layer description of the decode arena.
+// Per-layer description of the decode arena, with the layer's inputs of a step
+// (one record, so that a unit's parameter reads touch few constant-cache lines).
 struct DecLayer {
   int method;         // decode-phase operator (KVEV_*); FULL = append only
   int b;              // budget: slots kept by an evicting layer
@@ -160,20 +161,25 @@ struct DecLayer {
   int pre_method;     // prefill operator (its packed rows seed the arena)
   int pre_slots;      // prefill slots per unit (b_l)
   int unit_off;       // first unit of the layer
-  int att_end;        // H2O / TOVA units of layers 0..l (one CTA each in the step kernel)
-  int cheap_end;      // StreamingLLM and append-only units of layers 0..l (one warp each)
   long long row_off;  // first arena slot row of the layer
   long long pre_row_off;  // first packed prefill row of the layer
+  const void* k_new;  // [B][H_kv][d] bf16
+  const void* v_new;  // [B][H_kv][d]
+  const void* q_new;  // [B][H_q][d]
+  const float* attn;  // [B][H_kv][cap + 1] caller-supplied attention, or null
 };
+
+constexpr int kMaxDecCluster = 8;      // CTAs an H2O / TOVA unit's step may be split over
+constexpr int kDecCtasPerSm = 4;       // resident CTAs per SM of the step kernel (64 registers)
 
 struct DecodeParams {
   DecLayer layer[kMaxLayers];
-  const void* k_new[kMaxLayers];  // [B][H_kv][d] bf16 per layer
-  const void* v_new[kMaxLayers];  // [B][H_kv][d]
-  const void* q_new[kMaxLayers];  // [B][H_q][d]
-  const float* attn[kMaxLayers];  // [B][H_kv][cap + 1] caller-supplied attention, or null
+  // the layers with H2O / TOVA units and with StreamingLLM or append-only
+  // units (every layer has B * H_kv units of its kind)
+  uint8_t att_layer[kMaxLayers], cheap_layer[kMaxLayers];
   int L, B, H_kv, H_q, G, d, units;
   int n_att, n_cheap; // attending units; StreamingLLM and append-only units
+  int cluster;        // CTAs per attending unit (1, or the cluster size)
   int init_split;     // CTAs per unit of the initialisation
   float scale_log2;   // log2(e) / sqrt(d)
   void* K;            // arena rows [rows][d] bf16
@@ -592,6 +598,7 @@ cudaError_t launch_score(const ScoreParams& p, int d, int grid, size_t smem, cud
 int score_smem_bytes(int d, int q_rows, int q_bufs, int R_pad, int stages);
 bool decode_supported(int d, int G);
 cudaError_t launch_decode_init(const DecodeParams& p, cudaStream_t s);
+size_t decode_logit_bytes(int cap, int rows, int cluster);
 cudaError_t launch_decode_step(const DecodeParams& p, size_t smem, cudaStream_t s);
 int score_kernel_regs(int d, int R_pad);
 cudaError_t score_set_smem(int d, int R_pad, size_t smem);

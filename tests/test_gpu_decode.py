@@ -194,6 +194,46 @@ def test_decode_lockstep_mixed_rules(env, d):
                 assert set(range(first, n_now)) <= set(x["pos"].tolist())
 
 
+@pytest.mark.parametrize("H_q,H_kv,d,budgets", [
+    (4, 2, 64, (127, 96)),      # one CTA per unit
+    (4, 2, 128, (257, 128)),    # clusters of two: 17 tiles of 16 indices, and 9
+    (2, 2, 64, (527, 640)),     # four
+    (8, 1, 128, (1025, 33)),    # eight: three tiles for most CTAs, and none for some
+    (8, 2, 128, (1039, 2000)),  # eight, with a layer that is not full at first
+])
+def test_decode_split_units(env, H_q, H_kv, d, budgets):
+    # A unit's step is split over 1, 2, 4 or 8 CTAs by the largest capacity; units
+    # whose indices (slots and the new token) end at, one past and one short of
+    # a tile, whose CTAs have no tile, and that are not full yet.
+    torch, kvev, orc = env
+    n = 1900
+    wl = gen.Workload(name="split", L=4, H_q=H_q, H_kv=H_kv, d=d, B=2, lens=np.array([n, n - 411], np.int32),
+                      S_cap=n, W=8, pool_kernel=5, pool_type=gen.POOL_AVG,
+                      route=np.array([gen.H2O, gen.SNAPKV, gen.H2O, gen.STREAMING], np.int32),
+                      budget=np.array([budgets[0], budgets[1], budgets[1], 40], np.int32), sink=4, seed=9,
+                      sink_tokens=4, sink_scale=4.0,
+                      route_decode=np.array([gen.H2O, gen.TOVA, gen.H2O, gen.STREAMING], np.int32), decode_steps=5)
+    plan, bufs, arena = prefill_and_arena(torch, kvev, wl, 0)
+    g = Arena(torch, arena, wl)
+    units = list(range(len(g.units)))
+    states = [oracle_state(orc, wl, wl.route_decode, g, i) for i in units]
+    for step in range(wl.decode_steps):
+        toks, k, v, q = step_tokens(wl, step, range(wl.L))
+        arena.step(k, v, q)
+        kn, vn, qn = host_tokens(torch, toks, wl, units, g)
+        orc.decode_step(states, kn, vn, qn, wl.d, wl.G)
+        g.refresh(torch)
+        assert np.array_equal(g.lens, wl.lens + step + 1)
+        for i in units:
+            l, s, h = g.units[i][:3]
+            x = g.unit(i)
+            if compare_unit(states[i], x, f"step {step} layer {l} seq {s} head {h}") == "tie":
+                resync(states[i], x)
+            ev = int(g.evicted[g.units[i][3]])
+            assert ev == -1 or ev not in set(x["pos"].tolist())
+    assert plan.status() == kvev.OK
+
+
 def _bf16_to_f64(u16):
     return (np.asarray(u16, np.uint32) << 16).view(np.float32).astype(np.float64)
 
