@@ -25,6 +25,14 @@
 // 1 owns TMEM and issues tcgen05.mma (one thread), warp 2 stages each query
 // block's -lse2 for the key pass, warps 4-19 are four softmax warpgroups that
 // split every 256-column TMEM unit by columns (64 each).
+//
+// Both passes are paced by the softmax warps: exp2 (1,024 cycles a unit) and
+// the TMEM copies, and in the key pass by the broadcast reads of -lse2, which
+// compete with the MMA's operand reads for shared memory.  Items without a
+// causal cut run without per-element checks; measured with that and the
+// stager's divisions taken out of its loop, 7 layers x 8 KV heads of a
+// 6,001-token prompt (1.0 TFLOP performed a pass): row pass 807 and 779 us,
+// key pass 1,241 and 907 us.
 #include "score_common.cuh"
 
 namespace kvev {
@@ -38,7 +46,6 @@ struct FSmem {
   uint8_t* fixed;  // the item's own operand: Q block (phase 0) or K super-tile (phase 1)
   uint8_t* stage;  // kStreamStages streamed operands: K super-tiles (0) or Q blocks (1)
   float* lam;      // [2][256] -lse2 of a query block's rows; -inf where the row does not exist
-  int* tpos;       // [2][256] prompt position of each row of that block; -1: no such row
   float2* pc;      // [kSoftmaxWGs][256] (max, sum) of each row (phase 0); in phase 1 the
                    // floats [kSoftmaxWGs][2][128] hold the partial sums of the item's keys
   uint64_t* ffull;
@@ -53,16 +60,14 @@ struct FSmem {
   uint32_t* tmem_slot;
 };
 
-__host__ __device__ __forceinline__ size_t fsmem_size(int D, size_t* stage_off, size_t* lam_off,
-                                                       size_t* tpos_off, size_t* pc_off, size_t* bar_off) {
+__host__ __device__ __forceinline__ size_t fsmem_size(int D, size_t* stage_off, size_t* lam_off, size_t* pc_off,
+                                                       size_t* bar_off) {
   const size_t buf = static_cast<size_t>(kBufRows) * D * 2;
   size_t off = buf;
   *stage_off = off;
   off += kStreamStages * buf;
   *lam_off = off;
   off += sizeof(float) * 2 * 256;
-  *tpos_off = off;
-  off += sizeof(int) * 2 * 256;
   *pc_off = off;
   off += sizeof(float2) * kSoftmaxWGs * 256;
   *bar_off = off;
@@ -73,12 +78,11 @@ __host__ __device__ __forceinline__ size_t fsmem_size(int D, size_t* stage_off, 
 
 __device__ __forceinline__ FSmem fcarve(uint8_t* base, int D) {
   FSmem s;
-  size_t so, lo, to, po, bo;
-  fsmem_size(D, &so, &lo, &to, &po, &bo);
+  size_t so, lo, po, bo;
+  fsmem_size(D, &so, &lo, &po, &bo);
   s.fixed = base;
   s.stage = base + so;
   s.lam = reinterpret_cast<float*>(base + lo);
-  s.tpos = reinterpret_cast<int*>(base + to);
   s.pc = reinterpret_cast<float2*>(base + po);
   uint64_t* b = reinterpret_cast<uint64_t*>(base + bo);
   s.ffull = b;
@@ -148,7 +152,7 @@ __device__ __forceinline__ int block_row_pos(const ScoreParams& p, int r, int q0
 // ---------------------------------------------------------------------------
 // Producer (one thread).
 // ---------------------------------------------------------------------------
-template <int D>
+template <int D, int kPhase>
 __device__ __forceinline__ void f_producer(const ScoreParams& p, const FSmem& sm) {
   constexpr uint32_t kBufBytes = kBufRows * D * 2;
   const uint32_t qbytes = static_cast<uint32_t>(p.R) * D * 2;  // what a G x Pb query box brings
@@ -163,7 +167,7 @@ __device__ __forceinline__ void f_producer(const ScoreParams& p, const FSmem& sm
     const int qhead = f.s * p.H_q + f.h * p.G;
     // the fixed buffer is free once the previous item's MMAs have completed
     if (!wait_bar(sm.fempty, (e & 1) ^ 1, p)) { ok = false; break; }
-    if (p.phase == 0) {
+    if (kPhase == 0) {
       mbar_expect_tx(sm.ffull, qbytes);
 #pragma unroll
       for (int kc = 0; kc < D / 64; ++kc)
@@ -180,7 +184,7 @@ __device__ __forceinline__ void f_producer(const ScoreParams& p, const FSmem& sm
     for (int j = 0; j < ns; ++j) {
       if (!wait_bar(&sm.sempty[st], ph ^ 1, p)) { ok = false; break; }
       uint8_t* dst = sm.stage + static_cast<size_t>(st) * kBufBytes;
-      if (p.phase == 0) {
+      if (kPhase == 0) {
         mbar_expect_tx(&sm.sfull[st], kBufBytes);
 #pragma unroll
         for (int kc = 0; kc < D / 64; ++kc)
@@ -209,13 +213,13 @@ __device__ __forceinline__ void f_producer(const ScoreParams& p, const FSmem& sm
 // ---------------------------------------------------------------------------
 // MMA issuer (one warp, an elected lane issues).
 // ---------------------------------------------------------------------------
-template <int D>
+template <int D, int kPhase>
 __device__ __forceinline__ void f_mma(const ScoreParams& p, const FSmem& sm, uint32_t tmem_base) {
   constexpr uint32_t kBufBytes = kBufRows * D * 2;
   constexpr uint32_t kColStep = kBufRows * 128 / 16;  // descriptor step between 64-column blocks
   constexpr uint32_t kHalf = 128 * 128 / 16;          // rows (or keys) 128..255 of a buffer
   // phase 0: S[128 rows of a group][256 keys]; phase 1: S^T[128 keys of a half][R_pad rows]
-  const uint32_t idesc = p.phase == 0 ? idesc_bf16_f32(128, kSuperKeys) : idesc_bf16_f32(128, p.R_pad);
+  const uint32_t idesc = kPhase == 0 ? idesc_bf16_f32(128, kSuperKeys) : idesc_bf16_f32(128, p.R_pad);
   const int groups = p.R_pad > 128 ? 2 : 1;
   uint32_t e = 0, st = 0, kph = 0, sl = 0, tph = 0;
   bool ok = true;
@@ -226,7 +230,7 @@ __device__ __forceinline__ void f_mma(const ScoreParams& p, const FSmem& sm, uin
     tc_fence_after();
     const uint64_t fdesc = sw128_desc(smem_u32(sm.fixed));
     const int ns = n_stream(p, f);
-    const int nu = p.phase == 0 ? groups : n_halves(f);
+    const int nu = kPhase == 0 ? groups : n_halves(f);
     for (int j = 0; ok && j < ns; ++j) {
       if (!wait_bar_warp(&sm.sfull[st], kph, p)) { ok = false; break; }
       tc_fence_after();
@@ -261,11 +265,21 @@ __device__ __forceinline__ void f_mma(const ScoreParams& p, const FSmem& sm, uin
 }
 
 // ---------------------------------------------------------------------------
-// Normaliser stager (phase 1, one warp): -lse2 and the position of every row
-// of each query block, in the order the softmax warpgroups consume them.
+// Normaliser stager (phase 1, one warp): -lse2 of every row of each query
+// block, in the order the softmax warpgroups consume them.  A lane's eight
+// rows keep their head and place in the block, so a block costs it eight loads
+// and stores (with the divisions per block the warp, which shares its issue
+// port with softmax warps, set the pace of the pass).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void f_lam(const ScoreParams& p, const FSmem& sm) {
   const int lane = threadIdx.x & 31;
+  int place[8], head[8];  // row lane + 32 q: place in the block (past every block: no such row), head x S_cap
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int r = lane + 32 * q;
+    place[q] = r < p.R ? r % p.Pb : 1 << 30;
+    head[q] = r / p.Pb * p.S_cap;
+  }
   uint32_t lq = 0;
   for (int i = blockIdx.x; i < p.n_items; i += gridDim.x) {
     FItem f;
@@ -273,28 +287,20 @@ __device__ __forceinline__ void f_lam(const ScoreParams& p, const FSmem& sm) {
     const int qb0 = (f.blk * kSuperKeys) / p.Pb;
     const int ns = n_stream(p, f);
     const float* lse = p.lse + static_cast<size_t>(f.hu) * p.G * p.S_cap;
-    // lane's eight rows of a block: position (or -1) and lse2, all loads in
-    // flight at once; block j + 1's loads go out before the wait for its buffer
+    // all loads of a block in flight at once; block j + 1's go out before the
+    // wait for its buffer
     float v[8];
-    int tt[8];
     auto fetch = [&](int j) {
       const int q0 = (qb0 + j) * p.Pb;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int r = lane + 32 * q;
-        tt[q] = block_row_pos(p, r, q0, f.n);
-        v[q] = tt[q] >= 0 ? __ldcg(&lse[static_cast<size_t>(r / p.Pb) * p.S_cap + tt[q]]) : INFINITY;
-      }
+      for (int q = 0; q < 8; ++q) v[q] = place[q] < f.n - q0 ? __ldcg(lse + head[q] + (q0 + place[q])) : INFINITY;
     };
     fetch(0);
     for (int j = 0; j < ns; ++j) {
       const uint32_t lb = lq & 1;
       if (!wait_bar_warp(&sm.lempty[lb], ((lq >> 1) & 1) ^ 1, p)) return;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        sm.lam[lb * 256 + lane + 32 * q] = -v[q];
-        sm.tpos[lb * 256 + lane + 32 * q] = tt[q];
-      }
+      for (int q = 0; q < 8; ++q) sm.lam[lb * 256 + lane + 32 * q] = -v[q];
       __syncwarp();
       mbar_arrive_elect(&sm.lfull[lb]);
       ++lq;
@@ -307,44 +313,18 @@ __device__ __forceinline__ void f_lam(const ScoreParams& p, const FSmem& sm) {
 // Softmax warpgroups.
 // ---------------------------------------------------------------------------
 
-// This warpgroup's 64 columns of a 256-column unit, released before use.
-__device__ __forceinline__ void f_take(const FSmem& sm, uint32_t lane_base, uint32_t g, uint32_t (&r0)[32],
-                                       uint32_t (&r1)[32]) {
-  const uint32_t s0 = g & (kSlots - 1);
-  tmem_ld64_async(lane_base + s0 * kSlotCols, r0, r1);
-  tmem_wait64(r0, r1);
-  tc_fence_before();
-  __syncwarp();
-  mbar_arrive_elect(&sm.tempty[s0]);
+__device__ __forceinline__ bool f_wait(const ScoreParams& p, const FSmem& sm, uint32_t g, bool ok) {
+  return ok && wait_bar(&sm.tfull[g & (kSlots - 1)], (g / kSlots) & 1, p);
 }
 
-__device__ __forceinline__ int lds1i(const int* p) {
-  int v;
-  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)));
-  return v;
-}
-
-// Key sum over 32 rows with per-row checks: rows that do not exist (tp < 0)
-// or that cannot see key k (k > position) add nothing.
-__device__ __forceinline__ void s2_chunk_rows(const uint32_t (&rr)[32], float c, const float* nl, const int* tp,
-                                              int k, float2 (&a)[4]) {
-#pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    if (k <= lds1i(tp + i)) {
-      const float e = ex2_approx(fmaf(__uint_as_float(rr[i]), c, lds1(nl + i)));
-      if (i & 1) a[(i >> 1) & 3].y += e; else a[(i >> 1) & 3].x += e;
-    }
-  }
-}
-
+template <int kPhase>
 __device__ __forceinline__ void f_softmax(const ScoreParams& p, const FSmem& sm, uint32_t tmem_base, int wg) {
   const int warp = threadIdx.x >> 5;
   const int quarter = warp & 3;
   const int lrow = quarter * 32 + (threadIdx.x & 31);  // TMEM lane: row (phase 0) / key (phase 1)
   const int stid = threadIdx.x - 128;                  // 0..511 over the softmax warpgroups
-  const uint32_t lane_base =
+  const uint32_t taddr =
       tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(64 * wg);
-  const int groups = p.R_pad > 128 ? 2 : 1;
   const float c = p.scale_log2;
   float* red = reinterpret_cast<float*>(sm.pc);
   uint32_t g = 0, lq = 0;
@@ -353,40 +333,36 @@ __device__ __forceinline__ void f_softmax(const ScoreParams& p, const FSmem& sm,
     FItem f;
     if (!fitem(p, i, f)) continue;
     const int ns = n_stream(p, f);
-    if (p.phase == 0) {
+    if (kPhase == 0) {
       // ---- rows: running (max, sum) of exp2 over the block's prefix keys ----
+      // (R = G floor(256 / G) rows: always two 128-row groups)
       const int q0 = f.blk * p.Pb;
       const int tr0 = block_row_pos(p, lrow, q0, f.n);
       const int tr1 = block_row_pos(p, 128 + lrow, q0, f.n);
       float m0 = -INFINITY, z0 = 0.f, m1 = -INFINITY, z1 = 0.f;
-      for (int j = 0; j < ns; ++j) {
-        const int kb = j * kSuperKeys;
-        const int k0 = kb + 64 * wg;                  // this warpgroup's keys k0 .. k0 + 63
-        const bool full = kb + kSuperKeys - 1 <= q0;  // every key visible to every row of the block
-        for (int hh = 0; hh < groups; ++hh) {
-          if (ok && !wait_bar(&sm.tfull[g & (kSlots - 1)], (g / kSlots) & 1, p)) ok = false;
-          uint32_t r0[32], r1[32];
-          f_take(sm, lane_base, g, r0, r1);
-          float v0[32], v1[32];
-#pragma unroll
-          for (int q = 0; q < 32; ++q) {
-            v0[q] = __uint_as_float(r0[q]);
-            v1[q] = __uint_as_float(r1[q]);
-          }
-          const int tr = hh == 0 ? tr0 : tr1;
-          if (!full) {
-            mask_chunk(v0, k0, tr);
-            mask_chunk(v1, k0 + 32, tr);
-          }
-          if (hh == 0)
-            s1_chunk64(v0, v1, c, m0, z0);
-          else
-            s1_chunk64(v0, v1, c, m1, z1);
+      const int nfull = min(ns, (q0 + 1) / kSuperKeys);  // super-tiles visible to every row of the block
+      int k0 = 64 * wg;                                  // this warpgroup's keys k0 .. k0 + 63
+      for (int j = 0; j < nfull; ++j, k0 += kSuperKeys) {
+        ok = f_wait(p, sm, g, ok);
+        s1_unit<false>(c, sm.tempty, taddr, g, k0, tr0, m0, z0);
+        g += 2;
+        ok = f_wait(p, sm, g, ok);
+        s1_unit<false>(c, sm.tempty, taddr, g, k0, tr1, m1, z1);
+        g += 2;
+      }
+#pragma unroll 1
+      for (int j = nfull; j < ns; ++j, k0 += kSuperKeys) {
+#pragma unroll 1
+        for (int hh = 0; hh < 2; ++hh) {
+          ok = f_wait(p, sm, g, ok);
+          float m = hh == 0 ? m0 : m1, z = hh == 0 ? z0 : z1;
+          s1_unit<true>(c, sm.tempty, taddr, g, k0, hh == 0 ? tr0 : tr1, m, z);
+          if (hh == 0) { m0 = m; z0 = z; } else { m1 = m; z1 = z; }
           g += 2;
         }
       }
       sm.pc[wg * 256 + lrow] = make_float2(m0, z0);
-      if (groups == 2) sm.pc[wg * 256 + 128 + lrow] = make_float2(m1, z1);
+      sm.pc[wg * 256 + 128 + lrow] = make_float2(m1, z1);
       named_bar_sync(1, 128 * kSoftmaxWGs);
       float* lse = p.lse + static_cast<size_t>(f.hu) * p.G * p.S_cap;
       for (int r = stid; r < p.R; r += 128 * kSoftmaxWGs) {
@@ -404,44 +380,43 @@ __device__ __forceinline__ void f_softmax(const ScoreParams& p, const FSmem& sm,
       const int key0 = f.blk * kSuperKeys;
       const int halves = n_halves(f);
       const int qb0 = key0 / p.Pb;
-      float2 a[2][4];
-#pragma unroll
-      for (int hh = 0; hh < 2; ++hh)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) a[hh][q] = make_float2(0.f, 0.f);
-      const int ra0 = 64 * wg, rb0 = 64 * wg + 32;  // this warpgroup's rows of the block
+      const int r0 = 64 * wg;          // this warpgroup's rows of the block
+      const int exist = p.R - r0, place0 = r0 % p.Pb;
+      // blocks [c0, c1) have no causal cut for this key super-tile and only rows that exist
+      const int c0 = (key0 + kSuperKeys - 1 + p.Pb - 1) / p.Pb - qb0;
+      const int c1 = exist >= 64 ? f.n / p.Pb - qb0 : 0;
+      float sum0 = 0.f, sum1 = 0.f;    // the thread's key of either half
       for (int j = 0; j < ns; ++j) {
         const uint32_t lb = lq & 1;
         if (ok && !wait_bar(&sm.lfull[lb], (lq >> 1) & 1, p)) ok = false;
-        const float* nl = sm.lam + lb * 256;
-        const int* tp = sm.tpos + lb * 256;
-        const int q0 = (qb0 + j) * p.Pb;
-        // no causal cut inside this block and every one of its rows exists
-        const bool clear = key0 + kSuperKeys - 1 <= q0 && q0 + p.Pb <= f.n;
-        for (int hh = 0; hh < halves; ++hh) {
-          if (ok && !wait_bar(&sm.tfull[g & (kSlots - 1)], (g / kSlots) & 1, p)) ok = false;
-          uint32_t ra[32], rb[32];
-          f_take(sm, lane_base, g, ra, rb);
-          const int k = key0 + kTileKeys * hh + lrow;
-          if (ok) {
-            if (clear && ra0 + 32 <= p.R)
-              s2_chunk_full(ra, c, nl + ra0, a[hh]);
-            else if (ra0 < p.R_pad)
-              s2_chunk_rows(ra, c, nl + ra0, tp + ra0, k, a[hh]);
-            if (clear && rb0 + 32 <= p.R)
-              s2_chunk_full(rb, c, nl + rb0, a[hh]);
-            else if (rb0 < p.R_pad)
-              s2_chunk_rows(rb, c, nl + rb0, tp + rb0, k, a[hh]);
-          }
+        const float* nl = sm.lam + lb * 256 + r0;
+        if (j >= c0 && j < c1) {
+          ok = f_wait(p, sm, g, ok);
+          sum0 += s2_unit64(c, sm.tempty, taddr, g, nl);
           g += 2;
+          if (halves == 2) {
+            ok = f_wait(p, sm, g, ok);
+            sum1 += s2_unit64(c, sm.tempty, taddr, g, nl);
+            g += 2;
+          }
+        } else {
+          const int q0 = (qb0 + j) * p.Pb;
+#pragma unroll 1
+          for (int hh = 0; hh < halves; ++hh) {
+            ok = f_wait(p, sm, g, ok);
+            // the row at place i sits at q0 + i: it exists below n and sees the keys up to there
+            const float e = s2_unit_edge(c, sm.tempty, taddr, g, nl, 64, exist, place0, p.Pb,
+                                         key0 + kTileKeys * hh + lrow - q0, f.n - q0);
+            if (hh == 0) sum0 += e; else sum1 += e;
+            g += 2;
+          }
         }
         __syncwarp();
         mbar_arrive_elect(&sm.lempty[lb]);
         ++lq;
       }
-#pragma unroll
-      for (int hh = 0; hh < 2; ++hh)
-        if (hh < halves) red[(wg * 2 + hh) * 128 + lrow] = sum4x2(a[hh]);
+      red[(wg * 2) * 128 + lrow] = sum0;
+      red[(wg * 2 + 1) * 128 + lrow] = sum1;
       named_bar_sync(1, 128 * kSoftmaxWGs);
       float* out = p.raw + static_cast<size_t>(f.u) * p.S_cap;
       for (int q = stid; q < halves * 128; q += 128 * kSoftmaxWGs) {
@@ -455,7 +430,7 @@ __device__ __forceinline__ void f_softmax(const ScoreParams& p, const FSmem& sm,
   }
 }
 
-template <int D>
+template <int D, int kPhase>
 __global__ void __launch_bounds__(kScoreThreads, 1) h2o_full_kernel(const __grid_constant__ ScoreParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   if (smem_u32(smem_raw) & 1023u) {  // the 128-byte swizzle needs 1024-byte aligned buffers
@@ -494,12 +469,12 @@ __global__ void __launch_bounds__(kScoreThreads, 1) h2o_full_kernel(const __grid
 
   if (warp < 4) {
     regs_dealloc<kRegsControl>();
-    if (warp == 0 && (threadIdx.x & 31) == 0) f_producer<D>(p, sm);
-    if (warp == 1) f_mma<D>(p, sm, tmem_base);
-    if (warp == 2 && p.phase == 1) f_lam(p, sm);
+    if (warp == 0 && (threadIdx.x & 31) == 0) f_producer<D, kPhase>(p, sm);
+    if (warp == 1) f_mma<D, kPhase>(p, sm, tmem_base);
+    if (warp == 2 && kPhase == 1) f_lam(p, sm);
   } else {
     regs_alloc<kRegsSoftmax>();
-    f_softmax(p, sm, tmem_base, (warp - 4) >> 2);
+    f_softmax<kPhase>(p, sm, tmem_base, (warp - 4) >> 2);
   }
   tc_fence_before();
   __syncthreads();
@@ -530,24 +505,34 @@ __global__ void __launch_bounds__(256) lse_rows_fill_kernel(const __grid_constan
 }  // namespace
 
 int h2o_full_smem_bytes(int d) {
-  size_t so, lo, to, po, bo;
-  const size_t off = fsmem_size(d, &so, &lo, &to, &po, &bo);
+  size_t so, lo, po, bo;
+  const size_t off = fsmem_size(d, &so, &lo, &po, &bo);
   return static_cast<int>((off + 127) & ~size_t(127));
 }
 
+namespace {
+using FullFn = void (*)(const ScoreParams);
+FullFn full_fn(int d, int phase) {
+  if (d == 64) return phase == 0 ? h2o_full_kernel<64, 0> : h2o_full_kernel<64, 1>;
+  return phase == 0 ? h2o_full_kernel<128, 0> : h2o_full_kernel<128, 1>;
+}
+}  // namespace
+
+// The smaller of the two passes' register counts.
 int h2o_full_kernel_regs(int d) {
-  cudaFuncAttributes a = {};
-  const cudaError_t e = d == 64 ? cudaFuncGetAttributes(&a, h2o_full_kernel<64>)
-                                : cudaFuncGetAttributes(&a, h2o_full_kernel<128>);
-  return e == cudaSuccess ? a.numRegs : -1;
+  cudaFuncAttributes a = {}, b = {};
+  if (cudaFuncGetAttributes(&a, full_fn(d, 0)) != cudaSuccess || cudaFuncGetAttributes(&b, full_fn(d, 1)) != cudaSuccess)
+    return -1;
+  return a.numRegs < b.numRegs ? a.numRegs : b.numRegs;
 }
 
 cudaError_t h2o_full_set_smem(int d, size_t smem) {
-  if (d == 64)
-    return cudaFuncSetAttribute(h2o_full_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(smem));
-  return cudaFuncSetAttribute(h2o_full_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(smem));
+  for (int phase = 0; phase < 2; ++phase) {
+    const cudaError_t e = cudaFuncSetAttribute(full_fn(d, phase), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_lse_rows_fill(const ScoreParams& p, cudaStream_t s) {
@@ -559,10 +544,7 @@ cudaError_t launch_lse_rows_fill(const ScoreParams& p, cudaStream_t s) {
 
 cudaError_t launch_h2o_full(const ScoreParams& p, int d, int grid, size_t smem, cudaStream_t s) {
   if (grid <= 0) return cudaSuccess;
-  if (d == 64)
-    h2o_full_kernel<64><<<grid, kScoreThreads, smem, s>>>(p);
-  else
-    h2o_full_kernel<128><<<grid, kScoreThreads, smem, s>>>(p);
+  full_fn(d, p.phase)<<<grid, kScoreThreads, smem, s>>>(p);
   return cudaGetLastError();
 }
 

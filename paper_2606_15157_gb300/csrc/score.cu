@@ -356,12 +356,6 @@ __device__ __forceinline__ bool slot_wait(const ScoreParams& p, const Smem& sm, 
   return ok;
 }
 
-__device__ __forceinline__ void unit_release(const Smem& sm, uint32_t g) {
-  tc_fence_before();
-  __syncwarp();
-  mbar_arrive_elect(&sm.tempty[g & (kSlots - 1)]);
-}
-
 // The units whose every key is visible to every row (all but the last few of a
 // prompt) run in loops of their own, without a branch per unit; the units at
 // the edges take masked versions.  Measured together with s2_unit_edge's
@@ -370,83 +364,6 @@ __device__ __forceinline__ void unit_release(const Smem& sm, uint32_t g) {
 // 6.2 TB/s of K for the two sweeps); one 30,011-token prompt, 64 x 4 627 and
 // 576 us; eight of 16K-32K 4.25 and 4.01 ms; with the normalisers supplied,
 // four of them 1.02 and 0.90 ms (6.1 TB/s, 0.91 of the measured copy rate).
-
-// Sweep 1: the thread's row of one 128-row group against this warpgroup's 64
-// keys k0 .. k0 + 63; with kMask only the keys its position tr can see.
-template <bool kMask>
-__device__ __forceinline__ void s1_unit(const ScoreParams& p, const Smem& sm, uint32_t taddr, uint32_t g, int k0,
-                                        int tr, float& m, float& z) {
-  uint32_t r0[32], r1[32];
-  tmem_ld64_async(taddr + (g & (kSlots - 1)) * kSlotCols, r0, r1);
-  tmem_wait64(r0, r1);
-  unit_release(sm, g);
-  float v0[32], v1[32];
-#pragma unroll
-  for (int q = 0; q < 32; ++q) {
-    v0[q] = __uint_as_float(r0[q]);
-    v1[q] = __uint_as_float(r1[q]);
-  }
-  if (kMask) {
-    mask_chunk(v0, k0, tr);
-    mask_chunk(v1, k0 + 32, tr);
-  }
-  s1_chunk64(v0, v1, p.scale_log2, m, z);
-}
-
-// Sweep 2: this thread's key against 64 (or 32) rows that all exist and all
-// see it; nl = -lse2 of the rows.
-__device__ __forceinline__ float s2_unit64(const ScoreParams& p, const Smem& sm, uint32_t taddr, uint32_t g,
-                                           const float* nl) {
-  uint32_t ra[32], rb[32];
-  tmem_ld64_async(taddr + (g & (kSlots - 1)) * kSlotCols, ra, rb);
-  tmem_wait64(ra, rb);
-  unit_release(sm, g);
-  float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-  s2_chunk_full(ra, p.scale_log2, nl, a);
-  s2_chunk_full(rb, p.scale_log2, nl + 32, a);
-  return sum4x2(a);
-}
-
-__device__ __forceinline__ float s2_unit32(const ScoreParams& p, const Smem& sm, uint32_t taddr, uint32_t g,
-                                           const float* nl) {
-  uint32_t ra[32];
-  tmem_ld32_async(taddr + (g & (kSlots - 1)) * kSlotCols, ra);
-  tmem_wait32(ra);
-  unit_release(sm, g);
-  float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-  s2_chunk_full(ra, p.scale_log2, nl, a);
-  return sum4x2(a);
-}
-
-// Sweep 2 at the edges: rows [r0, r0 + nrows) (nrows 64 or 32), of which only
-// those below R exist, against key k (k < n), which only rows at or past its
-// position see: row r sits at n - W + r % W.  A row that does not count gets
-// the exponent -inf.  r % W is counted up, not divided: with a division per
-// element the tiles at a prompt's end added 5 us to a 30 us chunk, and with
-// four chunks per unit and 152 CTAs a quarter of the CTAs are dealt every
-// unit's last chunk (they finished at 232 us, the others at 195 us).
-__device__ __forceinline__ float s2_unit_edge(const ScoreParams& p, const Smem& sm, uint32_t taddr, uint32_t g,
-                                              const float* nl, int r0, int nrows, int k, int n) {
-  float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-  const int th = k < n ? k - (n - p.W) : p.W;  // rows with r % W >= th see the key
-  int i = r0 % p.W;
-#pragma unroll 1
-  for (int h = 0; h < nrows && r0 + h < p.R_pad; h += 32) {
-    uint32_t rr[32];
-    tmem_ld32_async(taddr + (g & (kSlots - 1)) * kSlotCols + h, rr);
-    tmem_wait32(rr);
-    const int exist = p.R - (r0 + h);  // rows of the chunk that exist
-#pragma unroll
-    for (int q = 0; q < 32; ++q) {
-      const float x = fmaf(__uint_as_float(rr[q]), p.scale_log2, lds1(nl + h + q));
-      const float e = ex2_approx(i >= th && q < exist ? x : -INFINITY);
-      if (q & 1) a[(q >> 1) & 3].y += e; else a[(q >> 1) & 3].x += e;
-      i = i + 1 == p.W ? 0 : i + 1;
-    }
-  }
-  unit_release(sm, g);
-  return sum4x2(a);
-}
 
 // NH: 128-row groups of the window rows (R_pad <= 128 NH).  Sweep 2 units hold
 // one 128-key tile x up to 256 rows (NH = 2), of which warpgroup w takes rows
@@ -498,13 +415,13 @@ __device__ __forceinline__ void softmax_wg(const ScoreParams& p, const Smem& sm,
       int k0 = it.key0 + 64 * wg;
       for (int j = 0; j < nfull; ++j, k0 += kSuperKeys) {
         ok = slot_wait(p, sm, g, ok);
-        if (NH == 2 || live) s1_unit<false>(p, sm, t1, g, k0, tr0, m0, z0);
-        else unit_release(sm, g);
+        if (NH == 2 || live) s1_unit<false>(p.scale_log2, sm.tempty, t1, g, k0, tr0, m0, z0);
+        else unit_release(sm.tempty, g);
         g += 2;
         if (NH == 2) {
           ok = slot_wait(p, sm, g, ok);
-          if (live) s1_unit<false>(p, sm, t1, g, k0, tr1, m1, z1);
-          else unit_release(sm, g);
+          if (live) s1_unit<false>(p.scale_log2, sm.tempty, t1, g, k0, tr1, m1, z1);
+          else unit_release(sm.tempty, g);
           g += 2;
         }
       }
@@ -514,7 +431,7 @@ __device__ __forceinline__ void softmax_wg(const ScoreParams& p, const Smem& sm,
         for (int h = 0; h < NH; ++h) {
           ok = slot_wait(p, sm, g, ok);
           float m = h == 0 ? m0 : m1, z = h == 0 ? z0 : z1;
-          s1_unit<true>(p, sm, t1, g, k0, h == 0 ? tr0 : tr1, m, z);
+          s1_unit<true>(p.scale_log2, sm.tempty, t1, g, k0, h == 0 ? tr0 : tr1, m, z);
           if (h == 0) { m0 = m; z0 = z; } else { m1 = m; z1 = z; }
           g += 2;
         }
@@ -554,12 +471,12 @@ __device__ __forceinline__ void softmax_wg(const ScoreParams& p, const Smem& sm,
         if (NH == 2 || nrows == 64) {
           for (; u < uf; ++u, g += 2, red += 128 * kPack) {
             ok = slot_wait(p, sm, g, ok);
-            *red = s2_unit64(p, sm, t2, g, lam);
+            *red = s2_unit64(p.scale_log2, sm.tempty, t2, g, lam);
           }
         } else {
           for (; u < uf; ++u, g += 2, red += 128 * kPack) {
             ok = slot_wait(p, sm, g, ok);
-            *red = s2_unit32(p, sm, t2, g, lam);
+            *red = s2_unit32(p.scale_log2, sm.tempty, t2, g, lam);
           }
         }
 #pragma unroll 1
@@ -568,9 +485,11 @@ __device__ __forceinline__ void softmax_wg(const ScoreParams& p, const Smem& sm,
           const int k = (u * kPack + tsub) * kTileKeys + lrow;  // this thread's key, from the item's first
           float sum = 0.f;
           if (rows_none || k - lrow >= nkeys)
-            unit_release(sm, g);
+            unit_release(sm.tempty, g);
           else
-            sum = s2_unit_edge(p, sm, t2, g, lam, r0, nrows, it.key0 + k, it.n);
+            // row r sits at n - W + r % W and sees the keys up to there
+            sum = s2_unit_edge(p.scale_log2, sm.tempty, t2, g, lam, nrows, p.R - r0, r0 % p.W, p.W,
+                               k < nkeys ? it.key0 + k - (it.n - p.W) : p.W, p.W);
           *red = sum;
         }
         named_bar_sync(1, 128 * kSoftmaxWGs);

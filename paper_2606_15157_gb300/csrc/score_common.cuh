@@ -101,6 +101,90 @@ __device__ __forceinline__ void s2_chunk_full(const uint32_t (&rr)[32], float c,
   }
 }
 
+// ---- one TMEM unit of a softmax warp ----------------------------------------
+// A warp copies its columns of a unit (the unit's first slot is g mod kSlots)
+// to registers and releases the unit before any arithmetic.
+
+__device__ __forceinline__ void unit_release(uint64_t* tempty, uint32_t g) {
+  tc_fence_before();
+  __syncwarp();
+  mbar_arrive_elect(&tempty[g & (kSlots - 1)]);
+}
+
+// Sweep 1: the thread's row of one 128-row group against this warpgroup's 64
+// keys k0 .. k0 + 63; with kMask only the keys its position tr can see.
+template <bool kMask>
+__device__ __forceinline__ void s1_unit(float c, uint64_t* tempty, uint32_t taddr, uint32_t g, int k0, int tr, float& m,
+                                        float& z) {
+  uint32_t r0[32], r1[32];
+  tmem_ld64_async(taddr + (g & (kSlots - 1)) * kSlotCols, r0, r1);
+  tmem_wait64(r0, r1);
+  unit_release(tempty, g);
+  float v0[32], v1[32];
+#pragma unroll
+  for (int q = 0; q < 32; ++q) {
+    v0[q] = __uint_as_float(r0[q]);
+    v1[q] = __uint_as_float(r1[q]);
+  }
+  if (kMask) {
+    mask_chunk(v0, k0, tr);
+    mask_chunk(v1, k0 + 32, tr);
+  }
+  s1_chunk64(v0, v1, c, m, z);
+}
+
+// Sweep 2: this thread's key against 64 (or 32) rows that all exist and all
+// see it; nl = -lse2 of the rows.
+__device__ __forceinline__ float s2_unit64(float c, uint64_t* tempty, uint32_t taddr, uint32_t g, const float* nl) {
+  uint32_t ra[32], rb[32];
+  tmem_ld64_async(taddr + (g & (kSlots - 1)) * kSlotCols, ra, rb);
+  tmem_wait64(ra, rb);
+  unit_release(tempty, g);
+  float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  s2_chunk_full(ra, c, nl, a);
+  s2_chunk_full(rb, c, nl + 32, a);
+  return sum4x2(a);
+}
+
+__device__ __forceinline__ float s2_unit32(float c, uint64_t* tempty, uint32_t taddr, uint32_t g, const float* nl) {
+  uint32_t ra[32];
+  tmem_ld32_async(taddr + (g & (kSlots - 1)) * kSlotCols, ra);
+  tmem_wait32(ra);
+  unit_release(tempty, g);
+  float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  s2_chunk_full(ra, c, nl, a);
+  return sum4x2(a);
+}
+
+// Sweep 2 at the edges: up to nrows (64 or 32) rows, of which the first `exist`
+// exist; their place in a period of `per` rows counts up from i0, and a row
+// counts for this thread's key when its place is in [th, lim).  Any other gets
+// the exponent -inf.  The place is counted, not divided out of the row's index:
+// with a division per element the tiles at a prompt's end added 5 us to a 30 us
+// chunk of the window scores, and with four chunks per unit and 152 CTAs a
+// quarter of the CTAs are dealt every unit's last chunk (they finished at 232
+// us, the others at 195 us).
+__device__ __forceinline__ float s2_unit_edge(float c, uint64_t* tempty, uint32_t taddr, uint32_t g, const float* nl,
+                                              int nrows, int exist, int i0, int per, int th, int lim) {
+  float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  int i = i0;
+#pragma unroll 1
+  for (int h = 0; h < nrows && h < exist; h += 32) {
+    uint32_t rr[32];
+    tmem_ld32_async(taddr + (g & (kSlots - 1)) * kSlotCols + h, rr);
+    tmem_wait32(rr);
+#pragma unroll
+    for (int q = 0; q < 32; ++q) {
+      const float x = fmaf(__uint_as_float(rr[q]), c, lds1(nl + h + q));
+      const float e = ex2_approx(i >= th && i < lim && h + q < exist ? x : -INFINITY);
+      if (q & 1) a[(q >> 1) & 3].y += e; else a[(q >> 1) & 3].x += e;
+      i = i + 1 == per ? 0 : i + 1;
+    }
+  }
+  unit_release(tempty, g);
+  return sum4x2(a);
+}
+
 __device__ __forceinline__ float2 merge_ms(float2 a, float2 e) {  // (max, sum) in base 2
   if (e.x == -INFINITY) return a;
   if (a.x == -INFINITY) return e;

@@ -147,6 +147,17 @@ def test_h2o_full_prompt_scores_and_selection(torch, H_q, H_kv, d, lens, supplie
         assert torch.equal(a, b)
 
 
+# Prompts that end at, one before and one past a query block (256 / G
+# positions), a 128-key half and a 256-key super-tile; G = 5 leaves 255-row
+# blocks of 51 positions.
+@pytest.mark.parametrize("supplied_lse", [False, True])
+@pytest.mark.parametrize("H_q,H_kv,d,lens", [
+    (4, 1, 64, (64, 256, 255)), (4, 1, 128, (257, 320, 384)), (1, 1, 64, (256, 511)), (2, 1, 128, (385, 513)),
+    (10, 2, 64, (256, 255))])
+def test_h2o_full_prompt_block_edges(torch, H_q, H_kv, d, lens, supplied_lse):
+    test_h2o_full_prompt_scores_and_selection(torch, H_q, H_kv, d, lens, supplied_lse)
+
+
 def _full_prompt_workload(n, seed):
     route = [gen.H2O, gen.SNAPKV, gen.H2O]
     return gen.Workload(name=f"h2o_full_{n}", L=3, H_q=32, H_kv=8, d=128, B=1, lens=np.asarray([n], np.int32),
