@@ -902,7 +902,7 @@ int evict_impl(kvev_plan& P, DevCtx& D, const void* const* K, const void* const*
   sel.keys = reinterpret_cast<uint32_t*>(wsb + ws.sel_keys);
   sel.key_stride = sel_key_stride(S_cap);
   mark(KVEV_K_SELECT, 0);
-  if (launch_select(sel, P.L * B * P.H_kv, s) != cudaSuccess) return KVEV_ECUDA;
+  if (launch_select(sel, P.L * B * P.H_kv, D.num_sms, s) != cudaSuccess) return KVEV_ECUDA;
   mark(KVEV_K_SELECT, 1);
 
   // ---- gather-compaction ---------------------------------------------------

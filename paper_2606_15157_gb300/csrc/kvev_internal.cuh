@@ -45,8 +45,7 @@ constexpr int kRegsNeeded = 128 * kRegsControl + 128 * kSoftmaxWGs * kRegsSoftma
 // 128-row groups of the window rows (1, 2).
 constexpr int kScoreVariants = 4;
 constexpr int score_variant(int d, int R_pad) { return (d == 64 ? 0 : 1) + (R_pad > 128 ? 2 : 0); }
-constexpr int kSelectThreads = 256;    // one selection CTA per unit
-constexpr int kSelectCtasPerSm = 4;    // resident selection CTAs an SM should hold
+constexpr int kSelectThreadsPerSm = 1024;  // threads of resident selection CTAs an SM should hold (64 registers)
 constexpr int kWsAlign = 256;
 
 // Bits of the device status word.
@@ -608,6 +607,6 @@ cudaError_t h2o_full_set_smem(int d, size_t smem);
 cudaError_t launch_h2o_full(const ScoreParams& p, int d, int grid, size_t smem, cudaStream_t s);
 cudaError_t launch_lse_fill(const LseParams& p, cudaStream_t s);
 cudaError_t launch_lse_rows_fill(const ScoreParams& p, cudaStream_t s);
-cudaError_t launch_select(const SelectParams& p, int grid, cudaStream_t s);
+cudaError_t launch_select(const SelectParams& p, int grid, int num_sms, cudaStream_t s);
 cudaError_t launch_gather(const GatherParams& p, cudaStream_t s, int num_sms);
 }  // namespace kvev

@@ -23,13 +23,18 @@
 // that the copies' HBM traffic overlaps the latency-bound selections.
 //
 // A unit takes a CTA of 256 threads, so that several units share an SM and
-// one unit's barriers and round trips overlap another's passes.  Keys are an
+// one unit's barriers and round trips overlap another's passes (512 or 1,024
+// when there are few units).  Bound by those round trips and the shared-memory
+// atomics of the histogram; per launch, before and after position-ordered bins
+// (transposed ones were stored two bytes at a time), eight keys per thread and
+// trip, the early sample reads and the shuffle-ranked candidates: one 8K prompt
+// 22 and 15 us, one of 30K 42 and 30 us, four ragged ones of 12K-24K with
+// supplied scores 79 and 65 us, eight of 16K-32K 175 and 142 us.  Keys are an
 // order-preserving uint32 image of the fp32 (pooled) scores.  The unit's row
 // of a workspace array holds, between the two passes, each key's 16-bit bin
-// (transposed in 256-position blocks, so that one 16-byte load gives a lane
-// eight positions and a warp's ballots rank them by position); it stays in
-// L2:
-//   0. 1024 keys sampled at even strides give the bins: their range, widened
+// (in position order: a thread stores four at a time and loads eight, and a
+// warp scan of the lanes' counts ranks them by position); it stays in L2:
+//   0. keys sampled at even strides (eight per thread) give the bins: their range, widened
 //      by half on either side, split into 8192 bins of 2^s keys (a unit's
 //      scores may crowd into a few per cent of one octave, or spread over
 //      many octaves: the range adapts the bins to either);
@@ -43,6 +48,7 @@
 //      them, and their keys are recomputed from the scores;
 //   3. radix passes of up to 9 bits over the candidates fix the threshold key
 //      T and how many keys equal to T to keep (ties keep the lower position);
+//      at most 32 candidates are ranked with shuffles instead;
 //   4. every warp merges its staged positions and its kept candidates into
 //      its share of the output, after the shares of the warps before it.
 // An end bin, or a candidate list that overflows (many equal keys), takes the
@@ -55,23 +61,30 @@ namespace kvev {
 
 namespace {
 
-constexpr int kSW = kSelectThreads / 32;   // warps of a selection CTA
 constexpr int kBins0 = 8192;               // bins of the sampled range
-constexpr int kCandPerWarp = 320;          // candidates a warp's list holds
+constexpr int kCandidates = 2560;          // candidates the warps' lists hold together
+constexpr int kFewCandidates = 32;         // ranked by shuffles, one per lane
 constexpr int kBins1 = 512;                // candidate digits: up to 9 bits a pass
 constexpr int kSegKeys = 128;              // a key block: four keys per lane
 constexpr int kBinBlock = 256;             // a bin block: eight positions per lane
+constexpr int kAhead = 2;                  // bin blocks in flight per warp
 
+// NT: threads of a selection CTA.
+template <int NT>
 struct CandLists {
-  uint32_t pos[kSW][kCandPerWarp];
-  uint32_t key[kSW][kCandPerWarp];
-  int sure[kSW][kCandPerWarp];  // sure positions of the segment before the candidate
+  static constexpr int kSW = NT / 32, kPerWarp = kCandidates / kSW;
+  uint32_t pos[kSW][kPerWarp];
+  uint32_t key[kSW][kPerWarp];
+  int sure[kSW][kPerWarp];  // sure positions of the segment before the candidate
 };
 
+template <int NT>
 struct __align__(16) SelShared {
+  static constexpr int kSW = NT / 32;        // warps
+  static constexpr int kCandPerWarp = CandLists<NT>::kPerWarp;
   union {
     int hist[kBins0];
-    CandLists c;
+    CandLists<NT> c;
   } u;
   int hist1[kBins1];
   int wsum[kSW];
@@ -80,12 +93,13 @@ struct __align__(16) SelShared {
   int wgt[kSW];   // per warp segment: keys above T (general path) / candidates above T
   int weq[kSW];   // per warp segment: keys (candidates) equal to T
   int bcast[2];
+  uint32_t few[kFewCandidates];  // the candidates' keys in position order
   uint32_t rlo, rhi;  // sampled key range, then the candidates' key range
   int overflow;
 };
 
-static_assert(sizeof(SelShared) <= 48 * 1024, "the selection's shared memory is static");
-static_assert(sizeof(CandLists) <= sizeof(int) * kBins0, "the candidate lists reuse the histogram");
+static_assert(sizeof(SelShared<1024>) <= 48 * 1024, "the selection's shared memory is static");
+static_assert(sizeof(CandLists<1024>) <= sizeof(int) * kBins0, "the candidate lists reuse the histogram");
 
 // Adds each valid lane's digit to the histogram, one shared-memory atomic per
 // distinct digit of the warp (for digits that crowd into few bins).  Every
@@ -123,16 +137,18 @@ __device__ __forceinline__ int warp_sum(int x) {
   return x;
 }
 
-// The bin of a histogram of `nbins` digits (a multiple of the block size)
-// that holds the kk-th largest key (1 <= kk <= keys counted), and the number
-// of keys in higher bins.  Thread t owns the q = nbins / 256 bins
-// nbins-1-q*t down to nbins-q*(t+1).
-__device__ void find_bin(const int* hist, int nbins, int kk, SelShared& sh, int& digit, int& above) {
+// The bin of a histogram of `nbins` digits (a power of two) that holds the
+// kk-th largest key (1 <= kk <= keys counted), and the number of keys in
+// higher bins.  Thread t owns the q = nbins / NT (at least one) bins
+// nbins-1-q*t down to nbins-q*(t+1), or none.
+template <int NT>
+__device__ void find_bin(const int* hist, int nbins, int kk, SelShared<NT>& sh, int& digit, int& above) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int q = nbins / kSelectThreads;
+  const int q = max(1, nbins / NT);
   const int lo = nbins - q * (threadIdx.x + 1);  // this thread's lowest bin
   int s = 0;
-  if (q % 4 == 0) {
+  if (lo < 0) {
+  } else if (q % 4 == 0) {
     const int4* h4 = reinterpret_cast<const int4*>(hist + lo);
     for (int j = 0; j < q / 4; ++j) {
       const int4 v = h4[j];
@@ -160,7 +176,9 @@ __device__ void find_bin(const int* hist, int nbins, int kk, SelShared& sh, int&
 
 // Warp segments of [0, E): contiguous, whole 256-position blocks, in warp
 // order, so that a warp's kept positions follow those of the warps before it.
+template <int NT>
 __device__ __forceinline__ int seg_len(int E) {
+  constexpr int kSW = NT / 32;
   return ((E + kSW - 1) / kSW + kBinBlock - 1) / kBinBlock * kBinBlock;
 }
 
@@ -180,109 +198,109 @@ __device__ __forceinline__ uint4 ld_block_keys(const uint32_t* keys, int b0) {
   return __ldcg(reinterpret_cast<const uint4*>(keys + b0 + 4 * (threadIdx.x & 31)));
 }
 
-// The fast path keeps 16-bit bins instead of keys, in 256-position blocks
-// transposed the same way: the bin of position b + 32u + L (u < 8) sits at
-// 16-bit index b + 8L + u, so one 16-byte load gives lane L eight positions.
-__device__ __forceinline__ int tpos16(int i) { return (i & ~255) | ((i & 31) << 3) | ((i >> 5) & 7); }
-
+// The fast path keeps 16-bit bins instead of keys, in position order: one
+// 16-byte load gives lane L positions b + 8L .. b + 8L + 7 of a 256-position
+// block.
 __device__ __forceinline__ uint4 ld_block_bins(const uint16_t* bins, int b0) {
   return __ldcg(reinterpret_cast<const uint4*>(bins + b0 + 8 * (threadIdx.x & 31)));
 }
 
-__device__ __forceinline__ uint32_t pick16(const uint4& v, int u) {
-  const uint32_t w = pick(v, u >> 1);
-  return (u & 1) ? (w >> 16) : (w & 0xFFFFu);
-}
-
-
 // Bulk prefetch of the floats [src, src + n) into L2, in 16 KiB pieces, one
 // per thread (the row is 16-byte aligned and padded to whole 16-byte blocks).
+template <int NT>
 __device__ __forceinline__ void prefetch_row_l2(const float* src, int n) {
   const uintptr_t a0 = reinterpret_cast<uintptr_t>(src);
   const uintptr_t a1 = (reinterpret_cast<uintptr_t>(src + n) + 15) & ~uintptr_t(15);
-  for (uintptr_t a = a0 + static_cast<uintptr_t>(threadIdx.x) * 16384; a < a1; a += 16384u * kSelectThreads) {
+  for (uintptr_t a = a0 + static_cast<uintptr_t>(threadIdx.x) * 16384; a < a1; a += 16384u * NT) {
     const uint32_t bytes = static_cast<uint32_t>(a1 - a < 16384 ? a1 - a : 16384);
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"(bytes) : "memory");
   }
 }
 
 // ---------------------------------------------------------------------------
-// Key generators: four consecutive keys of [0, E) from position i0 (a multiple
-// of four, i0 < E), in two halves -- load() issues the reads, keys() computes
+// Key generators: eight consecutive keys of [0, E) from position i0 (a multiple
+// of eight, i0 < E), in two halves -- load() issues the reads, keys() computes
 // -- so that a pass can have the next block's reads in flight while it works
 // on the current one.  Keys past E are computed but never used.
 // ---------------------------------------------------------------------------
+constexpr int kGen = 8;
 
 // Pooled keys from a 16-byte aligned score row (S_cap a multiple of 4): keys
-// i0 .. i0+3 have windows (P <= 9) inside the three aligned 4-float chunks
-// starting at i0 - 4, i0 and i0 + 4.  Only chunks that start before E are
+// i0 .. i0+7 have windows (P <= 9) inside the four aligned 4-float chunks
+// starting at i0 - 4 .. i0 + 8.  Only chunks that start before E are
 // read (none leaves the row); entries outside [0, E) count as -inf (max) or 0
 // (avg).  Avg pooling divides every window sum by the same p, so the sum
 // ranks the keys alike and is used instead.
-template <int P>
-struct Pooled4 {
+template <int P, bool kMax>
+struct Pooled {
+  static constexpr bool kRow = true;  // a 16-byte aligned row
   const float* raw;
   int E;
-  bool is_max;
+  static constexpr float kFill = kMax ? -INFINITY : 0.f;
   struct Regs {
-    float4 c[3];
+    float4 c[4];
   };
   __device__ __forceinline__ void load(int i0, Regs& r) const {
-    const float fill = is_max ? -INFINITY : 0.f;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
+    for (int c = 0; c < 4; ++c) {
       const int st = i0 - 4 + 4 * c;
-      r.c[c] = make_float4(fill, fill, fill, fill);
+      r.c[c] = make_float4(kFill, kFill, kFill, kFill);
       if (st >= 0 && st < E) r.c[c] = __ldg(reinterpret_cast<const float4*>(raw + st));  // neighbours': L1
     }
   }
-  __device__ __forceinline__ void keys(int i0, const Regs& r, uint32_t (&kq)[4]) const {
+  __device__ __forceinline__ void keys(int i0, const Regs& r, uint32_t (&kq)[kGen]) const {
     constexpr int h = P / 2;
-    static_assert(h <= 4, "the three chunks cover windows of up to 9");
-    float w[12];
+    static_assert(h <= 4, "the chunks cover windows of up to 9");
+    float w[16];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
+    for (int c = 0; c < 4; ++c) {
       w[4 * c + 0] = r.c[c].x;
       w[4 * c + 1] = r.c[c].y;
       w[4 * c + 2] = r.c[c].z;
       w[4 * c + 3] = r.c[c].w;
     }
-    if (i0 + 8 > E) {  // the last chunk may run past E
-      const float fill = is_max ? -INFINITY : 0.f;
+    if (i0 + 12 > E) {  // the last chunks may run past E
 #pragma unroll
-      for (int j = 0; j < 12; ++j)
-        if (i0 - 4 + j >= E) w[j] = fill;
+      for (int j = 0; j < 16; ++j)
+        if (i0 - 4 + j >= E) w[j] = kFill;
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < kGen; ++u) {
       float v = w[4 + u - h];
 #pragma unroll
-      for (int j = 1; j < P; ++j) v = is_max ? fmaxf(v, w[4 + u - h + j]) : v + w[4 + u - h + j];
+      for (int j = 1; j < P; ++j) v = kMax ? fmaxf(v, w[4 + u - h + j]) : v + w[4 + u - h + j];
       kq[u] = float_key(v);
     }
   }
 };
 
-// Raw keys (no pooling) from a 16-byte aligned score row.
-struct Raw4 {
+// Raw keys (no pooling) from a 16-byte aligned score row; only chunks that
+// start before E are read.
+struct Raw {
+  static constexpr bool kRow = true;  // a 16-byte aligned row
   const float* raw;
   int E;
   struct Regs {
-    float4 v;
+    float4 v[2];
   };
   __device__ __forceinline__ void load(int i0, Regs& r) const {
-    r.v = __ldg(reinterpret_cast<const float4*>(raw + i0));
+    r.v[0] = __ldg(reinterpret_cast<const float4*>(raw + i0));
+    r.v[1] = i0 + 4 < E ? __ldg(reinterpret_cast<const float4*>(raw + i0 + 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  __device__ __forceinline__ void keys(int, const Regs& r, uint32_t (&kq)[4]) const {
-    kq[0] = float_key(r.v.x);
-    kq[1] = float_key(r.v.y);
-    kq[2] = float_key(r.v.z);
-    kq[3] = float_key(r.v.w);
+  __device__ __forceinline__ void keys(int, const Regs& r, uint32_t (&kq)[kGen]) const {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      kq[4 * c + 0] = float_key(r.v[c].x);
+      kq[4 * c + 1] = float_key(r.v[c].y);
+      kq[4 * c + 2] = float_key(r.v[c].z);
+      kq[4 * c + 3] = float_key(r.v[c].w);
+    }
   }
 };
 
 // Any alignment and any odd pooling width: scalar loads, all in keys().
-struct Scalar4 {
+struct Scalar {
+  static constexpr bool kRow = false;
   const float* raw;
   int E, h;
   bool do_pool, is_max;
@@ -295,22 +313,31 @@ struct Scalar4 {
     return float_key(v);
   }
   __device__ __forceinline__ void load(int, Regs&) const {}
-  __device__ __forceinline__ void keys(int i0, const Regs&, uint32_t (&kq)[4]) const {
+  __device__ __forceinline__ void keys(int i0, const Regs&, uint32_t (&kq)[kGen]) const {
+#pragma unroll 1
+    for (int u = 0; u < kGen; u += 4) {
+      uint32_t q[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) kq[u] = i0 + u < E ? one(i0 + u) : 0u;
+      for (int v = 0; v < 4; ++v) q[v] = i0 + u + v < E ? one(i0 + u + v) : 0u;
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        if (u == 0) kq[v] = q[v];
+        else kq[4 + v] = q[v];
+      }
+    }
   }
 };
 
 template <class Gen>
-__device__ __forceinline__ void gen_keys(const Gen& gen, int i0, uint32_t (&kq)[4]) {
+__device__ __forceinline__ void gen_keys(const Gen& gen, int i0, uint32_t (&kq)[kGen]) {
   typename Gen::Regs r;
   gen.load(i0, r);
   gen.keys(i0, r, kq);
 }
 
 // ---------------------------------------------------------------------------
-// Step 0: the bracket.  Sample keys: thread t takes the group of four at
-// 4 * floor(t * ceil(E / 4) / 256).  Their range is widened by half of it on
+// Step 0: the bins.  Sample keys: thread t takes the group of eight at
+// 8 * floor(t * ceil(E / 8) / NT).  Their range is widened by half of it on
 // either side (at least 4096 key steps) and split into 8192 bins.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ Binning make_binning(uint32_t a, uint32_t b) {
@@ -323,22 +350,22 @@ __device__ __forceinline__ Binning make_binning(uint32_t a, uint32_t b) {
   return bn;
 }
 
-struct Bracket {
-  Binning bn;
-  uint32_t lo_bin, hi_bin;  // candidates: bins lo_bin .. hi_bin; sure: bins above hi_bin
-};
+template <int NT>
+__device__ __forceinline__ int sample_pos(int E) {
+  const int groups = (E + kGen - 1) / kGen;
+  return kGen * static_cast<int>((static_cast<long long>(threadIdx.x) * groups) / NT);
+}
 
-// The binning of the unit's keys from its sample.  Needs sh.rlo / sh.rhi
-// initialised.
-template <class Gen>
-__device__ Binning sample_binning(const Gen& gen, int E, SelShared& sh) {
-  const int groups = (E + 3) / 4;
-  const int i0 = 4 * static_cast<int>((static_cast<long long>(threadIdx.x) * groups) / kSelectThreads);
-  uint32_t kq[4];
-  gen_keys(gen, i0, kq);
+// The binning of the unit's keys from its sample, whose reads are in `r`.
+// Needs sh.rlo / sh.rhi initialised.
+template <int NT, class Gen>
+__device__ Binning sample_binning(const Gen& gen, const typename Gen::Regs& r, int E, SelShared<NT>& sh) {
+  const int i0 = sample_pos<NT>(E);
+  uint32_t kq[kGen];
+  gen.keys(i0, r, kq);
   uint32_t lo = 0xFFFFFFFFu, hi = 0u;
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
+  for (int u = 0; u < kGen; ++u) {
     if (i0 + u < E) {
       lo = min(lo, kq[u]);
       hi = max(hi, kq[u]);
@@ -354,71 +381,97 @@ __device__ Binning sample_binning(const Gen& gen, int E, SelShared& sh) {
   return make_binning(sh.rlo, sh.rhi);
 }
 
-// Step 1: the bin of every key of [0, E) into the unit's workspace row (16-bit
-// transposed blocks), and the histogram of the bins.
-template <class Gen>
+// Step 1: the bin of every key of [0, E) into the unit's workspace row (16 bits
+// each, a thread's eight in one store; the row is padded to whole groups), and
+// the histogram of the bins.
+template <int NT, class Gen>
 __device__ void build_row_hist(const Gen& gen, uint16_t* bins, int E, Binning bn, int* hist) {
   typename Gen::Regs nxt;
-  int i0 = 4 * threadIdx.x;
+  int i0 = kGen * threadIdx.x;
   if (i0 < E) gen.load(i0, nxt);
-  for (; i0 < E; i0 += 4 * kSelectThreads) {
+  for (; i0 < E; i0 += kGen * NT) {
     const typename Gen::Regs cur = nxt;
-    if (i0 + 4 * kSelectThreads < E) gen.load(i0 + 4 * kSelectThreads, nxt);  // next reads go out first
-    uint32_t kq[4];
-    gen.keys(i0, cur, kq);
+    if (i0 + kGen * NT < E) gen.load(i0 + kGen * NT, nxt);  // next reads go out first
+    uint32_t b[kGen];
+    gen.keys(i0, cur, b);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (i0 + u < E) {
-        const uint32_t b = bn.bin(kq[u]);
-        bins[tpos16(i0 + u)] = static_cast<uint16_t>(b);
-        atomicAdd(&hist[b], 1);
-      }
+    for (int u = 0; u < kGen; ++u) {
+      b[u] = bn.bin(b[u]);
+      if (i0 + u < E) atomicAdd(&hist[b[u]], 1);
     }
+    *reinterpret_cast<uint4*>(bins + i0) =
+        make_uint4(b[0] | b[1] << 16, b[2] | b[3] << 16, b[4] | b[5] << 16, b[6] | b[7] << 16);
   }
 }
 
 // ---------------------------------------------------------------------------
 // Step 2: each warp walks its segment [lo, hi) of the bins in order.  Keys of
-// bins above the bracket are kept for sure: their positions are staged, in
-// order, as 16-bit offsets at the start of the segment's row (a warp only
-// overwrites entries of positions it has passed, and has the next block's
-// bins in registers).  Keys inside the bracket (the candidates) go to the
-// warp's list with the count of sure positions before them; their keys are
+// bins above d are kept for sure: their positions are staged, in order, as
+// 16-bit offsets at the start of the segment's row (a warp only overwrites
+// entries of positions it has passed, and has the next block's bins in
+// registers).  Keys of bin d (the candidates) go to the warp's list with the count of sure positions before them; their keys are
 // recomputed from the scores afterwards.  A list that fills up sets
 // sh.overflow.
 // ---------------------------------------------------------------------------
-__device__ void classify_pass(uint16_t* bins, int E, const Bracket& br, SelShared& sh) {
+// Bits 15 and 31 of `t` (the two 16-bit halves of word j of a lane's eight
+// bins) as bits 2j and 2j + 1.
+__device__ __forceinline__ uint32_t half_bits(uint32_t t, int j) {
+  return ((t >> 15) & 1u) << (2 * j) | (t >> 31) << (2 * j + 1);
+}
+
+template <int NT>
+__device__ void classify_pass(uint16_t* bins, int E, uint32_t d, SelShared<NT>& sh) {
+  constexpr int kCandPerWarp = SelShared<NT>::kCandPerWarp;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t lt = (1u << lane) - 1u;
-  const int seg = seg_len(E);
+  const int seg = seg_len<NT>(E);
   const int lo = min(warp * seg, E), hi = min(lo + seg, E);
+  // Bins are below 2^13, so (q | 0x8000) - x keeps bit 15 exactly when q >= x,
+  // for both halves of a word at once.
+  const uint32_t above = (d + 1) * 0x00010001u, from = d * 0x00010001u;
   int ns = 0, nc = 0;  // sure positions staged, candidates listed
-  uint4 nxt = make_uint4(0, 0, 0, 0);
-  if (lo < hi) nxt = ld_block_bins(bins, lo);
-  for (int b0 = lo; b0 < hi; b0 += kBinBlock) {
-    const uint4 cur = nxt;
-    if (b0 + kBinBlock < hi) nxt = ld_block_bins(bins, b0 + kBinBlock);  // the next block goes out first
+  uint4 nxt[kAhead];  // the next blocks' bins
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int p = b0 + 32 * u + lane;
-      const uint32_t q = pick16(cur, u);
-      const bool valid = p < hi;
-      const bool sure = valid && q > br.hi_bin;
-      const bool cand = valid && q >= br.lo_bin && q <= br.hi_bin;
-      const uint32_t bs = __ballot_sync(0xffffffffu, sure), bc = __ballot_sync(0xffffffffu, cand);
-      const int js = ns + __popc(bs & lt);
-      // staged as offsets from the segment start, behind the positions already read
-      if (sure) bins[lo + js] = static_cast<uint16_t>(p - lo);
-      if (cand) {
-        const int jc = nc + __popc(bc & lt);
-        if (jc < kCandPerWarp) {
-          sh.u.c.pos[warp][jc] = static_cast<uint32_t>(p);
-          sh.u.c.sure[warp][jc] = js;
-        }
-      }
-      ns += __popc(bs);
-      nc += __popc(bc);
+  for (int a = 0; a < kAhead; ++a) {
+    nxt[a] = make_uint4(0, 0, 0, 0);
+    if (lo + a * kBinBlock < hi) nxt[a] = ld_block_bins(bins, lo + a * kBinBlock);
+  }
+  for (int b0 = lo; b0 < hi; b0 += kBinBlock) {
+    const uint4 cur = nxt[0];
+#pragma unroll
+    for (int a = 0; a + 1 < kAhead; ++a) nxt[a] = nxt[a + 1];
+    if (b0 + kAhead * kBinBlock < hi) nxt[kAhead - 1] = ld_block_bins(bins, b0 + kAhead * kBinBlock);
+    uint32_t sm = 0, cm = 0;  // the lane's sure positions and candidates, bit u: position p0 + u
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t w = pick(cur, j) | 0x80008000u;
+      sm |= half_bits(w - above, j);
+      cm |= half_bits(w - from, j);
     }
+    cm &= ~sm;
+    const int p0 = b0 + 8 * lane;
+    if (p0 + 8 > hi) {
+      const uint32_t valid = p0 < hi ? (1u << (hi - p0)) - 1u : 0u;
+      sm &= valid;
+      cm &= valid;
+    }
+    const int mine = __popc(sm) | __popc(cm) << 16;
+    const int incl = warp_incl(mine);
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    const int js = ns + ((incl - mine) & 0xFFFF);
+    int jc = nc + ((incl - mine) >> 16);
+    __syncwarp();  // every lane has its bins of this block before they are overwritten
+    // staged as offsets from the segment start, behind the positions already read
+    for (uint32_t m = sm, j = js; m != 0; m &= m - 1, ++j)
+      bins[lo + j] = static_cast<uint16_t>(p0 - lo + __ffs(m) - 1);
+    for (uint32_t m = cm; m != 0; m &= m - 1, ++jc) {
+      const int u = __ffs(m) - 1;
+      if (jc < kCandPerWarp) {
+        sh.u.c.pos[warp][jc] = static_cast<uint32_t>(p0 + u);
+        sh.u.c.sure[warp][jc] = js + __popc(sm & ((1u << u) - 1u));
+      }
+    }
+    ns += total & 0xFFFF;
+    nc += total >> 16;
   }
   if (lane == 0) {
     sh.wS[warp] = ns;
@@ -428,16 +481,68 @@ __device__ void classify_pass(uint16_t* bins, int E, const Bracket& br, SelShare
 }
 
 // The keys of each warp's listed candidates, from the scores.
-__device__ void candidate_keys(const Scalar4& sk, SelShared& sh) {
+template <int NT>
+__device__ void candidate_keys(const Scalar& sk, SelShared<NT>& sh) {
+  constexpr int kCandPerWarp = SelShared<NT>::kCandPerWarp;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nc = min(sh.wC[warp], kCandPerWarp);
   for (int i = lane; i < nc; i += 32) sh.u.c.key[warp][i] = sk.one(static_cast<int>(sh.u.c.pos[warp][i]));
 }
 
+// Steps 3 and 4 for at most 32 candidates (the sampled bins leave a handful as
+// a rule): the candidates' keys go to one array in position order, and every
+// warp ranks all of them with shuffles (a larger key, or an equal one of a
+// lower position, ranks before), so one barrier replaces the radix passes and
+// counts.  The kk best are kept; each warp then writes its share of the output,
+// which starts after the shares of the warps before it: a kept candidate goes
+// after the sure positions before it, a sure position after the kept
+// candidates before it.
+template <int NT>
+__device__ void finish_few(const Scalar& sk, const uint16_t* bins, int E, int kk, int k, int nd, SelShared<NT>& sh,
+                           int* out) {
+  constexpr int kSW = SelShared<NT>::kSW;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nc = sh.wC[warp], ns = sh.wS[warp];
+  const int c = lane < kSW ? sh.wC[lane] : 0;
+  const int cincl = warp_incl(c);
+  const int first = __shfl_sync(0xffffffffu, cincl - c, warp);  // index of the warp's first candidate
+  const int sbefore = warp_sum(lane < warp ? sh.wS[lane] : 0);
+  uint32_t pos = 0;
+  int sure = 0;
+  if (lane < nc) {
+    pos = sh.u.c.pos[warp][lane];
+    sure = sh.u.c.sure[warp][lane];
+    sh.few[first + lane] = sk.one(static_cast<int>(pos));
+  }
+  __syncthreads();
+  const uint32_t key = lane < nd ? sh.few[lane] : 0u;
+  int rank = 0;
+  for (int j = 0; j < nd; ++j) {
+    const uint32_t o = __shfl_sync(0xffffffffu, key, j);
+    rank += o > key || (o == key && j < lane);
+  }
+  const uint32_t kept = __ballot_sync(0xffffffffu, lane < nd && rank < kk);
+  const uint32_t mine = nc == 0 ? 0u : (kept >> first) & (0xFFFFFFFFu >> (32 - nc));
+  const int base = sbefore + (first >= 32 ? __popc(kept) : __popc(kept & ((1u << first) - 1u)));
+  if (mine >> lane & 1u) {
+    const int o = base + sure + __popc(mine & ((1u << lane) - 1u));
+    if (o < k) out[o] = static_cast<int>(pos);
+  }
+  const int lo = min(warp * seg_len<NT>(E), E);
+  for (int j0 = 0; j0 < ns; j0 += 32) {
+    const int j = j0 + lane;
+    int o = base + j;
+    for (uint32_t m = mine; m != 0; m &= m - 1) o += __shfl_sync(0xffffffffu, sure, __ffs(m) - 1) <= j;
+    if (j < ns && o < k) out[o] = lo + static_cast<int>(__ldcg(bins + lo + j));
+  }
+}
+
 // Step 3: threshold key T (the kk-th largest candidate) and how many keys
 // equal to T to keep, by radix passes of up to 9 bits over key - (least
 // candidate key); then each warp counts its candidates above and equal to T.
-__device__ void select_candidates(int kk, SelShared& sh, uint32_t& T, int& need) {
+template <int NT>
+__device__ void select_candidates(int kk, SelShared<NT>& sh, uint32_t& T, int& need) {
+  constexpr int kSW = SelShared<NT>::kSW, kCandPerWarp = SelShared<NT>::kCandPerWarp;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
     sh.rlo = 0xFFFFFFFFu;
@@ -462,9 +567,9 @@ __device__ void select_candidates(int kk, SelShared& sh, uint32_t& T, int& need)
   for (int r = bits; r > 0;) {
     const int nb = min(9, r), shift = r - nb;
     const uint32_t dm = (1u << nb) - 1u;
-    for (int i = threadIdx.x; i < kBins1; i += kSelectThreads) sh.hist1[i] = 0;
+    for (int i = threadIdx.x; i < kBins1; i += NT) sh.hist1[i] = 0;
     __syncthreads();
-    for (int c = threadIdx.x; c < kSW * kCandPerWarp; c += kSelectThreads) {
+    for (int c = threadIdx.x; c < kSW * kCandPerWarp; c += NT) {
       const int w = c / kCandPerWarp, i = c - w * kCandPerWarp;
       if (i < sh.wC[w]) {
         const uint32_t v = sh.u.c.key[w][i] - clo;
@@ -501,7 +606,8 @@ __device__ void select_candidates(int kk, SelShared& sh, uint32_t& T, int& need)
 // base + (sure positions before it) + (kept candidates before it); its sure
 // position j to base + j + (kept candidates with at most j sure positions
 // before them).
-__device__ void merge_write(const uint16_t* bins, int E, int k, int need, SelShared& sh, uint32_t T, int* out) {
+template <int NT>
+__device__ void merge_write(const uint16_t* bins, int E, int k, int need, SelShared<NT>& sh, uint32_t T, int* out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t lt = (1u << lane) - 1u;
   int base = 0, eq_base = 0;
@@ -535,7 +641,7 @@ __device__ void merge_write(const uint16_t* bins, int E, int k, int need, SelSha
     nk += __popc(kb);
     eq_base += __popc(eb);
   }
-  const int seg = seg_len(E);
+  const int seg = seg_len<NT>(E);
   const int lo = min(warp * seg, E);
   const int ns = sh.wS[warp];
   for (int j = lane; j < ns; j += 32) {
@@ -552,12 +658,14 @@ __device__ void merge_write(const uint16_t* bins, int E, int k, int need, SelSha
 
 // The general path: four 8-bit radix passes over every key, then each warp
 // counts its segment's keys above and equal to T.
-__device__ void select_all_keys(const uint32_t* keys, int E, int k, SelShared& sh, uint32_t& T, int& need) {
+template <int NT>
+__device__ void select_all_keys(const uint32_t* keys, int E, int k, SelShared<NT>& sh, uint32_t& T, int& need) {
+  constexpr int kSW = SelShared<NT>::kSW;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t prefix = 0, mask = 0;
   int kk = k;
   for (int shift = 24; shift >= 0; shift -= 8) {
-    for (int i = threadIdx.x; i < 256; i += kSelectThreads) sh.hist1[i] = 0;
+    for (int i = threadIdx.x; i < 256; i += NT) sh.hist1[i] = 0;
     __syncthreads();
     for (int b0 = 128 * warp; b0 < E; b0 += 128 * kSW) {  // blocks dealt to the warps in turn
       const uint4 kv = ld_block_keys(keys, b0);
@@ -577,7 +685,7 @@ __device__ void select_all_keys(const uint32_t* keys, int E, int k, SelShared& s
   }
   T = prefix;
   need = kk;
-  const int seg = seg_len(E);
+  const int seg = seg_len<NT>(E);
   const int lo = min(warp * seg, E), hi = min(lo + seg, E);
   int gt = 0, eq = 0;
   for (int b0 = lo; b0 < hi; b0 += kSegKeys) {
@@ -603,11 +711,12 @@ __device__ void select_all_keys(const uint32_t* keys, int E, int k, SelShared& s
 // out[0..k): keys above T, and the first `need` keys equal to T in position
 // order.
 // ---------------------------------------------------------------------------
-__device__ void write_kept(const uint32_t* keys, int E, int k, uint32_t T, int need, const SelShared& sh,
+template <int NT>
+__device__ void write_kept(const uint32_t* keys, int E, int k, uint32_t T, int need, const SelShared<NT>& sh,
                            int* out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t lt = (1u << lane) - 1u;
-  const int seg = seg_len(E);
+  const int seg = seg_len<NT>(E);
   const int lo = min(warp * seg, E), hi = min(lo + seg, E);
   int eq_base = 0, sel_base = 0;
   for (int w = 0; w < warp; ++w) {
@@ -635,43 +744,46 @@ __device__ void write_kept(const uint32_t* keys, int E, int k, uint32_t T, int n
 
 // Every key of [0, E) into the unit's workspace row, transposed blocks (the
 // general path).
-template <class Gen>
+template <int NT, class Gen>
 __device__ void build_row(const Gen& gen, uint32_t* row, int E) {
-  for (int i0 = 4 * threadIdx.x; i0 < E; i0 += 4 * kSelectThreads) {
-    uint32_t kq[4];
+  for (int i0 = kGen * threadIdx.x; i0 < E; i0 += kGen * NT) {
+    uint32_t kq[kGen];
     gen_keys(gen, i0, kq);
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < kGen; ++u)
       if (i0 + u < E) row[tpos(i0 + u)] = kq[u];
   }
 }
 
 // Top-k of the keys of [0, E) (1 <= k < E) into out[0 .. k), ascending.
-template <class Gen>
-__device__ void select_unit(const Gen& gen, const Scalar4& sk, uint32_t* row, int E, int k, SelShared& sh,
+template <int NT, class Gen>
+__device__ void select_unit(const Gen& gen, const Scalar& sk, uint32_t* row, int E, int k, SelShared<NT>& sh,
                             int* out) {
-  for (int i = threadIdx.x; i < kBins0; i += kSelectThreads) sh.u.hist[i] = 0;
+  typename Gen::Regs sample;
+  gen.load(sample_pos<NT>(E), sample);  // the sample's reads go out first
+  if (Gen::kRow) prefetch_row_l2<NT>(sk.raw, E);  // the passes' score reads become L2 hits
+  for (int i = threadIdx.x; i < kBins0 / 4; i += NT) reinterpret_cast<int4*>(sh.u.hist)[i] = make_int4(0, 0, 0, 0);
   if (threadIdx.x == 0) {
     sh.rlo = 0xFFFFFFFFu;
     sh.rhi = 0u;
     sh.overflow = 0;
   }
   __syncthreads();
-  const Binning bn = sample_binning(gen, E, sh);
+  const Binning bn = sample_binning(gen, sample, E, sh);
   uint16_t* bins = reinterpret_cast<uint16_t*>(row);
-  build_row_hist(gen, bins, E, bn, sh.u.hist);
+  build_row_hist<NT>(gen, bins, E, bn, sh.u.hist);
   __syncthreads();
   int d, above;
   find_bin(sh.u.hist, kBins0, k, sh, d, above);  // ends with a barrier
   const int nd = sh.u.hist[d];
   __syncthreads();  // every thread has read it before the candidate lists overwrite the histogram
   // the end bins also hold keys outside the sampled range: not one prefix
-  bool fast = d > 0 && d < kBins0 - 1 && nd <= kSW * kCandPerWarp && seg_len(E) <= 65536;
+  bool fast = d > 0 && d < kBins0 - 1 && nd <= kCandidates && seg_len<NT>(E) <= 65536;
   if (fast) {
-    const Bracket br{bn, static_cast<uint32_t>(d), static_cast<uint32_t>(d)};
-    classify_pass(bins, E, br, sh);
+    classify_pass(bins, E, static_cast<uint32_t>(d), sh);
     __syncthreads();
     fast = !sh.overflow;
+    if (nd <= kFewCandidates) return finish_few(sk, bins, E, k - above, k, nd, sh, out);
     if (fast) {
       candidate_keys(sk, sh);
       __syncthreads();
@@ -686,7 +798,7 @@ __device__ void select_unit(const Gen& gen, const Scalar4& sk, uint32_t* row, in
   }
   // the general path: many equal keys, or a sample that missed the k-th key:
   // the row holds bins, so the keys are built now
-  build_row(gen, row, E);
+  build_row<NT>(gen, row, E);
   __syncthreads();
   select_all_keys(row, E, k, sh, T, need);
   write_kept(row, E, k, T, need, sh, out);
@@ -694,8 +806,9 @@ __device__ void select_unit(const Gen& gen, const Scalar4& sk, uint32_t* row, in
 
 // The sequence of rank r in order of decreasing length (equal lengths: lower
 // index first), by warp 0 (B <= 32; larger batches keep the index order).
-__device__ int seq_of_rank(const SelectParams& p, int r, SelShared& sh) {
-  if (p.B > 32) return r;
+template <int NT>
+__device__ int seq_of_rank(const SelectParams& p, int r, SelShared<NT>& sh) {
+  if (p.B == 1 || p.B > 32) return r;
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
     const int n = lane < p.B ? p.lens[lane] : -1;
@@ -714,6 +827,7 @@ __device__ int seq_of_rank(const SelectParams& p, int r, SelShared& sh) {
 // A StreamingLLM unit's kept rows (positions pos_j of slots j < count) into its
 // packed output rows, K and V as 16-byte vectors, four of each in flight per
 // thread; slots past the count are zero-filled.
+template <int NT>
 __device__ void copy_streaming_rows(const SelectParams& p, int l, int rem, int n, int count, bool identity) {
   const LayerDesc& ld = p.layer[l];
   const int vec = p.d / 8, total = ld.slots * vec;
@@ -724,11 +838,11 @@ __device__ void copy_streaming_rows(const SelectParams& p, int l, int rem, int n
   uint4* Kd = static_cast<uint4*>(p.out_K) + dst0;
   uint4* Vd = static_cast<uint4*>(p.out_V) + dst0;
   constexpr int kU = 4;
-  for (int i0 = threadIdx.x; i0 < total; i0 += kU * kSelectThreads) {
+  for (int i0 = threadIdx.x; i0 < total; i0 += kU * NT) {
     uint4 kv[kU], vv[kU];
 #pragma unroll
     for (int q = 0; q < kU; ++q) {
-      const int i = i0 + q * kSelectThreads;
+      const int i = i0 + q * NT;
       kv[q] = make_uint4(0, 0, 0, 0);
       vv[q] = make_uint4(0, 0, 0, 0);
       const int j = i / vec;
@@ -741,7 +855,7 @@ __device__ void copy_streaming_rows(const SelectParams& p, int l, int rem, int n
     }
 #pragma unroll
     for (int q = 0; q < kU; ++q) {
-      const int i = i0 + q * kSelectThreads;
+      const int i = i0 + q * NT;
       if (i < total) {
         __stcs(Kd + i, kv[q]);
         __stcs(Vd + i, vv[q]);
@@ -750,8 +864,9 @@ __device__ void copy_streaming_rows(const SelectParams& p, int l, int rem, int n
   }
 }
 
-__global__ void __launch_bounds__(kSelectThreads, kSelectCtasPerSm) select_kernel(const __grid_constant__ SelectParams p) {
-  __shared__ SelShared sh;
+template <int NT>
+__global__ void __launch_bounds__(NT, kSelectThreadsPerSm / NT) select_kernel(const __grid_constant__ SelectParams p) {
+  __shared__ SelShared<NT> sh;
   const int per_layer = p.B * p.H_kv;
   // dispatch order: two lists, each in (sequence rank, layer, head) order --
   // the first L_first layers of p.order (the scoring layers) and the rest --
@@ -790,7 +905,7 @@ __global__ void __launch_bounds__(kSelectThreads, kSelectCtasPerSm) select_kerne
       for (int j = threadIdx.x; j < count; j += blockDim.x)
         idx[j] = j < p.sink ? j : n - ld.recent + (j - p.sink);
     }
-    copy_streaming_rows(p, l, rem, n, count, identity);
+    copy_streaming_rows<NT>(p, l, rem, n, count, identity);
   } else {
     identity = n <= b_l;
     count = identity ? n : b_l;
@@ -817,15 +932,18 @@ __global__ void __launch_bounds__(kSelectThreads, kSelectCtasPerSm) select_kerne
   uint32_t* row = p.keys + (static_cast<size_t>(ld.score_slot) * per_layer + rem) * p.key_stride;
   const bool do_pool = ld.method == KVEV_SNAPKV, is_max = p.pool_type == KVEV_POOL_MAX;
   const bool aligned4 = (reinterpret_cast<uintptr_t>(raw) & 15u) == 0 && (p.S_cap & 3) == 0;
-  if (aligned4) prefetch_row_l2(raw, E);  // the passes' score reads become L2 hits
-  const Scalar4 sk{raw, E, p.pool_kernel / 2, do_pool, is_max};  // one key at a time (candidates)
-  if (aligned4 && !do_pool) return select_unit(Raw4{raw, E}, sk, row, E, k, sh, idx);
+  const Scalar sk{raw, E, p.pool_kernel / 2, do_pool, is_max};  // one key at a time (candidates)
+  if (aligned4 && !do_pool) return select_unit(Raw{raw, E}, sk, row, E, k, sh, idx);
   if (aligned4) {
-    switch (p.pool_kernel) {
-      case 3: return select_unit(Pooled4<3>{raw, E, is_max}, sk, row, E, k, sh, idx);
-      case 5: return select_unit(Pooled4<5>{raw, E, is_max}, sk, row, E, k, sh, idx);
-      case 7: return select_unit(Pooled4<7>{raw, E, is_max}, sk, row, E, k, sh, idx);
-      case 9: return select_unit(Pooled4<9>{raw, E, is_max}, sk, row, E, k, sh, idx);
+    switch (2 * p.pool_kernel + is_max) {
+      case 6: return select_unit(Pooled<3, false>{raw, E}, sk, row, E, k, sh, idx);
+      case 7: return select_unit(Pooled<3, true>{raw, E}, sk, row, E, k, sh, idx);
+      case 10: return select_unit(Pooled<5, false>{raw, E}, sk, row, E, k, sh, idx);
+      case 11: return select_unit(Pooled<5, true>{raw, E}, sk, row, E, k, sh, idx);
+      case 14: return select_unit(Pooled<7, false>{raw, E}, sk, row, E, k, sh, idx);
+      case 15: return select_unit(Pooled<7, true>{raw, E}, sk, row, E, k, sh, idx);
+      case 18: return select_unit(Pooled<9, false>{raw, E}, sk, row, E, k, sh, idx);
+      case 19: return select_unit(Pooled<9, true>{raw, E}, sk, row, E, k, sh, idx);
       default: break;
     }
   }
@@ -834,9 +952,18 @@ __global__ void __launch_bounds__(kSelectThreads, kSelectCtasPerSm) select_kerne
 
 }  // namespace
 
-cudaError_t launch_select(const SelectParams& p, int grid, cudaStream_t s) {
+cudaError_t launch_select(const SelectParams& p, int grid, int num_sms, cudaStream_t s) {
   if (grid == 0) return cudaSuccess;
-  select_kernel<<<grid, kSelectThreads, 0, s>>>(p);
+  // As many threads per unit as leave every unit resident at once: a unit's
+  // passes are chains of L2 round trips and barriers, which more threads
+  // shorten while the SMs have room.  One 8,192-token prompt (256 units): 18.5
+  // us with 256 threads, 15.2 with 512, 28 with 1,024 (two rounds of units).
+  if (grid <= num_sms)
+    select_kernel<1024><<<grid, 1024, 0, s>>>(p);
+  else if (grid <= 2 * num_sms)
+    select_kernel<512><<<grid, 512, 0, s>>>(p);
+  else
+    select_kernel<256><<<grid, 256, 0, s>>>(p);
   return cudaGetLastError();
 }
 

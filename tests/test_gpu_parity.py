@@ -315,6 +315,42 @@ def test_select_crowded_first_bin(torch, orc):
     parity.check_workload(wl, dev, wl.lens)
 
 
+@pytest.mark.parametrize("B", [1, 60, 110])  # 1,024, 512 and 256 threads per unit
+@pytest.mark.parametrize("levels", [5, 40, 400, 0])
+def test_select_score_levels(torch, B, levels):
+    # Selection alone, from supplied scores of `levels` distinct values (0: all
+    # distinct): everything in a few bins (the general path), a threshold bin of
+    # hundreds or tens of equal keys (radix passes), and of a handful (shuffles),
+    # with prompts that end around the key groups of eight, the bin blocks of
+    # 256 and the warps' segments.  Against a stable sort: a larger score
+    # first, equal ones by position.
+    from paper_2606_15157_gb300 import kvev
+    rng = np.random.default_rng(100 * B + levels)
+    W, S_cap, b = 8, 4160, 150
+    lens = np.array(([4160] if B == 1 else [151, 159, 160, 263, 264, 265, 519, 520, 2056, 2057, 4159, 4160] * 10)[:B],
+                    np.int32)
+    raw = rng.random((2, B, 2, S_cap)).astype(np.float32) ** 4
+    if levels:
+        raw = np.ceil(raw * levels).astype(np.float32) / np.float32(levels)
+    plan = kvev.Plan(2, 2, 2, 64, [gen.H2O, gen.SNAPKV], [b, b], W, 5, gen.POOL_MAX, h2o_recent=0)
+    bufs = plan.buffers(B, S_cap)
+    kv = torch.zeros((B, 2, S_cap, 64), dtype=torch.bfloat16, device="cuda")
+    scores = [torch.from_numpy(raw[l]).cuda() for l in range(2)]
+    plan.evict_prefill([kv, kv], [kv, kv], None, torch.from_numpy(lens).cuda(), B, S_cap, bufs, scores=scores)
+    torch.cuda.synchronize()
+    assert plan.status() == kvev.OK
+    idx = bufs["out_idx"].cpu().numpy()[: 2 * B * 2 * b].reshape(2, B, 2, b)
+    for s, n in enumerate(lens):
+        for h in range(2):
+            keep = np.sort(np.argsort(-raw[0, s, h, :n], kind="stable")[:b])
+            assert np.array_equal(idx[0, s, h], keep), f"H2O n={n}"
+            E = n - W
+            pad = np.pad(raw[1, s, h, :E], 2, constant_values=-np.inf)
+            pooled = np.max(np.lib.stride_tricks.sliding_window_view(pad, 5), axis=1)
+            keep = np.concatenate([np.sort(np.argsort(-pooled, kind="stable")[:b - W]), np.arange(E, n)])
+            assert np.array_equal(idx[1, s, h], keep), f"SnapKV n={n}"
+
+
 def test_capacity_beyond_shared_memory(torch, orc):
     # Capacities past what one CTA's shared memory could hold as keys (53,504
     # positions at 4 bytes): the selection keeps them in the workspace at any
