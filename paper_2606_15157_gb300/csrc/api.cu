@@ -60,9 +60,12 @@ bool is_scoring(int m) { return m == KVEV_SNAPKV || m == KVEV_H2O; }
 
 struct WsLayout {
   int n_units = 0, R = 0, R_pad = 0, max_items = 0, n_h2o_units = 0;
-  size_t lens = 0, abort_flag = 0, node_cnt = 0, ready = 0, chunk_start = 0, item = 0, part = 0,
+  size_t lens = 0, abort_flag = 0, group_cnt = 0, ready = 0, chunk_start = 0, item = 0, part = 0,
          lam = 0, raw = 0, lse = 0, sel_keys = 0, total = 0;
 };
+
+// 128-key tiles per scoring work item (chunk), at least.
+int min_chunk_tiles(int R_pad) { return R_pad > 128 ? kMinChunkTiles2 : kMinChunkTiles1; }
 
 // Entries of a selection key row: S_cap rounded up to whole 128-key blocks.
 int sel_key_stride(int S_cap) { return (S_cap + 127) & ~127; }
@@ -72,7 +75,7 @@ WsLayout ws_layout(const kvev_plan& p, int B, int S_cap) {
   w.n_units = static_cast<int>(p.score_layers.size()) * B * p.H_kv;
   w.R = p.G * p.W;
   w.R_pad = (w.R + 31) / 32 * 32;  // whole 32-column TMEM loads in the second sweep
-  const int chunk_min = kTileKeys * kMinChunkTiles;
+  const int chunk_min = kTileKeys * min_chunk_tiles(w.R_pad);
   w.max_items = w.n_units * ((S_cap + chunk_min - 1) / chunk_min);
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -82,15 +85,17 @@ WsLayout ws_layout(const kvev_plan& p, int B, int S_cap) {
   };
   w.lens = take(sizeof(int) * std::max(B, 1));
   w.abort_flag = take(sizeof(int));
-  w.node_cnt = take(sizeof(int) * static_cast<size_t>(std::max(w.max_items, 1)) * kTreeLevels);
+  w.group_cnt = take(sizeof(int) * static_cast<size_t>(std::max(w.max_items, 1)));
   w.ready = take(sizeof(int) * std::max(w.n_units, 1));
   w.chunk_start = take(sizeof(int) * (w.n_units + 1));
-  w.item = take(sizeof(int4) * std::max(w.max_items, 1));
-  w.part = take(sizeof(float2) * static_cast<size_t>(w.max_items) * w.R_pad);  // one per chunk
+  w.item = take(2 * sizeof(int4) * static_cast<size_t>(std::max(w.max_items, 1)));
   w.lam = take(sizeof(float) * static_cast<size_t>(w.n_units) * w.R_pad);
   w.raw = take(sizeof(float) * static_cast<size_t>(w.n_units) * S_cap);
-  // the selection's keys, one 16-byte aligned row per scoring unit
-  w.sel_keys = take(sizeof(uint32_t) * static_cast<size_t>(w.n_units) * sel_key_stride(S_cap));
+  // the selection's keys, one 16-byte aligned row per scoring unit; before the
+  // selection the same bytes hold the score kernel's records, one per chunk
+  const size_t keys = sizeof(uint32_t) * static_cast<size_t>(w.n_units) * sel_key_stride(S_cap);
+  const size_t records = sizeof(float2) * static_cast<size_t>(w.max_items) * w.R_pad;
+  w.sel_keys = w.part = take(std::max(keys, records));
   if (p.h2o_full) {  // base-2 log-sum-exp of every prompt row of every H2O unit
     for (int l : p.score_layers) w.n_h2o_units += p.route_pre[l] == KVEV_H2O ? B * p.H_kv : 0;
     w.lse = take(sizeof(float) * static_cast<size_t>(w.n_h2o_units) * p.G * S_cap);
@@ -666,12 +671,8 @@ int evict_impl(kvev_plan& P, DevCtx& D, const void* const* K, const void* const*
   const int grid = D.num_sms;
   const int tiles_max = (S_cap + kTileKeys - 1) / kTileKeys;
   // (an even number of tiles: chunks are swept in 256-key super-tiles)
-  const int chunk_tiles = (std::max(kMinChunkTiles, (tiles_max + grid - 1) / grid) + 1) & ~1;
+  const int chunk_tiles = (std::max(min_chunk_tiles(ws.R_pad), (tiles_max + grid - 1) / grid) + 1) & ~1;
   if (chunk_tiles > 0xFFFF) return KVEV_ENOTSUP;  // tiles per item are packed in 16 bits
-  // the normaliser's merge tree has kTreeLevels internal levels of fan-in kTreeFanIn
-  int leaves = 1;
-  for (int i = 0; i < kTreeLevels; ++i) leaves *= kTreeFanIn;
-  if ((tiles_max + chunk_tiles - 1) / chunk_tiles > leaves) return KVEV_ENOTSUP;
   PrologueParams pp = {};
   pp.n_units = ws.n_units;
   pp.B = B;
@@ -686,8 +687,9 @@ int evict_impl(kvev_plan& P, DevCtx& D, const void* const* K, const void* const*
   pp.lens = lens_ok;
   pp.S_cap = S_cap;
   pp.status = D.status;
-  pp.node_cnt = reinterpret_cast<int*>(wsb + ws.node_cnt);
-  pp.n_node_cnt = std::max(ws.max_items, 1) * kTreeLevels;
+  pp.H_q = P.H_q;
+  pp.group_cnt = reinterpret_cast<int*>(wsb + ws.group_cnt);
+  pp.max_items = ws.max_items;
   pp.ready = reinterpret_cast<int*>(wsb + ws.ready);
   pp.abort_flag = reinterpret_cast<int*>(wsb + ws.abort_flag);
   pp.chunk_start = reinterpret_cast<int*>(wsb + ws.chunk_start);
@@ -774,7 +776,9 @@ int evict_impl(kvev_plan& P, DevCtx& D, const void* const* K, const void* const*
     sp.lens = lens_ok;
     sp.chunk_start = pp.chunk_start;
     sp.item = pp.item;
-    sp.node_cnt = pp.node_cnt;
+    sp.group_cnt = pp.group_cnt;
+    sp.lag = ws.R_pad > 128 ? kLag2 : kLag1;
+    sp.group = ws.R_pad > 128 ? kGroup2 : kGroup1;
     sp.ready = pp.ready;
     sp.abort_flag = pp.abort_flag;
     sp.status = D.status;

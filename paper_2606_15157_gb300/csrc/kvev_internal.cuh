@@ -15,19 +15,25 @@ constexpr int kMaxLayers = 128;       // layers in one plan
 constexpr int kMaxScoreLayers = 64;   // SnapKV/H2O layers (tensor maps travel as kernel params)
 constexpr int kTileKeys = 128;        // keys per tensor-core tile (MMA M or N)
 constexpr int kSuperKeys = 256;       // keys per K stage (sweep 1 MMAs take N = 256 keys)
-// Tiles per scoring work item (chunk), at least.  Larger chunks give each CTA
-// more slack before it needs a unit's normaliser and halve the partials to
-// merge; the cost is reuse distance (grid * chunk bytes between a tile's two
-// reads, ~78 MB at 16 tiles on 152 SMs, inside the 126 MB L2).
-constexpr int kMinChunkTiles = 16;
-// The per-row (max, sum) records of a unit's chunks are merged up a tree of
-// fan-in kTreeFanIn (the last child to arrive merges its siblings), so the
-// normaliser is ready a few load round trips after the unit's last chunk.
 // What a prologue + score launch covers (PrologueParams::mode).
 constexpr int kScoreAll = 0;       // every scoring layer, rows = the observation window
 constexpr int kScoreNoH2O = 1;     // SnapKV layers only (H2O layers are scored over the whole prompt)
-constexpr int kTreeFanIn = 4;
-constexpr int kTreeLevels = 5;        // internal levels: up to 4^5 = 1024 chunks per unit
+// The score kernel's schedule, by the window rows: the least 128-key tiles per
+// work item (chunk), by how many items sweep 2 of an item runs behind its sweep
+// 1, and of how many chunks the records are merged into one before they are
+// published (when a unit has more).
+//   R_pad <= 128: the sweeps move a tile faster than HBM delivers it, so K has
+//     to be in L2 still when sweep 2 reads it again: 2 x 152 x 320 KB are
+//     between the reads.  One 8,192-token prompt, 32 SnapKV layers: 10 tiles and
+//     lag 1 140 us, 12 and 1 159, 8 and 1 171, 16 and 1 173, 10 and 2 166, 8 and
+//     2 183, 16 and 2 175 (8 tiles leave the normaliser too little time).
+//   R_pad > 128: the softmax warps are the pace and an item reloads 64 KB of Q:
+//     eight prompts of 16K-32K, 16 tiles and lag 2 3.98 ms, 16 and 1 4.06, 12
+//     and 1 4.10, 20 and 1 4.09, 12 and 2 4.25; groups of 8 4.01, of 32 4.16
+//     (the merges take issue slots from the softmax warps beside them).
+constexpr int kMaxGroup = 8;
+constexpr int kMinChunkTiles1 = 10, kLag1 = 1, kGroup1 = 8;
+constexpr int kMinChunkTiles2 = 16, kLag2 = 2, kGroup2 = 4;
 constexpr int kSoftmaxWGs = 4;        // softmax warpgroups of the score kernel
 constexpr int kRedTiles = 8;          // sweep-2 tiles whose key sums are combined at once
 constexpr int kScoreThreads = 128 * (1 + kSoftmaxWGs);  // + warpgroup 0: TMA, MMA, publisher, normaliser warps
@@ -74,14 +80,15 @@ struct PrologueParams {
   const int* lens_in; // caller's lengths
   int* lens;          // validated copy (out-of-range lengths become 0, flagged)
   int* status;
-  int* node_cnt;      // [items][kTreeLevels] arrival counters of the merge tree (zeroed here)
-  int n_node_cnt;     // counters in node_cnt (workspace capacity)
+  int* group_cnt;     // [items] arrivals at the group of chunks whose first is the item (zeroed here)
+  int max_items;      // items the workspace holds
+  int H_q;
   int W;              // observation window
   int mode;           // kScoreAll, or kScoreNoH2O (H2O layers are scored over the whole prompt)
   int* ready;
   int* abort_flag;
   int* chunk_start;   // [n_units + 1]
-  int4* item;         // [items] {unit, n, first key, tiles | chunks of the unit << 16}
+  int4* item;         // [items][2] work items (see ScoreParams)
 };
 
 struct ScoreParams {
@@ -97,14 +104,17 @@ struct ScoreParams {
   float inv_G;
   const int* lens;
   const int* chunk_start;
-  const int4* item;   // [items] {unit, n, first key, tiles | chunks of the unit << 16}
-  int* node_cnt;      // [items][kTreeLevels]: counter of the tree node whose first leaf is the item
-  int* ready;
+  const int4* item;   // [items][2] {unit, n, first key, tiles | chunks of the unit << 16},
+                      // {row of the first key in K, first query row, scoring layer, unit's first item}
+  int* group_cnt;     // [items]: arrivals at the group of chunks whose first is the item
+  int* ready;         // [n_units] records published (all of the unit's: its normaliser can be formed)
+  int group;          // chunks of a unit with more than this publish one record per `group`
+  int lag;            // sweep 2 of an item runs `lag` items after its sweep 1
   int* abort_flag;
   int* status;
-  float2* part;       // [items][R_pad] per-row (max, sum) of a chunk, or of the tree node
-                      // whose first leaf is that chunk, base-2 units
-  float* lam;         // [n_units][R_pad] per-row log2-sum-exp
+  float2* part;       // [items][R_pad] per-row (max, sum) of a chunk, or of the group whose first
+                      // chunk it is, base-2 units
+  float* lam;         // [n_units][R_pad] per-row log2-sum-exp (supplied normalisers)
   float* raw;         // [n_units][S_cap] window scores
   long long wait_ns;
   int stall_unit;

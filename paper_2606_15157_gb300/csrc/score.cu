@@ -16,17 +16,18 @@
 //   sweep 2: S^T = K Q^T on the tensor core (keys on TMEM lanes), each thread
 //            owns one key and sums exp2(s*log2e/sqrt(d) - lse2_r) over the rows.
 // Work items are chunks of chunk_keys keys (an even number of 128-key tiles,
-// swept in 256-key super-tiles).  A CTA runs sweep 1 of item j + kLag before
+// swept in 256-key super-tiles).  A CTA runs sweep 1 of item j + lag before
 // sweep 2 of item j, so the unit's normaliser, which needs every chunk of the
 // unit (some on other CTAs), is almost always published by the time sweep 2
-// needs it.  The chunk whose partials complete the unit's merge tree publishes
-// lse2 (release flag); sweep-2 readers wait on it with a time bound.  All CTAs
+// needs it.  Every chunk publishes its rows' (max, sum) and counts itself in;
+// a sweep-2 reader waits for the unit's count with a time bound and merges the
+// records itself, in chunk order (the result does not depend on the schedule).  All CTAs
 // are co-resident (cooperative launch) and a unit spans at most two rounds of
 // items, so the wait always ends.
 //
 // Roles per CTA (640 threads, five warpgroups): warp 0 issues TMA loads (one
 // thread); warp 1 owns TMEM and issues tcgen05.mma (an elected lane); warp 2
-// publishes each chunk's row partials and climbs the unit's merge tree; warp 3
+// publishes each chunk's row partials; warp 3 merges a unit's records and
 // stages -lse2 for sweep 2; warpgroups 1-4 are softmax warpgroups.  The tensor
 // core fills 256-column TMEM units (two adjacent 128-column slots) in a ring
 // of two: sweep 1 one unit per (super-tile, 128-row group), sweep 2 one unit
@@ -110,47 +111,33 @@ __device__ __forceinline__ Smem carve(uint8_t* base, const ScoreParams& p, int D
 }
 
 struct ItemInfo {
-  int u, s, h, ls, n, key0, ntiles, cs, nchunks;
+  int u, n, key0, ntiles, nchunks;
+  int krow, qrow, ls, cs;
 };
 
-// Work item t from its packed record (written by the prologue: one 16-byte load).
-__device__ __forceinline__ int4 load_item(const ScoreParams& p, int t) { return __ldg(&p.item[t]); }
-
-__device__ __forceinline__ ItemInfo decode_item(const ScoreParams& p, int t, int4 r) {
-  ItemInfo it;
-  it.u = r.x;
-  it.n = r.y;
-  it.key0 = r.z;
-  it.ntiles = r.w & 0xFFFF;
-  it.nchunks = r.w >> 16;
-  it.cs = t - it.key0 / p.chunk_keys;
-  const int per_layer = p.B * p.H_kv;
-  it.ls = it.u / per_layer;
-  const int rem = it.u - it.ls * per_layer;
-  it.s = rem / p.H_kv;
-  it.h = rem - it.s * p.H_kv;
-  return it;
+// Work item t from its packed record (written by the prologue: two 16-byte loads).
+__device__ __forceinline__ ItemInfo load_item(const ScoreParams& p, int t) {
+  const int4 a = __ldg(&p.item[2 * t]), b = __ldg(&p.item[2 * t + 1]);
+  return ItemInfo{a.x, a.y, a.z, a.w & 0xFFFF, a.w >> 16, b.x, b.y, b.z, b.w};
 }
 
-// Items a role needs at step j of the lag-1 loop: j (sweep 1) and j-1
-// (sweep 2).  At step j it pulls the record of item j+1 into L1, so the load at
-// step j+1 is an L1 hit instead of a round trip to L2 on the critical path.
+// At step j a role pulls the record of item j+1 into L1, so the load at step
+// j+1 is an L1 hit instead of a round trip to L2 on the critical path.
 __device__ __forceinline__ void prefetch_item(const ScoreParams& p, int first, int stride, int j, int J) {
-  if (j + 1 < J) asm volatile("prefetch.global.L1 [%0];" ::"l"(p.item + first + (j + 1) * stride));
+  if (j + 1 < J) asm volatile("prefetch.global.L1 [%0];" ::"l"(p.item + 2 * (first + (j + 1) * stride)));
 }
 
-// A CTA's work entries in order: at step j = 0 .. J + kLag - 1, sweep 1 of
-// item j (j < J), then sweep 2 of item j - kLag (j >= kLag).  Sweep 2 of an
-// item runs kLag sweep-1 items after its own sweep 1, so the unit's row
+// A CTA's work entries in order: at step j = 0 .. J + lag - 1, sweep 1 of
+// item j (j < J), then sweep 2 of item j - lag (j >= lag).  Sweep 2 of an
+// item runs lag sweep-1 items after its own sweep 1, so the unit's row
 // normalisers (which need every chunk of the unit, some of them on other
 // CTAs) are almost always published by then.  With the normalisers supplied
 // (single sweep), the entries are sweep 2 of items 0 .. J-1.  Every entry
 // loads its own Q (buffer e mod 2 for entry e).
-constexpr int kLag = 2;
 struct EntryIter {
-  int J, j = 0, sweep = -1;
+  int J, lag, j = 0, sweep = -1;
   bool single;
-  __device__ __forceinline__ EntryIter(int J_, bool single_) : J(J_), single(single_) {}
+  __device__ __forceinline__ EntryIter(int J_, const ScoreParams& p) : J(J_), lag(p.lag), single(p.single != 0) {}
   // Next entry: item index jj (of this CTA) and sweep; false at the end.
   __device__ __forceinline__ bool next(int& jj, int& sw) {
     if (single) {
@@ -164,8 +151,8 @@ struct EntryIter {
         sweep = 0;
         ++j;
       }
-      if (j >= J + kLag) return false;
-      jj = sweep == 0 ? j : j - kLag;
+      if (j >= J + lag) return false;
+      jj = sweep == 0 ? j : j - lag;
       if (jj >= 0 && jj < J) {
         sw = sweep;
         return true;
@@ -181,11 +168,10 @@ template <int D>
 __device__ __forceinline__ void load_q(const ScoreParams& p, const Smem& sm, uint32_t e, const ItemInfo& it) {
   const uint32_t qb = e % p.q_bufs;
   mbar_expect_tx(&sm.qfull[qb], static_cast<uint32_t>(p.R_pad) * D * 2);
-  const int qrow = (it.s * p.H_q + it.h * p.G) * p.W;
 #pragma unroll
   for (int kc = 0; kc < D / 64; ++kc)
     tma_load_2d(sm.qbuf + qb * sm.qbytes + static_cast<size_t>(kc) * p.q_rows * 128, &p.qmap[it.ls],
-                kc * 64, qrow, &sm.qfull[qb]);
+                kc * 64, it.qrow, &sm.qfull[qb]);
 }
 
 template <int D>
@@ -200,17 +186,16 @@ __device__ __forceinline__ void producer(const ScoreParams& p, const Smem& sm, i
   // Q of entry x goes into buffer x mod nq once entry x - nq has released it
   auto q_free = [&](uint32_t x) { return mbar_try_wait(&sm.qempty[x % nq], ((x / nq) & 1) ^ 1); };
   bool ok = true;
-  EntryIter ei(J, p.single != 0);
+  EntryIter ei(J, p);
   int jj, sw;
   for (uint32_t e = 0; ok && ei.next(jj, sw); ++e) {
     const int t = first + jj * stride;
     if (sw == 0) prefetch_item(p, first, stride, jj, J);
-    const ItemInfo it = decode_item(p, t, load_item(p, t));
+    const ItemInfo it = load_item(p, t);
     EntryIter la = ei;
     int jn, swn;
     const bool has_next = la.next(jn, swn);
     const CUtensorMap* kmap = &p.kmap[it.ls];
-    const int row0 = (it.s * p.H_kv + it.h) * p.S_cap + it.key0;
     const int nst = (it.ntiles + 1) / 2;  // 256-key super-tiles of the item
     // This entry's Q goes out as soon as its buffer is free, and at the
     // latest before the super-tile that fills the last stage (the K loads
@@ -225,7 +210,7 @@ __device__ __forceinline__ void producer(const ScoreParams& p, const Smem& sm, i
       }
       if (nq > 1 && has_next && q_issued == e + 1 && q_free(e + 1)) {
         const int tn = first + jn * stride;
-        load_q<D>(p, sm, e + 1, decode_item(p, tn, load_item(p, tn)));
+        load_q<D>(p, sm, e + 1, load_item(p, tn));
         ++q_issued;
       }
       const uint32_t st = pst, ph = pph;
@@ -235,7 +220,7 @@ __device__ __forceinline__ void producer(const ScoreParams& p, const Smem& sm, i
       mbar_expect_tx(&sm.kfull[st], kStageBytes);
 #pragma unroll
       for (int kc = 0; kc < D / 64; ++kc)
-        tma_load_2d_hint(dst + kc * (kSuperKeys * 128), kmap, kc * 64, row0 + i * kSuperKeys,
+        tma_load_2d_hint(dst + kc * (kSuperKeys * 128), kmap, kc * 64, it.krow + i * kSuperKeys,
                          &sm.kfull[st], sw == 0 ? keep : drop);
     }
   }
@@ -274,12 +259,12 @@ __device__ __forceinline__ void mma_issuer(const ScoreParams& p, const Smem& sm,
   uint32_t st = 0, kph = 0;  // K stage ring: position and phase of the next super-tile
   uint32_t sl = 0, tph = 0;  // TMEM ring of two 256-column units: first slot and phase
   bool ok = true;
-  EntryIter ei(J, p.single != 0);
+  EntryIter ei(J, p);
   int jj, sw;
   for (uint32_t e = 0; ok && ei.next(jj, sw); ++e) {
     const int t = first + jj * stride;
     if (sw == 0) prefetch_item(p, first, stride, jj, J);
-    const ItemInfo it = decode_item(p, t, load_item(p, t));
+    const ItemInfo it = load_item(p, t);
     const uint32_t qb = e % p.q_bufs;
     const uint64_t qdesc0 = sw128_desc(smem_u32(sm.qbuf) + qb * sm.qbytes);
     if (!wait_bar_warp(&sm.qfull[qb], (e / p.q_bufs) & 1, p)) { ok = false; break; }
@@ -394,14 +379,14 @@ __device__ __forceinline__ void softmax_wg(const ScoreParams& p, const Smem& sm,
   uint32_t q1 = 0, q2 = 0;  // sweep-1 / sweep-2 entries done
   bool ok = true;
 
-  EntryIter ei(J, p.single != 0);
+  EntryIter ei(J, p);
   int jj, sw;
   while (ei.next(jj, sw)) {
     // ---------------- sweep 1 ----------------
     if (sw == 0) {
       prefetch_item(p, first, stride, jj, J);
       const int t = first + jj * stride;
-      const ItemInfo it = decode_item(p, t, load_item(p, t));
+      const ItemInfo it = load_item(p, t);
       float m0 = -INFINITY, z0 = 0.f, m1 = -INFINITY, z1 = 0.f;
       const int tr0 = lrow < p.R ? row_pos(p, lrow, it.n) : -1;
       const int tr1 = NH == 2 && 128 + lrow < p.R ? row_pos(p, 128 + lrow, it.n) : -1;
@@ -449,7 +434,7 @@ __device__ __forceinline__ void softmax_wg(const ScoreParams& p, const Smem& sm,
     // ---------------- sweep 2 ----------------
     else {
       const int t = first + jj * stride;
-      const ItemInfo it = decode_item(p, t, load_item(p, t));
+      const ItemInfo it = load_item(p, t);
       // -lse2 of the unit, loaded ahead by the normaliser warp
       const uint32_t lb = q2 & 1;
       if (!wait_bar(&sm.lfull[lb], (q2 >> 1) & 1, p)) ok = false;
@@ -513,117 +498,94 @@ __device__ __forceinline__ void softmax_wg(const ScoreParams& p, const Smem& sm,
 
 // ---------------------------------------------------------------------------
 // Publisher warp: for each sweep-1 entry, merge the four warpgroups' (max,
-// sum) of every row into the chunk's record, then climb the unit's merge tree:
-// a node's record lives in the slot of its first leaf chunk; the last of a
-// node's (up to kTreeFanIn) children to arrive merges its siblings' records
-// into its own and carries the result one level up.  Whoever completes the
-// root turns it into the unit's lse2 and releases it.
+// sum) of every row into the chunk's record and count the chunk in.  A unit of
+// more than p.group chunks publishes groups of that many: the last chunk
+// of a group to arrive merges the group's records (in chunk order) into the
+// slot of its first chunk and counts the group in.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void publisher(const ScoreParams& p, const Smem& sm, int first, int stride, int J) {
   constexpr int kRowsPerLane = 8;  // R_pad <= 256
   const int lane = threadIdx.x & 31;
   const int nr = p.R_pad >> 5;
   uint32_t q1 = 0;
-  EntryIter ei(J, p.single != 0);
+  EntryIter ei(J, p);
   int jj, sw;
   while (ei.next(jj, sw)) {
     if (sw != 0) continue;
     const int t = first + jj * stride;
-    const ItemInfo it = decode_item(p, t, load_item(p, t));
+    const ItemInfo it = load_item(p, t);
     if (!wait_bar_warp(&sm.pfull[0], q1 & 1, p)) return;
-    float2 acc[kRowsPerLane];  // rows lane + 32 i of the current tree node
+    float2* rec = p.part + static_cast<size_t>(t) * p.R_pad;
 #pragma unroll
     for (int i = 0; i < kRowsPerLane; ++i) {
-      acc[i] = make_float2(-INFINITY, 0.f);
       if (i < nr) {
+        float2 e[kSoftmaxWGs];
 #pragma unroll
-        for (int w = 0; w < kSoftmaxWGs; ++w) acc[i] = merge_ms(acc[i], sm.pc[w * p.R_pad + lane + 32 * i]);
+        for (int w = 0; w < kSoftmaxWGs; ++w) e[w] = sm.pc[w * p.R_pad + lane + 32 * i];
+        rec[lane + 32 * i] = merge_records(make_float2(-INFINITY, 0.f), e);
       }
     }
     __syncwarp();
     mbar_arrive_elect(&sm.pempty[0]);  // pc may be overwritten
     ++q1;
-    int c = t - it.cs;         // index of the current node within its level (a leaf: the chunk)
-    int nodes = it.nchunks;    // nodes of the current level
-    int span = 1;              // leaf chunks under a node of the current level
-    int level = 0;
-    bool root = nodes == 1;
-    while (!root) {
-      float2* rec = p.part + static_cast<size_t>(it.cs + c * span) * p.R_pad;
-#pragma unroll
-      for (int i = 0; i < kRowsPerLane; ++i)
-        if (i < nr) rec[lane + 32 * i] = acc[i];
+    if (it.nchunks > p.group) {
+      const int c0 = (t - it.cs) / p.group * p.group;  // the group's first chunk
+      const int n = min(p.group, it.nchunks - c0);
       __threadfence();
       __syncwarp();
-      const int c0 = c / kTreeFanIn * kTreeFanIn;  // first sibling
-      const int nchild = min(kTreeFanIn, nodes - c0);
       int last = 0;
       if (lane == 0) {
-        int* cnt = p.node_cnt + static_cast<size_t>(it.cs + c0 * span) * kTreeLevels + level;
-        last = atomicAdd(cnt, 1) == nchild - 1;
+        last = atomicAdd(&p.group_cnt[it.cs + c0], 1) == n - 1;
         __threadfence();
       }
-      last = __shfl_sync(0xffffffffu, last, 0);
-      if (!last) break;
-      for (int k = 0; k < nchild; ++k) {
-        if (c0 + k == c) continue;
-        const float2* sib = p.part + static_cast<size_t>(it.cs + (c0 + k) * span) * p.R_pad;
+      if (!__shfl_sync(0xffffffffu, last, 0)) continue;
+      float2* g = p.part + static_cast<size_t>(it.cs + c0) * p.R_pad;
+      for (int i = 0; i < nr; ++i) {
+        float2 e[kMaxGroup];
 #pragma unroll
-        for (int h = 0; h < kRowsPerLane; h += 4) {  // four loads in flight (64 registers)
-          float2 e[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            e[i] = h + i < nr ? __ldcg(&sib[lane + 32 * (h + i)]) : make_float2(-INFINITY, 0.f);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) acc[h + i] = merge_ms(acc[h + i], e[i]);
-        }
+        for (int q = 0; q < kMaxGroup; ++q)
+          e[q] = q < n ? __ldcg(&g[static_cast<size_t>(q) * p.R_pad + lane + 32 * i]) : make_float2(-INFINITY, 0.f);
+        g[lane + 32 * i] = merge_records(make_float2(-INFINITY, 0.f), e);
       }
-      c /= kTreeFanIn;
-      nodes = (nodes + kTreeFanIn - 1) / kTreeFanIn;
-      span *= kTreeFanIn;
-      ++level;
-      root = nodes == 1;
-    }
-    if (!root) continue;
-    // The root: lse2 = M + log2(Z) per row.
-#pragma unroll
-    for (int i = 0; i < kRowsPerLane; ++i) {
-      if (i < nr)
-        p.lam[static_cast<size_t>(it.u) * p.R_pad + lane + 32 * i] =
-            (acc[i].x == -INFINITY || acc[i].y <= 0.f) ? INFINITY : acc[i].x + lg2_approx(acc[i].y);
     }
     __threadfence();
     __syncwarp();
-    if (lane == 0 && it.u != p.stall_unit) st_release(&p.ready[it.u], 1);
+    if (lane == 0 && it.u != p.stall_unit) atomicAdd(&p.ready[it.u], 1);
   }
 }
 
 // ---------------------------------------------------------------------------
-// Normaliser warp: for each sweep-2 entry, wait for the unit's lse2 (bounded)
-// and copy -lse2 into the entry's lam buffer ahead of the softmax warpgroups.
+// Normaliser warp: for each sweep-2 entry, wait (bounded) until the unit's
+// records are all published, merge them into its rows' lse2 and put -lse2 into
+// the entry's lam buffer, ahead of the softmax warpgroups.
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ float row_lse2(float2 a) {  // +inf: no key, the row counts nowhere
+  return a.x == -INFINITY || a.y <= 0.f ? INFINITY : a.x + lg2_approx(a.y);
+}
+
 __device__ __forceinline__ void lam_loader(const ScoreParams& p, const Smem& sm, int first, int stride, int J) {
   const int lane = threadIdx.x & 31;
   uint32_t q2 = 0;
-  EntryIter ei(J, p.single != 0);
+  EntryIter ei(J, p);
   int jj, sw;
   while (ei.next(jj, sw)) {
     if (sw != 1) continue;
     const int t = first + jj * stride;
-    const ItemInfo it = decode_item(p, t, load_item(p, t));
+    const ItemInfo it = load_item(p, t);
+    const int step = it.nchunks > p.group ? p.group : 1;  // chunks per record
+    const int nrec = p.single ? 1 : (it.nchunks + step - 1) / step;
     const uint32_t lb = q2 & 1;
     if (!wait_bar_warp(&sm.lempty[lb], ((q2 >> 1) & 1) ^ 1, p)) return;
-    // The whole warp polls the unit's flag; between polls it sleeps on a
+    // The whole warp polls the unit's count; between polls it sleeps on a
     // shared-memory barrier that never completes (a suspended wait, which
     // unlike a spin leaves this warp's issue port to the softmax warps that
-    // share it).  The normaliser is needed one entry later at the earliest,
-    // so a microsecond between polls costs nothing.
+    // share it).
     int ready = 0;
     const uint64_t t0 = globaltimer_ns();
     for (;;) {
       int v = 0, stop = 0;
       if (lane == 0) {
-        v = ld_acquire(&p.ready[it.u]);
+        v = ld_acquire(&p.ready[it.u]) >= nrec;
         if (!v && ld_volatile(p.abort_flag)) stop = 1;
         if (!v && !stop && globaltimer_ns() - t0 > static_cast<uint64_t>(p.wait_ns)) {
           atomicExch(p.abort_flag, 1);
@@ -633,12 +595,32 @@ __device__ __forceinline__ void lam_loader(const ScoreParams& p, const Smem& sm,
       }
       ready = __shfl_sync(0xffffffffu, v, 0);
       if (ready || __shfl_sync(0xffffffffu, stop, 0)) break;
-      mbar_try_wait_sleep(sm.nap, 0, 1000);
+      mbar_try_wait_sleep(sm.nap, 0, 300);
     }
-    __syncwarp();  // the other lanes read lse2 after lane 0's acquire
+    __syncwarp();  // the other lanes read the records after lane 0's acquire
     float* lam = sm.lam + lb * p.R_pad;
-    for (int r = lane; r < p.R_pad; r += 32)  // stored negated: exp2(s*c + (-lse2))
-      lam[r] = ready ? -__ldcg(&p.lam[static_cast<size_t>(it.u) * p.R_pad + r]) : -INFINITY;
+    if (!ready || p.single) {
+      for (int r = lane; r < p.R_pad; r += 32)  // stored negated: exp2(s*c + (-lse2))
+        lam[r] = ready ? -__ldcg(&p.lam[static_cast<size_t>(it.u) * p.R_pad + r]) : -INFINITY;
+    } else {
+      const float4* rec = reinterpret_cast<const float4*>(p.part + static_cast<size_t>(it.cs) * p.R_pad);
+      const size_t stride4 = static_cast<size_t>(step) * p.R_pad / 2;  // float4 (two rows) between records
+      for (int r = lane; r < p.R_pad / 2; r += 32) {
+        float2 a = make_float2(-INFINITY, 0.f), b = a;
+        for (int k = 0; k < nrec; k += 8) {  // eight loads in flight
+          float2 ea[8], eb[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const float4 e = k + q < nrec ? __ldcg(rec + (k + q) * stride4 + r) : make_float4(-INFINITY, 0.f, -INFINITY, 0.f);
+            ea[q] = make_float2(e.x, e.y);
+            eb[q] = make_float2(e.z, e.w);
+          }
+          a = merge_records(a, ea);
+          b = merge_records(b, eb);
+        }
+        *reinterpret_cast<float2*>(lam + 2 * r) = make_float2(-row_lse2(a), -row_lse2(b));
+      }
+    }
     __syncwarp();
     mbar_arrive_elect(&sm.lfull[lb]);
     ++q2;
@@ -781,17 +763,21 @@ __global__ void __launch_bounds__(1024) prologue_kernel(const __grid_constant__ 
     if (u >= u0 && u < u1) {
       p.chunk_start[u] = excl;
       p.ready[u] = 0;
-      if ((excl + c) * kTreeLevels > p.n_node_cnt) {  // never for a workspace of ws_layout's size
+      if (excl + c > p.max_items) {  // never for a workspace of ws_layout's size
         atomicOr(p.status, kStatusDevice);
         c = 0;
       }
+      const int ls = u / per_layer;
+      const int rem = u - ls * per_layer;          // sequence x KV head
+      const int G = p.H_q / p.H_kv;
+      const int s = rem / p.H_kv, h = rem - s * p.H_kv;
       for (int q = 0; q < c; ++q) {
         const int key0 = q * p.chunk_keys;
         const int nk = min(p.chunk_keys, n - key0);
         const int ntiles = (nk + kTileKeys - 1) / kTileKeys;
-        p.item[excl + q] = make_int4(u, n, key0, ntiles | (c << 16));
-#pragma unroll
-        for (int lv = 0; lv < kTreeLevels; ++lv) p.node_cnt[(excl + q) * kTreeLevels + lv] = 0;
+        p.item[2 * (excl + q)] = make_int4(u, n, key0, ntiles | (c << 16));
+        p.item[2 * (excl + q) + 1] = make_int4(rem * p.S_cap + key0, (s * p.H_q + h * G) * p.W, ls, excl);
+        p.group_cnt[excl + q] = 0;
       }
     }
     __syncthreads();

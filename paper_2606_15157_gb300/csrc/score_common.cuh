@@ -185,6 +185,20 @@ __device__ __forceinline__ float s2_unit_edge(float c, uint64_t* tempty, uint32_
   return sum4x2(a);
 }
 
+// N (max, sum) records of a row, and those before them (a), merged in order
+// against their common maximum.
+template <int N>
+__device__ __forceinline__ float2 merge_records(float2 a, const float2 (&e)[N]) {
+  float m = a.x;
+#pragma unroll
+  for (int i = 0; i < N; ++i) m = fmaxf(m, e[i].x);
+  const float base = m == -INFINITY ? 0.f : m;
+  float z = a.y * ex2_approx(a.x - base);
+#pragma unroll
+  for (int i = 0; i < N; ++i) z = fmaf(e[i].y, ex2_approx(e[i].x - base), z);
+  return make_float2(m, z);
+}
+
 __device__ __forceinline__ float2 merge_ms(float2 a, float2 e) {  // (max, sum) in base 2
   if (e.x == -INFINITY) return a;
   if (a.x == -INFINITY) return e;
