@@ -815,10 +815,13 @@ int evict_impl(kvev_plan& P, DevCtx& D, const void* const* K, const void* const*
     if (launch_lse_fill(lp, s) != cudaSuccess) return KVEV_ECUDA;
   }
   mark(KVEV_K_PROLOGUE, 1);
-  if (ws.n_units > 0) mark(KVEV_K_SCORE, 0);
-  if (ws.n_units > 0 &&
-      launch_score(sp, P.d, score_grid, score_smem, s) != cudaSuccess)
-    return KVEV_ECUDA;
+  // nothing to launch when every scoring layer's scores are supplied or come
+  // from the whole-prompt kernels
+  bool any_window = false;
+  for (int i = 0; i < n_slayers; ++i)
+    any_window |= !supplied(P.score_layers[i]) && !(full_prompt && P.route_pre[P.score_layers[i]] == KVEV_H2O);
+  if (any_window || full_prompt) mark(KVEV_K_SCORE, 0);
+  if (any_window && launch_score(sp, P.d, score_grid, score_smem, s) != cudaSuccess) return KVEV_ECUDA;
   if (full_prompt) {
     // row pass (lse2 of every prompt row), then key pass (the scores)
     ScoreParams fp = sp;
@@ -856,7 +859,7 @@ int evict_impl(kvev_plan& P, DevCtx& D, const void* const* K, const void* const*
         return KVEV_ECUDA;
     }
   }
-  if (ws.n_units > 0) mark(KVEV_K_SCORE, 1);
+  if (any_window || full_prompt) mark(KVEV_K_SCORE, 1);
 
   // ---- selection --------------------------------------------------------
   SelectParams sel;

@@ -561,6 +561,8 @@ template <int D, int G, bool kSplit>
 __global__ void __launch_bounds__(kDecodeThreads, kDecCtasPerSm) decode_step_kernel(const __grid_constant__ DecodeParams p) {
   extern __shared__ float lg[];
   __shared__ DecShared<kSplit> sh;
+  pdl_wait();
+  pdl_trigger();
   // the H2O / TOVA units, and eight cheap units per CTA: after the others, or,
   // split, before them (every CTA is resident at once, and those end first)
   const int n_cheap_ctas = kSplit ? static_cast<int>(gridDim.x) - p.n_att * p.cluster : 0;
@@ -598,6 +600,8 @@ __global__ void decode_advance_kernel(int32_t* lens, int B) {
 // 32 layers x 8 heads x 2,048 slots, one CTA per unit and one vector of each
 // at a time before: batch 1 169 and 83 us (6.4 TB/s), batch 16 1.32 and 1.28 ms (6.7 TB/s).
 __global__ void __launch_bounds__(kDecodeThreads) decode_init_kernel(const __grid_constant__ DecodeParams p) {
+  pdl_wait();
+  pdl_trigger();
   const int u = blockIdx.x / p.init_split, part = blockIdx.x - u * p.init_split;
   const int l = find_dec_layer(p, u);
   const DecLayer& ly = p.layer[l];
@@ -660,20 +664,8 @@ cudaError_t launch_step_dgs(const DecodeParams& p, size_t smem, cudaStream_t st)
     if (e != cudaSuccess) return e;
   }
   const int cheap = (p.n_cheap + kDecodeWarps - 1) / kDecodeWarps;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(p.n_att * p.cluster + (cheap + p.cluster - 1) / p.cluster * p.cluster);  // whole clusters
-  cfg.blockDim = dim3(kDecodeThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  if (kSplit) {
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = p.cluster;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-  }
-  return cudaLaunchKernelEx(&cfg, decode_step_kernel<D, G, kSplit>, p);
+  const int grid = p.n_att * p.cluster + (cheap + p.cluster - 1) / p.cluster * p.cluster;  // whole clusters
+  return launch_overlapped(decode_step_kernel<D, G, kSplit>, p, grid, kDecodeThreads, smem, st, p.cluster);
 }
 
 template <int D, int G>
@@ -707,8 +699,7 @@ size_t decode_logit_bytes(int cap, int rows, int cluster) {
 
 cudaError_t launch_decode_init(const DecodeParams& p, cudaStream_t st) {
   if (p.units == 0) return cudaSuccess;
-  decode_init_kernel<<<p.units * p.init_split, kDecodeThreads, 0, st>>>(p);
-  return cudaGetLastError();
+  return launch_overlapped(decode_init_kernel, p, p.units * p.init_split, kDecodeThreads, 0, st);
 }
 
 cudaError_t launch_decode_step(const DecodeParams& p, size_t smem, cudaStream_t st) {

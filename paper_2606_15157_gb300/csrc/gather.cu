@@ -34,6 +34,7 @@ __device__ __forceinline__ int find_layer(const GatherParams& p, long long g) {
 }
 
 __global__ void __launch_bounds__(kGatherThreads) gather_kernel(const __grid_constant__ GatherParams p) {
+  pdl_wait();
   const int tpr = p.d / 8;  // threads per row, 16 bytes each
   const int rows_per_block = kGatherThreads / tpr;
   const int sub = threadIdx.x % tpr;
@@ -76,8 +77,7 @@ cudaError_t launch_gather(const GatherParams& p, cudaStream_t s, int num_sms) {
   long long blocks = (p.total_rows + rows_per_block - 1) / rows_per_block;
   const long long cap = static_cast<long long>(num_sms) * 8;
   if (blocks > cap) blocks = cap;
-  gather_kernel<<<static_cast<int>(blocks), kGatherThreads, 0, s>>>(p);
-  return cudaGetLastError();
+  return launch_overlapped(gather_kernel, p, static_cast<int>(blocks), kGatherThreads, 0, s);
 }
 
 }  // namespace kvev

@@ -340,6 +340,15 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
+// ---- programmatic dependent launch ---------------------------------------------
+// A kernel launched with the programmatic attribute may start while the kernels
+// before it on the stream still run: it waits (pdl_wait) before it touches any
+// memory, so that only its launch and its parameter reads overlap them.  A
+// kernel lets its successor start as soon as all of its own CTAs have
+// (pdl_trigger), which saves most of the 2-3 us between two launches.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---- tcgen05 -----------------------------------------------------------------
 
 __device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t ncols) {
@@ -602,6 +611,30 @@ __device__ __forceinline__ uint32_t float_key(float f) {
 
 // Launchers implemented by the kernel translation units.
 namespace kvev {
+// A launch of `fn` that may overlap the end of the kernels before it on the
+// stream (fn calls pdl_wait), in clusters of `cluster` CTAs when that is not 1.
+template <class P>
+cudaError_t launch_overlapped(void (*fn)(const P), const P& p, int grid, int threads, size_t smem, cudaStream_t s,
+                              int cluster = 1) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cluster > 1) {
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
+  }
+  return cudaLaunchKernelEx(&cfg, fn, p);
+}
+
 cudaError_t launch_prologue(const PrologueParams& p, cudaStream_t s);
 cudaError_t launch_score(const ScoreParams& p, int d, int grid, size_t smem, cudaStream_t s);
 int score_smem_bytes(int d, int q_rows, int q_bufs, int R_pad, int stages);

@@ -637,6 +637,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_kernel(const __grid_co
   }
   const Smem sm = carve(smem_raw, p, D);
   const int warp = threadIdx.x >> 5;
+  pdl_trigger();
   if (threadIdx.x == 0) {
     for (int i = 0; i < p.stages; ++i) {
       mbar_init(&sm.kfull[i], 1);
@@ -703,6 +704,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_kernel(const __grid_co
 __global__ void __launch_bounds__(1024) prologue_kernel(const __grid_constant__ PrologueParams p) {
   __shared__ int warp_sums[32];
   __shared__ int carry;
+  pdl_trigger();
   const int tid = threadIdx.x;
   const int slice = (p.n_units + gridDim.x - 1) / gridDim.x;
   const int u0 = min(static_cast<int>(blockIdx.x) * slice, p.n_units);
@@ -795,6 +797,8 @@ __global__ void __launch_bounds__(1024) prologue_kernel(const __grid_constant__ 
 // sees them).  Runs after the prologue, which clears the ready flags.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) lse_fill_kernel(const __grid_constant__ LseParams p) {
+  pdl_wait();
+  pdl_trigger();
   const int u = blockIdx.x;
   const int per_layer = p.B * p.H_kv;
   const int ls = u / per_layer;
@@ -819,8 +823,7 @@ __global__ void __launch_bounds__(256) lse_fill_kernel(const __grid_constant__ L
 
 cudaError_t launch_lse_fill(const LseParams& p, cudaStream_t s) {
   if (p.n_units == 0) return cudaSuccess;
-  lse_fill_kernel<<<p.n_units, 256, 0, s>>>(p);
-  return cudaGetLastError();
+  return launch_overlapped(lse_fill_kernel, p, p.n_units, 256, 0, s);
 }
 
 int score_smem_bytes(int d, int q_rows, int q_bufs, int R_pad, int stages) {

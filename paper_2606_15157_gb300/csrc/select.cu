@@ -867,6 +867,8 @@ __device__ void copy_streaming_rows(const SelectParams& p, int l, int rem, int n
 template <int NT>
 __global__ void __launch_bounds__(NT, kSelectThreadsPerSm / NT) select_kernel(const __grid_constant__ SelectParams p) {
   __shared__ SelShared<NT> sh;
+  pdl_wait();
+  pdl_trigger();
   const int per_layer = p.B * p.H_kv;
   // dispatch order: two lists, each in (sequence rank, layer, head) order --
   // the first L_first layers of p.order (the scoring layers) and the rest --
@@ -959,12 +961,9 @@ cudaError_t launch_select(const SelectParams& p, int grid, int num_sms, cudaStre
   // shorten while the SMs have room.  One 8,192-token prompt (256 units): 18.5
   // us with 256 threads, 15.2 with 512, 28 with 1,024 (two rounds of units).
   if (grid <= num_sms)
-    select_kernel<1024><<<grid, 1024, 0, s>>>(p);
-  else if (grid <= 2 * num_sms)
-    select_kernel<512><<<grid, 512, 0, s>>>(p);
-  else
-    select_kernel<256><<<grid, 256, 0, s>>>(p);
-  return cudaGetLastError();
+    return launch_overlapped(select_kernel<1024>, p, grid, 1024, 0, s);
+  if (grid <= 2 * num_sms) return launch_overlapped(select_kernel<512>, p, grid, 512, 0, s);
+  return launch_overlapped(select_kernel<256>, p, grid, 256, 0, s);
 }
 
 }  // namespace kvev
