@@ -10,6 +10,7 @@ from __future__ import annotations
 import ctypes as C
 import os
 import threading
+from array import array
 
 import numpy as np
 
@@ -108,6 +109,30 @@ def _check(rc: int, what: str):
         raise KvevError(rc, what)
 
 
+def _ptr_array(ptrs, n: int):
+    """Per-layer pointers (ints, None = NULL) as a C array of n 64-bit words, missing ones NULL.
+    The caller keeps it until the library call returns.  (A ctypes array of 32
+    pointers takes 3 us to make, this 0.4; a decode step passes three.)"""
+    try:
+        a = array("Q", ptrs)
+    except TypeError:
+        a = array("Q", [0 if x is None else x for x in ptrs])
+    if len(a) != n:
+        if len(a) > n:
+            raise IndexError(f"{len(a)} pointers for {n} layers")
+        a.extend([0] * (n - len(a)))
+    return a
+
+
+def _addr(a):
+    return None if a is None else a.buffer_info()[0]
+
+
+def _data_ptrs(tensors):
+    """Device pointers of per-layer tensors (None = NULL)."""
+    return [0 if t is None else t.data_ptr() for t in tensors]
+
+
 # ---------------------------------------------------------------------------
 # C-named wrappers
 # ---------------------------------------------------------------------------
@@ -165,11 +190,10 @@ def kvev_plan_layer_offset(handle: int, B: int, layer: int) -> int:
 def kvev_evict_prefill(handle, K_ptrs, V_ptrs, Q_ptrs, lens_ptr, B, S_cap, out_K, out_V, out_idx,
                        out_count, h2o_state, workspace, workspace_bytes, stream) -> int:
     """Pointer-level call; returns the status code (does not raise)."""
-    Ln = len(K_ptrs)
-    arr = C.c_void_p * Ln
-    Ka, Va = arr(*K_ptrs), arr(*V_ptrs)
-    Qa = arr(*Q_ptrs) if Q_ptrs is not None else None
-    return load().kvev_evict_prefill(handle, Ka, Va, Qa, lens_ptr, B, S_cap, out_K, out_V,
+    n = len(K_ptrs)
+    Ka, Va = _ptr_array(K_ptrs, n), _ptr_array(V_ptrs, n)
+    Qa = None if Q_ptrs is None else _ptr_array(Q_ptrs, n)
+    return load().kvev_evict_prefill(handle, _addr(Ka), _addr(Va), _addr(Qa), lens_ptr, B, S_cap, out_K, out_V,
                                      out_idx, out_count, h2o_state, workspace, workspace_bytes,
                                      stream)
 
@@ -177,12 +201,11 @@ def kvev_evict_prefill(handle, K_ptrs, V_ptrs, Q_ptrs, lens_ptr, B, S_cap, out_K
 def kvev_evict_prefill_scored(handle, K_ptrs, V_ptrs, Q_ptrs, score_ptrs, lens_ptr, B, S_cap, out_K, out_V,
                               out_idx, out_count, h2o_state, workspace, workspace_bytes, stream) -> int:
     """Pointer-level call with caller-supplied scores; returns the status code."""
-    Ln = len(K_ptrs)
-    arr = C.c_void_p * Ln
-    Ka, Va = arr(*K_ptrs), arr(*V_ptrs)
-    Sa = arr(*score_ptrs) if score_ptrs is not None else None
-    Qa = arr(*Q_ptrs) if Q_ptrs is not None else None
-    return load().kvev_evict_prefill_scored(handle, Ka, Va, Qa, Sa, lens_ptr, B, S_cap, out_K, out_V,
+    n = len(K_ptrs)
+    Ka, Va = _ptr_array(K_ptrs, n), _ptr_array(V_ptrs, n)
+    Sa = None if score_ptrs is None else _ptr_array(score_ptrs, n)
+    Qa = None if Q_ptrs is None else _ptr_array(Q_ptrs, n)
+    return load().kvev_evict_prefill_scored(handle, _addr(Ka), _addr(Va), _addr(Qa), _addr(Sa), lens_ptr, B, S_cap, out_K, out_V,
                                             out_idx, out_count, h2o_state, workspace, workspace_bytes,
                                             stream)
 
@@ -190,12 +213,11 @@ def kvev_evict_prefill_scored(handle, K_ptrs, V_ptrs, Q_ptrs, score_ptrs, lens_p
 def kvev_evict_prefill_lse(handle, K_ptrs, V_ptrs, Q_ptrs, lse_ptrs, lens_ptr, B, S_cap, out_K, out_V,
                            out_idx, out_count, h2o_state, workspace, workspace_bytes, stream) -> int:
     """Pointer-level call with the caller's window-row log-sum-exp; returns the status code."""
-    Ln = len(K_ptrs)
-    arr = C.c_void_p * Ln
-    Ka, Va = arr(*K_ptrs), arr(*V_ptrs)
-    La = arr(*lse_ptrs) if lse_ptrs is not None else None
-    Qa = arr(*Q_ptrs) if Q_ptrs is not None else None
-    return load().kvev_evict_prefill_lse(handle, Ka, Va, Qa, La, lens_ptr, B, S_cap, out_K, out_V,
+    n = len(K_ptrs)
+    Ka, Va = _ptr_array(K_ptrs, n), _ptr_array(V_ptrs, n)
+    La = None if lse_ptrs is None else _ptr_array(lse_ptrs, n)
+    Qa = None if Q_ptrs is None else _ptr_array(Q_ptrs, n)
+    return load().kvev_evict_prefill_lse(handle, _addr(Ka), _addr(Va), _addr(Qa), _addr(La), lens_ptr, B, S_cap, out_K, out_V,
                                          out_idx, out_count, h2o_state, workspace, workspace_bytes,
                                          stream)
 
@@ -207,10 +229,10 @@ def kvev_evict_prefill_noalloc(handle, K_ptrs, V_ptrs, Q_ptrs, lens_ptr, B, S_ca
                                out_idx, out_count, h2o_state, device_status, stream) -> int:
     """Pointer-level call of the entry point that allocates nothing (its scratch is
     a fixed library-owned device array); returns the status code."""
-    arr = C.c_void_p * len(K_ptrs)
-    Ka, Va = arr(*K_ptrs), arr(*V_ptrs)
-    Qa = arr(*Q_ptrs) if Q_ptrs is not None else None
-    return load().kvev_evict_prefill_noalloc(handle, Ka, Va, Qa, lens_ptr, B, S_cap, out_K, out_V,
+    n = len(K_ptrs)
+    Ka, Va = _ptr_array(K_ptrs, n), _ptr_array(V_ptrs, n)
+    Qa = None if Q_ptrs is None else _ptr_array(Q_ptrs, n)
+    return load().kvev_evict_prefill_noalloc(handle, _addr(Ka), _addr(Va), _addr(Qa), lens_ptr, B, S_cap, out_K, out_V,
                                              out_idx, out_count, h2o_state, device_status, stream)
 
 
@@ -244,17 +266,19 @@ def kvev_decode_init(handle, B, growth, pre_K, pre_V, pre_idx, pre_count, h2o_st
 
 def kvev_decode_step(handle, B, growth, dec_K, dec_V, dec_state, k_ptrs, v_ptrs, q_ptrs,
                      stream) -> int:
-    arr = C.c_void_p * len(k_ptrs)
-    return load().kvev_decode_step(handle, B, growth, dec_K, dec_V, dec_state, arr(*k_ptrs),
-                                   arr(*v_ptrs), arr(*q_ptrs), stream)
+    n = len(k_ptrs)
+    ka, va, qa = _ptr_array(k_ptrs, n), _ptr_array(v_ptrs, n), _ptr_array(q_ptrs, n)
+    return load().kvev_decode_step(handle, B, growth, dec_K, dec_V, dec_state, _addr(ka), _addr(va),
+                                   _addr(qa), stream)
 
 
 def kvev_decode_step_attn(handle, B, growth, dec_K, dec_V, dec_state, k_ptrs, v_ptrs, attn_ptrs,
                           stream) -> int:
     """Pointer-level call; returns the status code (does not raise)."""
-    arr = C.c_void_p * len(k_ptrs)
-    return load().kvev_decode_step_attn(handle, B, growth, dec_K, dec_V, dec_state, arr(*k_ptrs),
-                                        arr(*v_ptrs), arr(*attn_ptrs), stream)
+    n = len(k_ptrs)
+    ka, va, aa = _ptr_array(k_ptrs, n), _ptr_array(v_ptrs, n), _ptr_array(attn_ptrs, n)
+    return load().kvev_decode_step_attn(handle, B, growth, dec_K, dec_V, dec_state, _addr(ka), _addr(va),
+                                        _addr(aa), stream)
 
 
 def kvev_status(handle: int) -> int:
@@ -443,11 +467,10 @@ class Plan:
         import torch
         if stream is None:
             stream = torch.cuda.current_stream()
-        ptr = lambda t: None if t is None else t.data_ptr()
         if lse is not None:
             rc = kvev_evict_prefill_lse(
-                self.handle, [ptr(k) for k in K], [ptr(v) for v in V],
-                [ptr(q) for q in Q] if Q is not None else None, [ptr(x) for x in lse], lens.data_ptr(),
+                self.handle, _data_ptrs(K), _data_ptrs(V),
+                _data_ptrs(Q) if Q is not None else None, _data_ptrs(lse), lens.data_ptr(),
                 B, S_cap, bufs["out_K"].data_ptr(), bufs["out_V"].data_ptr(), bufs["out_idx"].data_ptr(),
                 bufs["out_count"].data_ptr(), bufs["h2o_state"].data_ptr(), bufs["workspace"].data_ptr(),
                 bufs["workspace"].numel(), stream.cuda_stream)
@@ -456,8 +479,8 @@ class Plan:
             return rc
         if scores is not None:
             rc = kvev_evict_prefill_scored(
-                self.handle, [ptr(k) for k in K], [ptr(v) for v in V],
-                [ptr(q) for q in Q] if Q is not None else None, [ptr(x) for x in scores], lens.data_ptr(),
+                self.handle, _data_ptrs(K), _data_ptrs(V),
+                _data_ptrs(Q) if Q is not None else None, _data_ptrs(scores), lens.data_ptr(),
                 B, S_cap, bufs["out_K"].data_ptr(), bufs["out_V"].data_ptr(), bufs["out_idx"].data_ptr(),
                 bufs["out_count"].data_ptr(), bufs["h2o_state"].data_ptr(), bufs["workspace"].data_ptr(),
                 bufs["workspace"].numel(), stream.cuda_stream)
@@ -465,8 +488,8 @@ class Plan:
                 _check(rc, "kvev_evict_prefill_scored")
             return rc
         rc = kvev_evict_prefill(
-            self.handle, [ptr(k) for k in K], [ptr(v) for v in V],
-            [ptr(q) for q in Q] if Q is not None else None, lens.data_ptr(), B, S_cap,
+            self.handle, _data_ptrs(K), _data_ptrs(V),
+            _data_ptrs(Q) if Q is not None else None, lens.data_ptr(), B, S_cap,
             bufs["out_K"].data_ptr(), bufs["out_V"].data_ptr(), bufs["out_idx"].data_ptr(),
             bufs["out_count"].data_ptr(), bufs["h2o_state"].data_ptr(),
             bufs["workspace"].data_ptr(), bufs["workspace"].numel(), stream.cuda_stream)
@@ -540,10 +563,9 @@ class DecodeArena:
         import torch
         if stream is None:
             stream = torch.cuda.current_stream()
-        ptr = lambda t: None if t is None else t.data_ptr()
         _check(kvev_decode_step_attn(self.plan.handle, self.B, self.growth, self.K.data_ptr(),
-                                     self.V.data_ptr(), self.state.data_ptr(), [ptr(t) for t in k_new],
-                                     [ptr(t) for t in v_new], [ptr(t) for t in attn],
+                                     self.V.data_ptr(), self.state.data_ptr(), _data_ptrs(k_new),
+                                     _data_ptrs(v_new), _data_ptrs(attn),
                                      stream.cuda_stream), "kvev_decode_step_attn")
 
     def step(self, k_new, v_new, q_new, stream=None):
@@ -551,8 +573,7 @@ class DecodeArena:
         import torch
         if stream is None:
             stream = torch.cuda.current_stream()
-        ptr = lambda t: None if t is None else t.data_ptr()
         _check(kvev_decode_step(self.plan.handle, self.B, self.growth, self.K.data_ptr(),
-                                self.V.data_ptr(), self.state.data_ptr(), [ptr(t) for t in k_new],
-                                [ptr(t) for t in v_new], [ptr(t) for t in q_new],
+                                self.V.data_ptr(), self.state.data_ptr(), _data_ptrs(k_new),
+                                _data_ptrs(v_new), _data_ptrs(q_new),
                                 stream.cuda_stream), "kvev_decode_step")
