@@ -496,12 +496,18 @@ __device__ __forceinline__ void softmax_wg(const ScoreParams& p, const Smem& sm,
   }
 }
 
+__device__ __forceinline__ float row_lse2(float2 a) {  // +inf: no key, the row counts nowhere
+  return a.x == -INFINITY || a.y <= 0.f ? INFINITY : a.x + lg2_approx(a.y);
+}
+
 // ---------------------------------------------------------------------------
 // Publisher warp: for each sweep-1 entry, merge the four warpgroups' (max,
 // sum) of every row into the chunk's record and count the chunk in.  A unit of
 // more than p.group chunks publishes groups of that many: the last chunk
 // of a group to arrive merges the group's records (in chunk order) into the
-// slot of its first chunk and counts the group in.
+// slot of its first chunk and counts the group in.  A unit of one chunk goes
+// straight into the lam buffer of its sweep-2 entry: no other CTA needs it,
+// and the way through memory is 3 us of a short prompt's call.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void publisher(const ScoreParams& p, const Smem& sm, int first, int stride, int J) {
   constexpr int kRowsPerLane = 8;  // R_pad <= 256
@@ -515,19 +521,33 @@ __device__ __forceinline__ void publisher(const ScoreParams& p, const Smem& sm, 
     const int t = first + jj * stride;
     const ItemInfo it = load_item(p, t);
     if (!wait_bar_warp(&sm.pfull[0], q1 & 1, p)) return;
-    float2* rec = p.part + static_cast<size_t>(t) * p.R_pad;
+    float2 acc[kRowsPerLane];
 #pragma unroll
     for (int i = 0; i < kRowsPerLane; ++i) {
       if (i < nr) {
         float2 e[kSoftmaxWGs];
 #pragma unroll
         for (int w = 0; w < kSoftmaxWGs; ++w) e[w] = sm.pc[w * p.R_pad + lane + 32 * i];
-        rec[lane + 32 * i] = merge_records(make_float2(-INFINITY, 0.f), e);
+        acc[i] = merge_records(make_float2(-INFINITY, 0.f), e);
       }
     }
     __syncwarp();
     mbar_arrive_elect(&sm.pempty[0]);  // pc may be overwritten
     ++q1;
+    if (it.nchunks == 1) {
+      const uint32_t lb = jj & 1;  // the item's sweep-2 entry is this CTA's jj-th
+      if (!wait_bar_warp(&sm.lempty[lb], ((jj >> 1) & 1) ^ 1, p)) return;
+#pragma unroll
+      for (int i = 0; i < kRowsPerLane; ++i)
+        if (i < nr) sm.lam[lb * p.R_pad + lane + 32 * i] = -row_lse2(acc[i]);
+      __syncwarp();
+      if (it.u != p.stall_unit) mbar_arrive_elect(&sm.lfull[lb]);
+      continue;
+    }
+    float2* rec = p.part + static_cast<size_t>(t) * p.R_pad;
+#pragma unroll
+    for (int i = 0; i < kRowsPerLane; ++i)
+      if (i < nr) rec[lane + 32 * i] = acc[i];
     if (it.nchunks > p.group) {
       const int c0 = (t - it.cs) / p.group * p.group;  // the group's first chunk
       const int n = min(p.group, it.nchunks - c0);
@@ -559,10 +579,6 @@ __device__ __forceinline__ void publisher(const ScoreParams& p, const Smem& sm, 
 // records are all published, merge them into its rows' lse2 and put -lse2 into
 // the entry's lam buffer, ahead of the softmax warpgroups.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float row_lse2(float2 a) {  // +inf: no key, the row counts nowhere
-  return a.x == -INFINITY || a.y <= 0.f ? INFINITY : a.x + lg2_approx(a.y);
-}
-
 __device__ __forceinline__ void lam_loader(const ScoreParams& p, const Smem& sm, int first, int stride, int J) {
   const int lane = threadIdx.x & 31;
   uint32_t q2 = 0;
@@ -572,6 +588,10 @@ __device__ __forceinline__ void lam_loader(const ScoreParams& p, const Smem& sm,
     if (sw != 1) continue;
     const int t = first + jj * stride;
     const ItemInfo it = load_item(p, t);
+    if (it.nchunks == 1 && !p.single) {  // the publisher warp's
+      ++q2;
+      continue;
+    }
     const int step = it.nchunks > p.group ? p.group : 1;  // chunks per record
     const int nrec = p.single ? 1 : (it.nchunks + step - 1) / step;
     const uint32_t lb = q2 & 1;
