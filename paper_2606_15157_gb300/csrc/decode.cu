@@ -15,9 +15,9 @@
 // One CTA per H2O / TOVA unit, or a cluster of up to eight when there are few
 // units (each CTA takes a run of 16-slot tiles; the softmax normalisers and the
 // eviction candidates cross the cluster through distributed shared memory),
-// and one warp per StreamingLLM or append-only unit (eight per CTA).  H2O / TOVA: the G query rows of the new token attend to
-// every retained slot and to the new token, p_j = (1/G) sum_g softmax_j(q_g .
-// k_j / sqrt(d)); acc += p (H2O) or acc = p (TOVA).  When the unit already
+// and one warp per StreamingLLM or append-only unit (eight per CTA).  H2O /
+// TOVA: the G query rows of the new token attend to every retained slot and to
+// the new token, p_j = (1/G) sum_g softmax_j(q_g . k_j / sqrt(d)); acc += p (H2O) or acc = p (TOVA).  When the unit already
 // holds b slots, the slot with the smallest acc among positions older than
 // the protected recent window (r = h2o_recent for H2O, 0 for TOVA) is
 // evicted, ties to the higher position, and the new token takes its place
@@ -31,7 +31,6 @@ namespace kvev {
 namespace {
 
 constexpr int kDecodeThreads = 256;
-
 
 // Unit index -> layer: the last layer whose first unit is <= u (layers
 // without slots own no units and share their unit_off with the next layer).
@@ -305,6 +304,8 @@ __device__ void attend_unit(const DecodeParams& p, const DecLayer& ly, const Uni
 #pragma unroll
     for (int g = 0; g < G; ++g) {
       mg[g] = over_warps<true>(sh.wmax[g]);
+      // another CTA may hold a finite logit: -inf here then weighs 0, not NaN
+      if (kSplit && mg[g] == -INFINITY) mg[g] = 0.f;
       z[g] = 0.f;
     }
     for (int j = threadIdx.x; j < m; j += blockDim.x) {  // each thread keeps its own exponentials

@@ -21,9 +21,9 @@
 // unit (some on other CTAs), is almost always published by the time sweep 2
 // needs it.  Every chunk publishes its rows' (max, sum) and counts itself in;
 // a sweep-2 reader waits for the unit's count with a time bound and merges the
-// records itself, in chunk order (the result does not depend on the schedule).  All CTAs
-// are co-resident (cooperative launch) and a unit spans at most two rounds of
-// items, so the wait always ends.
+// records itself, in chunk order (the result does not depend on the schedule).
+// All CTAs are co-resident (cooperative launch) and a unit spans at most two
+// rounds of items, so the wait always ends.
 //
 // Roles per CTA (640 threads, five warpgroups): warp 0 issues TMA loads (one
 // thread); warp 1 owns TMEM and issues tcgen05.mma (an elected lane); warp 2
@@ -31,9 +31,9 @@
 // stages -lse2 for sweep 2; warpgroups 1-4 are softmax warpgroups.  The tensor
 // core fills 256-column TMEM units (two adjacent 128-column slots) in a ring
 // of two: sweep 1 one unit per (super-tile, 128-row group), sweep 2 one unit
-// per 128-key tile, or per two tiles when the rows fit 128 columns.  All four softmax warpgroups consume every unit, 64
-// columns each, copying them with one tcgen05.ld and releasing the unit
-// before any arithmetic.  setmaxnreg moves registers from warpgroup 0 to the
+// per 128-key tile, or per two tiles when the rows fit 128 columns.  All four
+// softmax warpgroups consume every unit, 64 columns each, copying them with
+// one tcgen05.ld and releasing the unit before any arithmetic.  setmaxnreg moves registers from warpgroup 0 to the
 // softmax warpgroups.
 #include "score_common.cuh"
 
@@ -718,7 +718,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_kernel(const __grid_co
 // Each CTA takes a contiguous slice of the units: it scans the chunk counts
 // of every unit up to the end of its slice (a few block-wide scans; the
 // counts are cheap to recompute) and writes its units' start offsets, work
-// items and cleared merge-tree counters, so that the writes are spread over
+// items and cleared record counters, so that the writes are spread over
 // the grid instead of queued behind one SM.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(1024) prologue_kernel(const __grid_constant__ PrologueParams p) {

@@ -186,16 +186,17 @@ __device__ __forceinline__ float s2_unit_edge(float c, uint64_t* tempty, uint32_
 }
 
 // N (max, sum) records of a row, and those before them (a), merged in order
-// against their common maximum.
+// against their common maximum.  A record without a maximum counts for
+// nothing, whatever its sum (NaN, where every logit was).
 template <int N>
 __device__ __forceinline__ float2 merge_records(float2 a, const float2 (&e)[N]) {
   float m = a.x;
 #pragma unroll
   for (int i = 0; i < N; ++i) m = fmaxf(m, e[i].x);
   const float base = m == -INFINITY ? 0.f : m;
-  float z = a.y * ex2_approx(a.x - base);
+  float z = (a.x == -INFINITY ? 0.f : a.y) * ex2_approx(a.x - base);
 #pragma unroll
-  for (int i = 0; i < N; ++i) z = fmaf(e[i].y, ex2_approx(e[i].x - base), z);
+  for (int i = 0; i < N; ++i) z = fmaf(e[i].x == -INFINITY ? 0.f : e[i].y, ex2_approx(e[i].x - base), z);
   return make_float2(m, z);
 }
 

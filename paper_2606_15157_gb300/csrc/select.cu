@@ -32,11 +32,11 @@
 // supplied scores 79 and 65 us, eight of 16K-32K 175 and 142 us.  Keys are an
 // order-preserving uint32 image of the fp32 (pooled) scores.  The unit's row
 // of a workspace array holds, between the two passes, each key's 16-bit bin
-// (in position order: a thread stores four at a time and loads eight, and a
+// (in position order: a thread stores and loads eight at a time, and a
 // warp scan of the lanes' counts ranks them by position); it stays in L2:
-//   0. keys sampled at even strides (eight per thread) give the bins: their range, widened
-//      by half on either side, split into 8192 bins of 2^s keys (a unit's
-//      scores may crowd into a few per cent of one octave, or spread over
+//   0. keys sampled at even strides give the bins: their range, widened by
+//      half on either side, split into 8192 bins of 2^s keys (a unit's scores
+//      may crowd into a few per cent of one octave, or spread over
 //      many octaves: the range adapts the bins to either);
 //   1. build the keys, store their bins and histogram them (the two end bins
 //      also take every key outside the range);

@@ -234,6 +234,29 @@ def test_decode_split_units(env, H_q, H_kv, d, budgets):
     assert plan.status() == kvev.OK
 
 
+def test_decode_split_infinite_logits(env):
+    # Every slot of some of a unit's CTAs has the logit -inf: they weigh nothing,
+    # and the others' softmax stands (one H2O unit over eight CTAs of nine tiles).
+    torch, kvev, orc = env
+    n = 1900
+    wl = gen.Workload(name="split_inf", L=1, H_q=2, H_kv=1, d=64, B=1, lens=np.array([n], np.int32), S_cap=n, W=8,
+                      pool_kernel=5, pool_type=gen.POOL_AVG, route=np.array([gen.H2O], np.int32),
+                      budget=np.array([1040], np.int32), sink=4, seed=11, sink_tokens=4, sink_scale=4.0,
+                      route_decode=np.array([gen.H2O], np.int32), decode_steps=1)
+    plan, bufs, arena = prefill_and_arena(torch, kvev, wl, 0)
+    arena.K.view(-1, wl.d)[0:300, 0] = float("-inf")
+    g = Arena(torch, arena, wl)
+    state = oracle_state(orc, wl, wl.route_decode, g, 0)
+    toks, k, v, q = step_tokens(wl, 0, range(1))
+    q[0][..., 0] = 1.0
+    arena.step(k, v, q)
+    orc.decode_step([state], *host_tokens(torch, toks, wl, [0], g), wl.d, wl.G)
+    g.refresh(torch)
+    assert np.isfinite(g.unit(0)["acc"]).all()
+    compare_unit(state, g.unit(0), "-inf logits")
+    assert plan.status() == kvev.OK
+
+
 def _bf16_to_f64(u16):
     return (np.asarray(u16, np.uint32) << 16).view(np.float32).astype(np.float64)
 
