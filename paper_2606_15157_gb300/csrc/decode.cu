@@ -558,21 +558,53 @@ __device__ void step_cheap_warp(const DecodeParams& p, int i, int D) {
   place_new_warp(p, r, D, bs < c ? bs : -1, n, 0.f, c, bp);
 }
 
+// What a unit (`rem` of its layer) reads of the caller's tensors, on its way to
+// L2 before the wait for the step before: thread t of n.  The new token's rows
+// are read at the end of the step's chain of round trips, and from HBM when the
+// caller wrote them some time ago.  Measured with 32 steps' tokens laid out
+// beforehand, 2,048 slots: batch 1 13.4 and 13.0 us a step, batch 16 91.6 and
+// 90.6; 512 slots with the attention supplied, batch 8: 8.2 and 7.5.
+__device__ __forceinline__ void prefetch_l2(const void* base, size_t bytes, size_t at) {
+  if (at < bytes) asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const char*>(base) + at));
+}
+template <int D, int G>
+__device__ __forceinline__ void prefetch_token(const DecLayer& ly, int rem, bool attends, int t, int n) {
+  constexpr size_t kRow = D * sizeof(uint16_t);
+  const size_t at = 128 * static_cast<size_t>(t);
+  prefetch_l2(static_cast<const char*>(ly.k_new) + rem * kRow, kRow, at);
+  prefetch_l2(static_cast<const char*>(ly.v_new) + rem * kRow, kRow, at);
+  if (!attends) return;
+  if (ly.attn == nullptr) {
+    prefetch_l2(static_cast<const char*>(ly.q_new) + rem * (G * kRow), G * kRow, at);
+  } else {
+    const size_t row = sizeof(float) * (static_cast<size_t>(ly.cap) + 1);
+    for (size_t a = at; a < row; a += 128 * static_cast<size_t>(n))
+      prefetch_l2(reinterpret_cast<const char*>(ly.attn) + rem * row, row, a);
+  }
+}
+
 template <int D, int G, bool kSplit>
 __global__ void __launch_bounds__(kDecodeThreads, kDecCtasPerSm) decode_step_kernel(const __grid_constant__ DecodeParams p) {
   extern __shared__ float lg[];
   __shared__ DecShared<kSplit> sh;
-  pdl_wait();
-  pdl_trigger();
   // the H2O / TOVA units, and eight cheap units per CTA: after the others, or,
   // split, before them (every CTA is resident at once, and those end first)
   const int n_cheap_ctas = kSplit ? static_cast<int>(gridDim.x) - p.n_att * p.cluster : 0;
   const int n_att_ctas = kSplit ? 0 : p.n_att;
   const int b = static_cast<int>(blockIdx.x);
+  const int per_layer = p.B * p.H_kv;
   if (kSplit ? b >= n_cheap_ctas : b < n_att_ctas) {
-    step_attend<D, G, kSplit>(p, kSplit ? (b - n_cheap_ctas) / p.cluster : b, lg, sh);
+    const int a = kSplit ? (b - n_cheap_ctas) / p.cluster : b;
+    prefetch_token<D, G>(p.layer[p.att_layer[a / per_layer]], a % per_layer, true, threadIdx.x, kDecodeThreads);
+    pdl_wait();
+    pdl_trigger();
+    step_attend<D, G, kSplit>(p, a, lg, sh);
   } else {
     const int i = (b - n_att_ctas) * kDecodeWarps + (threadIdx.x >> 5);
+    if (i < p.n_cheap)
+      prefetch_token<D, G>(p.layer[p.cheap_layer[i / per_layer]], i % per_layer, false, threadIdx.x & 31, 32);
+    pdl_wait();
+    pdl_trigger();
     if (i < p.n_cheap) step_cheap_warp(p, i, D);
   }
   // The last CTA of the step to finish advances every sequence by one token:
