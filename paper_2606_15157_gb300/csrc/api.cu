@@ -1044,8 +1044,8 @@ int dec_att_cap(const kvev_plan& P, const DecLayout& d) {
 // attention supplied: a unit is then a few loads per thread, and the cluster's
 // barriers cost what the split gains (batch 1: 6.4 against 5.8 us at 512
 // slots).  Measured per step, 32 layers of which 7 are H2O with 2,048 slots, 8
-// KV heads, one CTA per unit and split: batch 1 24.5 and 13.7 us (eight CTAs),
-// batch 2 26.4 and 19.3 (four), batch 4 31.6 and 29.0 (two).
+// KV heads, one CTA per unit and split: batch 1 24.5 and 13.0 us (eight CTAs),
+// batch 2 26.4 and 18.5 (four), batch 4 31.6 and 28.5 (two).
 int dec_cluster(int n_att, int cap, int num_sms) {
   int c = kMaxDecCluster;
   while (c > 1 && (static_cast<int64_t>(n_att) * c > 3 * static_cast<int64_t>(num_sms) || cap < 16 * 8 * c)) c >>= 1;
