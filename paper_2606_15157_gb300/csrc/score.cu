@@ -588,14 +588,19 @@ __device__ __forceinline__ void lam_loader(const ScoreParams& p, const Smem& sm,
     if (sw != 1) continue;
     const int t = first + jj * stride;
     const ItemInfo it = load_item(p, t);
+    // Every entry's wait, also where the publisher warp fills the buffer: a
+    // parity tells two phases apart only for a warp that is at most one behind.
+    // (Without it, a lag of two and the pattern short, short, short, short,
+    // long would let this warp overwrite the third unit's rows while the
+    // softmax warps still read them.)
+    const uint32_t lb = q2 & 1;
+    if (!wait_bar_warp(&sm.lempty[lb], ((q2 >> 1) & 1) ^ 1, p)) return;
     if (it.nchunks == 1 && !p.single) {  // the publisher warp's
       ++q2;
       continue;
     }
     const int step = it.nchunks > p.group ? p.group : 1;  // chunks per record
     const int nrec = p.single ? 1 : (it.nchunks + step - 1) / step;
-    const uint32_t lb = q2 & 1;
-    if (!wait_bar_warp(&sm.lempty[lb], ((q2 >> 1) & 1) ^ 1, p)) return;
     // The whole warp polls the unit's count; between polls it sleeps on a
     // shared-memory barrier that never completes (a suspended wait, which
     // unlike a spin leaves this warp's issue port to the softmax warps that

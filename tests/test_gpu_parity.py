@@ -291,6 +291,44 @@ def test_score_tile_edges(torch, orc, H_q, H_kv, W, d):
     parity.check_workload(wl, device_workload(wl), wl.lens)
 
 
+@pytest.mark.parametrize("H_q,W,lens", [
+    (8, 64, [1100 + 63 * i for i in range(15)] + [6000]),                 # 15 prompts of one chunk, one of three
+    (8, 64, [6100, 1500, 2048, 1400, 2049, 1300, 900, 700, 1200, 4097]),  # one or two between longer ones
+    (4, 32, [300 + 65 * i for i in range(15)] + [6000])])                 # 128 rows: chunks of ten tiles
+def test_scores_of_short_and_long_prompts_together(torch, H_q, W, lens):
+    # Prompts of one chunk and of several in one launch, ten work items per CTA and
+    # more: the normalisers of the first kind stay in the CTA, the others' come
+    # through memory, and both pass through the same two buffers.  Every
+    # sequence's scores are, bit for bit, those of a call of its own (one item
+    # per CTA at most), every time.
+    from paper_2606_15157_gb300 import kvev
+    H_kv, d, S_cap, B = 4, 64, 6144, len(lens)
+    L = 1 + 2500 // (H_kv * sum((n + 1279) // 1280 for n in lens))
+    route = [gen.H2O if l % 2 else gen.SNAPKV for l in range(L)]
+    plan = kvev.Plan(L, H_q, H_kv, d, route, [W + 60] * L, W, 5, gen.POOL_AVG)
+    torch.manual_seed(5)
+    K = torch.randn((B, H_kv, S_cap, d), dtype=torch.bfloat16, device="cuda")
+    Q = [torch.randn((B, H_q, W, d), dtype=torch.bfloat16, device="cuda") for _ in range(L)]
+    n_dev = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    bufs = plan.buffers(B, S_cap)
+
+    def scores(bufs, B, s, n):
+        return [plan.scores(bufs, B, S_cap, l)[s, :, :n].clone() for l in range(L)]
+
+    alone = []
+    for i in range(B):
+        one = plan.buffers(1, S_cap)
+        plan.evict_prefill([K[i:i + 1]] * L, [K[i:i + 1]] * L, [q[i:i + 1].contiguous() for q in Q], n_dev[i:i + 1], 1,
+                           S_cap, one)
+        alone.append(scores(one, 1, 0, lens[i]))
+    for _ in range(10):
+        plan.evict_prefill([K] * L, [K] * L, Q, n_dev, B, S_cap, bufs)
+        for i in range(B):
+            for l, x in enumerate(scores(bufs, B, i, lens[i])):
+                assert torch.equal(x, alone[i][l]), f"sequence {i} (n={lens[i]}), layer {l}"
+    assert plan.status() == kvev.OK
+
+
 def test_h2o_recent_override_and_ties(torch, orc):
     # h2o_recent = 0 (pure heavy hitters) and = b (pure recency); plus all-zero
     # queries so every score in a row ties and the lower-position rule decides.
