@@ -25,8 +25,12 @@ struct DevCtx {
   int device = -1;
   int num_sms = 0;
   int smem_optin = 0;
-  // dynamic shared memory each compiled variant was last set to
-  size_t score_smem_set[kScoreVariants] = {}, h2o_full_smem_set[2] = {};
+  // whether the compiled variants' dynamic shared memory limits were raised.  A
+  // limit belongs to the kernel, which every plan and thread of the device
+  // shares, so it is only ever set to one value per variant: what a call needs
+  // varies (with the window rows), and another plan's smaller need must not
+  // lower it.
+  bool score_smem_set[kScoreVariants] = {}, h2o_full_smem_set[2] = {};
   int* status = nullptr;
 };
 
@@ -168,8 +172,8 @@ int query_device(DevCtx& c, int dev) {
     return KVEV_ECUDA;
   if (major < 10) return KVEV_ENOTSUP;
   c.device = dev;
-  for (size_t& b : c.score_smem_set) b = 0;
-  for (size_t& b : c.h2o_full_smem_set) b = 0;
+  for (bool& b : c.score_smem_set) b = false;
+  for (bool& b : c.h2o_full_smem_set) b = false;
   return KVEV_OK;
 }
 
@@ -753,10 +757,10 @@ int evict_impl(kvev_plan& P, DevCtx& D, const void* const* K, const void* const*
     // resident per SM: its TMEM allocation then never waits on another CTA.
     const size_t smem = std::max<size_t>(score_smem_bytes(P.d, q_rows, q_bufs, ws.R_pad, stages),
                                          static_cast<size_t>(D.smem_optin) / 2 + 1024);
-    size_t& smem_set = D.score_smem_set[score_variant(P.d, ws.R_pad)];
-    if (smem_set != smem) {
-      if (score_set_smem(P.d, ws.R_pad, smem) != cudaSuccess) return KVEV_ECUDA;
-      smem_set = smem;
+    bool& smem_set = D.score_smem_set[score_variant(P.d, ws.R_pad)];
+    if (!smem_set) {  // all a block may have: the kernel uses no static shared memory
+      if (score_set_smem(P.d, ws.R_pad, D.smem_optin) != cudaSuccess) return KVEV_ECUDA;
+      smem_set = true;
     }
     sp.n_units = ws.n_units;
     sp.B = B;
@@ -843,10 +847,10 @@ int evict_impl(kvev_plan& P, DevCtx& D, const void* const* K, const void* const*
     const size_t fsmem = std::max<size_t>(static_cast<size_t>(h2o_full_smem_bytes(P.d)),
                                           static_cast<size_t>(D.smem_optin) / 2 + 1024);
     if (fsmem + 1024 > static_cast<size_t>(D.smem_optin)) return KVEV_ENOTSUP;
-    size_t& fsmem_set = D.h2o_full_smem_set[P.d == 64 ? 0 : 1];
-    if (fsmem_set != fsmem) {
+    bool& fsmem_set = D.h2o_full_smem_set[P.d == 64 ? 0 : 1];
+    if (!fsmem_set) {  // fsmem follows from d alone
       if (h2o_full_set_smem(P.d, fsmem) != cudaSuccess) return KVEV_ECUDA;
-      fsmem_set = fsmem;
+      fsmem_set = true;
     }
     if (lse_win) {  // the caller's every-row normalisers replace the row pass
       for (int j = 0; j < fp.n_h2o; ++j) fp.lse_src[j] = lse_win[P.score_layers[fp.h2o_slot[j]]];
@@ -1192,7 +1196,7 @@ int decode_step_impl(kvev_plan* plan, int B, int growth, void* dec_K, void* dec_
   dp.status = P.ctx.status;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   P.last_stream = s;
-  return launch_decode_step(dp, smem, s) == cudaSuccess ? KVEV_OK : KVEV_ECUDA;
+  return launch_decode_step(dp, smem, P.ctx.smem_optin, s) == cudaSuccess ? KVEV_OK : KVEV_ECUDA;
 }
 
 }  // namespace

@@ -689,11 +689,14 @@ __global__ void __launch_bounds__(kDecodeThreads) decode_init_kernel(const __gri
 }
 
 template <int D, int G, bool kSplit>
-cudaError_t launch_step_dgs(const DecodeParams& p, size_t smem, cudaStream_t st) {
+cudaError_t launch_step_dgs(const DecodeParams& p, size_t smem, int smem_optin, cudaStream_t st) {
   if (smem > 48 * 1024) {
+    // one value for every call (all a block may have beside the static part):
+    // the limit is the kernel's, and other plans and threads launch it too
+    constexpr int kStatic = sizeof(DecShared<kSplit>) <= 1024 ? 1024 : 2048;
+    static_assert(sizeof(DecShared<kSplit>) <= kStatic, "the limit leaves room for the static part");
     const cudaError_t e = cudaFuncSetAttribute(decode_step_kernel<D, G, kSplit>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               static_cast<int>(smem));
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin - kStatic);
     if (e != cudaSuccess) return e;
   }
   const int cheap = (p.n_cheap + kDecodeWarps - 1) / kDecodeWarps;
@@ -702,17 +705,17 @@ cudaError_t launch_step_dgs(const DecodeParams& p, size_t smem, cudaStream_t st)
 }
 
 template <int D, int G>
-cudaError_t launch_step_dg(const DecodeParams& p, size_t smem, cudaStream_t st) {
-  return p.cluster > 1 ? launch_step_dgs<D, G, true>(p, smem, st) : launch_step_dgs<D, G, false>(p, smem, st);
+cudaError_t launch_step_dg(const DecodeParams& p, size_t smem, int smem_optin, cudaStream_t st) {
+  return p.cluster > 1 ? launch_step_dgs<D, G, true>(p, smem, smem_optin, st) : launch_step_dgs<D, G, false>(p, smem, smem_optin, st);
 }
 
 template <int D>
-cudaError_t launch_step_d(const DecodeParams& p, size_t smem, cudaStream_t st) {
+cudaError_t launch_step_d(const DecodeParams& p, size_t smem, int smem_optin, cudaStream_t st) {
   switch (p.G) {
-    case 1: return launch_step_dg<D, 1>(p, smem, st);
-    case 2: return launch_step_dg<D, 2>(p, smem, st);
-    case 4: return launch_step_dg<D, 4>(p, smem, st);
-    case 8: return launch_step_dg<D, 8>(p, smem, st);
+    case 1: return launch_step_dg<D, 1>(p, smem, smem_optin, st);
+    case 2: return launch_step_dg<D, 2>(p, smem, smem_optin, st);
+    case 4: return launch_step_dg<D, 4>(p, smem, smem_optin, st);
+    case 8: return launch_step_dg<D, 8>(p, smem, smem_optin, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -735,9 +738,9 @@ cudaError_t launch_decode_init(const DecodeParams& p, cudaStream_t st) {
   return launch_overlapped(decode_init_kernel, p, p.units * p.init_split, kDecodeThreads, 0, st);
 }
 
-cudaError_t launch_decode_step(const DecodeParams& p, size_t smem, cudaStream_t st) {
+cudaError_t launch_decode_step(const DecodeParams& p, size_t smem, int smem_optin, cudaStream_t st) {
   if (p.units > 0)  // the step kernel advances lens itself
-    return p.d == 64 ? launch_step_d<64>(p, smem, st) : launch_step_d<128>(p, smem, st);
+    return p.d == 64 ? launch_step_d<64>(p, smem, smem_optin, st) : launch_step_d<128>(p, smem, smem_optin, st);
   decode_advance_kernel<<<1, 256, 0, st>>>(p.lens, p.B);
   return cudaGetLastError();
 }

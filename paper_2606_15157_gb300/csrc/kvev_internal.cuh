@@ -607,7 +607,7 @@ int score_smem_bytes(int d, int q_rows, int q_bufs, int R_pad, int stages);
 bool decode_supported(int d, int G);
 cudaError_t launch_decode_init(const DecodeParams& p, cudaStream_t s);
 size_t decode_logit_bytes(int cap, int rows, int cluster);
-cudaError_t launch_decode_step(const DecodeParams& p, size_t smem, cudaStream_t s);
+cudaError_t launch_decode_step(const DecodeParams& p, size_t smem, int smem_optin, cudaStream_t s);
 int score_kernel_regs(int d, int R_pad);
 cudaError_t score_set_smem(int d, int R_pad, size_t smem);
 int h2o_full_smem_bytes(int d);

@@ -329,6 +329,35 @@ def test_scores_of_short_and_long_prompts_together(torch, H_q, W, lens):
     assert plan.status() == kvev.OK
 
 
+@pytest.mark.parametrize("d", [64, 128])
+def test_plans_of_other_windows_in_turn(torch, d):
+    # One compiled kernel, shared memory by the window rows: a plan of fewer rows,
+    # used in between, leaves the larger plan's calls as they were, through the
+    # workspace entry and the one without allocation.
+    from paper_2606_15157_gb300 import kvev
+    n = 700
+    torch.manual_seed(3)
+    K = torch.randn((1, 1, n, d), dtype=torch.bfloat16, device="cuda")
+    lens = torch.tensor([n], dtype=torch.int32, device="cuda")
+    runs = []
+    for W in (32, 8, 64, 40):  # 128 and 32 rows of one variant, 256 and 160 of the other
+        plan = kvev.Plan(1, 4, 1, d, [kvev.SNAPKV], [W + 20], W, 5, kvev.POOL_AVG)
+        runs.append((plan, plan.buffers(1, n), torch.randn((1, 4, W, d), dtype=torch.bfloat16, device="cuda")))
+    first = {}
+    for i in (0, 1, 0, 2, 3, 2, 1, 0):
+        plan, b, Q = runs[i]
+        plan.evict_prefill([K], [K], [Q], lens, 1, n, b)
+        got = b["out_idx"].clone()
+        status = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+        assert kvev.kvev_evict_prefill_noalloc(
+            plan.handle, [K.data_ptr()], [K.data_ptr()], [Q.data_ptr()], lens.data_ptr(), 1, n, b["out_K"].data_ptr(),
+            b["out_V"].data_ptr(), b["out_idx"].data_ptr(), b["out_count"].data_ptr(), b["h2o_state"].data_ptr(),
+            status.data_ptr(), torch.cuda.current_stream().cuda_stream) == kvev.OK
+        assert int(status.item()) == 0 and plan.status() == kvev.OK
+        assert torch.equal(b["out_idx"], got)
+        assert torch.equal(first.setdefault(i, got), got)
+
+
 def test_h2o_recent_override_and_ties(torch, orc):
     # h2o_recent = 0 (pure heavy hitters) and = b (pure recency); plus all-zero
     # queries so every score in a row ties and the lower-position rule decides.
