@@ -293,3 +293,19 @@ def test_binding_argtypes_match_header(kv):
             want = _kind(decl)
             # size_t and int64_t are both 64-bit on the supported (LP64) hosts
             assert got == want or {got, want} == {"i64", "size"}, (name, decl, a)
+
+
+@pytest.mark.parametrize("make", [
+    lambda: [3, 4], lambda: (3, None), lambda: [C.c_void_p(5), C.c_void_p()], lambda: [None, C.c_void_p(7)],
+    lambda: [-1, (1 << 64) + 9], lambda: (x for x in [3, 4]), lambda: (x for x in [None, 7]), lambda: iter([C.c_void_p(5)]),
+    lambda: [3], lambda: [], lambda: [3, 4, 5], lambda: [1.5, 2], lambda: "ab", lambda: b"ab", lambda: None])
+def test_pointer_lists_convert_as_ctypes_does(kv, make):
+    # the pointer-level functions take what an array of void pointers takes, and refuse what it refuses
+    def words(f):
+        try:
+            a = f()
+        except Exception as e:
+            return type(e)
+        return list((C.c_uint64 * 2).from_address(kv._addr(a)))
+    assert words(lambda: kv._ptr_array(make(), 2)) == words(lambda: (C.c_void_p * 2)(*make()))
+    assert kv._addr(None) is None
