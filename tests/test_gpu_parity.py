@@ -418,6 +418,48 @@ def test_select_score_levels(torch, B, levels):
             assert np.array_equal(idx[1, s, h], keep), f"SnapKV n={n}"
 
 
+def _select_supplied(torch, raw, lens, b, W, pool, pool_type, S_cap):
+    """Kept positions of an H2O layer (no protected tail) and a SnapKV layer with supplied scores raw
+    [2][B][H][S_cap], one array [B][H][b] each."""
+    from paper_2606_15157_gb300 import kvev
+    _, B, H, _ = raw.shape
+    plan = kvev.Plan(2, H, H, 64, [gen.H2O, gen.SNAPKV], [b, b], W, pool, pool_type, h2o_recent=0)
+    bufs = plan.buffers(B, S_cap)
+    kv = torch.zeros((B, H, S_cap, 64), dtype=torch.bfloat16, device="cuda")
+    scores = [torch.from_numpy(raw[l]).cuda() for l in range(2)]
+    plan.evict_prefill([kv, kv], [kv, kv], None, torch.from_numpy(lens).cuda(), B, S_cap, bufs, scores=scores)
+    torch.cuda.synchronize()
+    assert plan.status() == kvev.OK
+    return bufs["out_idx"].cpu().numpy()[: 2 * B * H * b].reshape(2, B, H, b)
+
+
+def _top(x, k):
+    """The k largest of x, equal ones by position, in position order."""
+    return np.sort(np.argsort(-x, kind="stable")[:k])
+
+
+@pytest.mark.parametrize("S_cap", [1032, 1031])  # aligned score rows, and rows read one score at a time
+@pytest.mark.parametrize("pool,pool_type", [(1, gen.POOL_AVG), (1, gen.POOL_MAX), (5, gen.POOL_AVG), (11, gen.POOL_AVG),
+                                            (11, gen.POOL_MAX), (33, gen.POOL_AVG), (257, gen.POOL_MAX)])
+def test_select_wide_pooling(torch, S_cap, pool, pool_type):
+    # Pooling widths without vector loads, eight keys per thread, down to rows
+    # shorter than the window; the averages' sums in position order, in fp32.
+    rng = np.random.default_rng(pool)
+    b, W = 40, 8
+    lens = np.array([1031, 1030, 1024, 520, 264, 129, 57, 49, 41], np.int32)
+    raw = rng.random((2, len(lens), 2, S_cap)).astype(np.float32) ** 4
+    idx = _select_supplied(torch, raw, lens, b, W, pool, pool_type, S_cap)
+    is_max = pool_type == gen.POOL_MAX
+    for s, n in enumerate(lens):
+        for h in range(2):
+            E = n - W
+            pad = np.pad(raw[1, s, h, :E], pool // 2, constant_values=-np.inf if is_max else 0)
+            pooled = pad[:E].copy()
+            for j in range(1, pool):
+                pooled = np.maximum(pooled, pad[j:j + E]) if is_max else pooled + pad[j:j + E]
+            assert np.array_equal(idx[1, s, h], np.concatenate([_top(pooled, b - W), np.arange(E, n)])), f"n={n}"
+
+
 def test_capacity_beyond_shared_memory(torch, orc):
     # Capacities past what one CTA's shared memory could hold as keys (53,504
     # positions at 4 bytes): the selection keeps them in the workspace at any
