@@ -69,27 +69,27 @@ constexpr int kSegKeys = 128;              // a key block: four keys per lane
 constexpr int kBinBlock = 256;             // a bin block: eight positions per lane
 constexpr int kAhead = 2;                  // bin blocks in flight per warp
 
-// NT: threads of a selection CTA.
-template <int NT>
+// The candidates: each warp's list is a run of entries from wB of the warp.
 struct CandLists {
-  static constexpr int kSW = NT / 32, kPerWarp = kCandidates / kSW;
-  uint32_t pos[kSW][kPerWarp];
-  uint32_t key[kSW][kPerWarp];
-  int sure[kSW][kPerWarp];  // sure positions of the segment before the candidate
+  uint32_t pos[kCandidates];
+  uint32_t key[kCandidates];
+  int sure[kCandidates];  // sure positions of the segment before the candidate
 };
 
+// NT: threads of a selection CTA.
 template <int NT>
 struct __align__(16) SelShared {
   static constexpr int kSW = NT / 32;        // warps
-  static constexpr int kCandPerWarp = CandLists<NT>::kPerWarp;
+  static constexpr int kCandPerWarp = kCandidates / kSW;
   union {
     int hist[kBins0];
-    CandLists<NT> c;
+    CandLists c;
   } u;
   int hist1[kBins1];
   int wsum[kSW];
   int wS[kSW];    // per warp segment: sure positions staged
   int wC[kSW];    // per warp segment: candidates
+  int wB[kSW];    // per warp segment: first entry of its candidate list
   int wgt[kSW];   // per warp segment: keys above T (general path) / candidates above T
   int weq[kSW];   // per warp segment: keys (candidates) equal to T
   int bcast[2];
@@ -99,7 +99,7 @@ struct __align__(16) SelShared {
 };
 
 static_assert(sizeof(SelShared<1024>) <= 48 * 1024, "the selection's shared memory is static");
-static_assert(sizeof(CandLists<1024>) <= sizeof(int) * kBins0, "the candidate lists reuse the histogram");
+static_assert(sizeof(CandLists) <= sizeof(int) * kBins0, "the candidate lists reuse the histogram");
 
 // Adds each valid lane's digit to the histogram, one shared-memory atomic per
 // distinct digit of the warp (for digits that crowd into few bins).  Every
@@ -432,8 +432,7 @@ __device__ __forceinline__ uint32_t half_bits(uint32_t t, int j) {
 }
 
 template <int NT>
-__device__ void classify_pass(uint16_t* bins, int E, uint32_t d, SelShared<NT>& sh) {
-  constexpr int kCandPerWarp = SelShared<NT>::kCandPerWarp;
+__device__ void classify_pass(uint16_t* bins, int E, uint32_t d, int first, int room, SelShared<NT>& sh) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int seg = seg_len<NT>(E);
   const int lo = min(warp * seg, E), hi = min(lo + seg, E);
@@ -477,9 +476,9 @@ __device__ void classify_pass(uint16_t* bins, int E, uint32_t d, SelShared<NT>& 
       bins[lo + j] = static_cast<uint16_t>(p0 - lo + __ffs(m) - 1);
     for (uint32_t m = cm; m != 0; m &= m - 1, ++jc) {
       const int u = __ffs(m) - 1;
-      if (jc < kCandPerWarp) {
-        sh.u.c.pos[warp][jc] = static_cast<uint32_t>(p0 + u);
-        sh.u.c.sure[warp][jc] = js + __popc(sm & ((1u << u) - 1u));
+      if (jc < room) {
+        sh.u.c.pos[first + jc] = static_cast<uint32_t>(p0 + u);
+        sh.u.c.sure[first + jc] = js + __popc(sm & ((1u << u) - 1u));
       }
     }
     ns += total & 0xFFFF;
@@ -488,17 +487,34 @@ __device__ void classify_pass(uint16_t* bins, int E, uint32_t d, SelShared<NT>& 
   if (lane == 0) {
     sh.wS[warp] = ns;
     sh.wC[warp] = nc;
-    if (nc > kCandPerWarp) sh.overflow = 1;
+    sh.wB[warp] = first;
+    if (nc > room) sh.overflow = 1;
   }
+}
+
+// How many bins of the warp's segment are d: what its candidate list has to hold.
+template <int NT>
+__device__ int count_candidates(const uint16_t* bins, int E, uint32_t d) {
+  const int lane = threadIdx.x & 31, seg = seg_len<NT>(E);
+  const int lo = min(static_cast<int>(threadIdx.x >> 5) * seg, E), hi = min(lo + seg, E);
+  int n = 0;
+  for (int b0 = lo; b0 < hi; b0 += kBinBlock) {
+    const uint4 v = ld_block_bins(bins, b0);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const uint32_t w = pick(v, u >> 1);
+      n += b0 + 8 * lane + u < hi && ((u & 1) ? w >> 16 : w & 0xFFFFu) == d;
+    }
+  }
+  return warp_sum(n);
 }
 
 // The keys of each warp's listed candidates, from the scores.
 template <int NT>
 __device__ void candidate_keys(const Scalar& sk, SelShared<NT>& sh) {
-  constexpr int kCandPerWarp = SelShared<NT>::kCandPerWarp;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nc = min(sh.wC[warp], kCandPerWarp);
-  for (int i = lane; i < nc; i += 32) sh.u.c.key[warp][i] = sk.one(static_cast<int>(sh.u.c.pos[warp][i]));
+  const int nc = sh.wC[warp], first = sh.wB[warp];
+  for (int i = lane; i < nc; i += 32) sh.u.c.key[first + i] = sk.one(static_cast<int>(sh.u.c.pos[first + i]));
 }
 
 // Steps 3 and 4 for at most 32 candidates (the sampled bins leave a handful as
@@ -522,8 +538,8 @@ __device__ void finish_few(const Scalar& sk, const uint16_t* bins, int E, int kk
   uint32_t pos = 0;
   int sure = 0;
   if (lane < nc) {
-    pos = sh.u.c.pos[warp][lane];
-    sure = sh.u.c.sure[warp][lane];
+    pos = sh.u.c.pos[sh.wB[warp] + lane];
+    sure = sh.u.c.sure[sh.wB[warp] + lane];
     sh.few[first + lane] = sk.one(static_cast<int>(pos));
   }
   __syncthreads();
@@ -554,17 +570,18 @@ __device__ void finish_few(const Scalar& sk, const uint16_t* bins, int E, int kk
 // candidate key); then each warp counts its candidates above and equal to T.
 template <int NT>
 __device__ void select_candidates(int kk, SelShared<NT>& sh, uint32_t& T, int& need) {
-  constexpr int kSW = SelShared<NT>::kSW, kCandPerWarp = SelShared<NT>::kCandPerWarp;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
     sh.rlo = 0xFFFFFFFFu;
     sh.rhi = 0u;
   }
   __syncthreads();
+  const uint32_t* keys = sh.u.c.key + sh.wB[warp];
+  const int nc = sh.wC[warp];
   uint32_t lo = 0xFFFFFFFFu, hi = 0u;
-  for (int i = lane; i < sh.wC[warp]; i += 32) {
-    lo = min(lo, sh.u.c.key[warp][i]);
-    hi = max(hi, sh.u.c.key[warp][i]);
+  for (int i = lane; i < nc; i += 32) {
+    lo = min(lo, keys[i]);
+    hi = max(hi, keys[i]);
   }
   lo = __reduce_min_sync(0xffffffffu, lo);
   hi = __reduce_max_sync(0xffffffffu, hi);
@@ -581,12 +598,9 @@ __device__ void select_candidates(int kk, SelShared<NT>& sh, uint32_t& T, int& n
     const uint32_t dm = (1u << nb) - 1u;
     for (int i = threadIdx.x; i < kBins1; i += NT) sh.hist1[i] = 0;
     __syncthreads();
-    for (int c = threadIdx.x; c < kSW * kCandPerWarp; c += NT) {
-      const int w = c / kCandPerWarp, i = c - w * kCandPerWarp;
-      if (i < sh.wC[w]) {
-        const uint32_t v = sh.u.c.key[w][i] - clo;
-        if ((v & mask) == prefix) atomicAdd(&sh.hist1[(v >> shift) & dm], 1);
-      }
+    for (int i = lane; i < nc; i += 32) {
+      const uint32_t v = keys[i] - clo;
+      if ((v & mask) == prefix) atomicAdd(&sh.hist1[(v >> shift) & dm], 1);
     }
     __syncthreads();
     int digit, above;
@@ -599,8 +613,8 @@ __device__ void select_candidates(int kk, SelShared<NT>& sh, uint32_t& T, int& n
   T = clo + prefix;
   need = kk;
   int gt = 0, eq = 0;
-  for (int i = lane; i < sh.wC[warp]; i += 32) {
-    const uint32_t key = sh.u.c.key[warp][i];
+  for (int i = lane; i < nc; i += 32) {
+    const uint32_t key = keys[i];
     gt += key > T;
     eq += key == T;
   }
@@ -627,16 +641,16 @@ __device__ void merge_write(const uint16_t* bins, int E, int k, int need, SelSha
     base += sh.wS[w] + sh.wgt[w] + min(max(need - eq_base, 0), sh.weq[w]);
     eq_base += sh.weq[w];
   }
-  const int nc = sh.wC[warp];
-  int* sure = sh.u.c.sure[warp];
+  const int nc = sh.wC[warp], first = sh.wB[warp];
+  int* sure = sh.u.c.sure + first;
   int nk = 0;  // kept candidates so far; their sure counts are compacted into sure[0 .. nk)
   for (int i0 = 0; i0 < nc; i0 += 32) {
     const int i = i0 + lane;
     uint32_t key = 0, pos = 0;
     int sb = 0;
     if (i < nc) {
-      key = sh.u.c.key[warp][i];
-      pos = sh.u.c.pos[warp][i];
+      key = sh.u.c.key[first + i];
+      pos = sh.u.c.pos[first + i];
       sb = sure[i];
     }
     const bool e = i < nc && key == T;
@@ -792,7 +806,22 @@ __device__ void select_unit(const Gen& gen, const Scalar& sk, uint32_t* row, int
   // the end bins also hold keys outside the sampled range: not one prefix
   bool fast = d > 0 && d < kBins0 - 1 && nd <= kCandidates && seg_len<NT>(E) <= 65536;
   if (fast) {
-    classify_pass(bins, E, static_cast<uint32_t>(d), sh);
+    constexpr int kCandPerWarp = SelShared<NT>::kCandPerWarp;
+    const int warp = threadIdx.x >> 5;
+    int first = warp * kCandPerWarp, room = kCandPerWarp;
+    if (NT > 256 && nd > kCandPerWarp) {
+      // The more warps, the shorter an equal share of the list (160 or 80
+      // entries; 320 for 256 threads), and crowded scores lie in few segments:
+      // the shares are counted out first.  200 equal scores in a run, 256 units
+      // of 8,192: the call 29.0 us, with equal shares (the general path) 37.6; with
+      // 256 threads their 320 entries hold them, 29.2.
+      room = count_candidates<NT>(bins, E, static_cast<uint32_t>(d));
+      if ((threadIdx.x & 31) == 0) sh.wC[warp] = room;
+      __syncthreads();
+      const int lane = threadIdx.x & 31;
+      first = warp_sum(lane < warp ? sh.wC[lane] : 0);
+    }
+    classify_pass(bins, E, static_cast<uint32_t>(d), first, room, sh);
     __syncthreads();
     fast = !sh.overflow;
     if (nd <= kFewCandidates) return finish_few(sk, bins, E, k - above, k, nd, sh, out);

@@ -438,6 +438,29 @@ def _top(x, k):
     return np.sort(np.argsort(-x, kind="stable")[:k])
 
 
+@pytest.mark.parametrize("B", [1, 60, 110])  # 1,024, 512 and 256 threads per unit
+@pytest.mark.parametrize("run", [79, 81, 161, 320, 900, 2559, 2561])
+def test_select_crowded_run(torch, B, run):
+    # `run` equal scores side by side around the threshold, so that the candidates
+    # lie in few warps' segments: lists of an equal share each, counted-out lists,
+    # and more than the lists hold (the general path).
+    rng = np.random.default_rng(run + B)
+    S_cap, b, W = 4352, 230, 8
+    lens = np.array(([4352] if B == 1 else [4352, 4099, 3001 + run // 2, 2950] * 30)[:B], np.int32)
+    raw = rng.random((2, B, 2, S_cap)).astype(np.float32) * np.float32(0.5)
+    raw[..., 201:201 + run] = 0.75
+    for u in raw.reshape(-1, S_cap):
+        u[rng.choice(200, 60, replace=False)] = 0.9
+    idx = _select_supplied(torch, raw, lens, b, W, 3, gen.POOL_MAX, S_cap)
+    for s, n in enumerate(lens):
+        for h in range(2):
+            assert np.array_equal(idx[0, s, h], _top(raw[0, s, h, :n], b)), f"H2O n={n}"
+            E = n - W
+            pad = np.pad(raw[1, s, h, :E], 1, constant_values=-np.inf)
+            pooled = np.maximum(np.maximum(pad[:-2], pad[1:-1]), pad[2:])
+            assert np.array_equal(idx[1, s, h], np.concatenate([_top(pooled, b - W), np.arange(E, n)])), f"SnapKV n={n}"
+
+
 @pytest.mark.parametrize("S_cap", [1032, 1031])  # aligned score rows, and rows read one score at a time
 @pytest.mark.parametrize("pool,pool_type", [(1, gen.POOL_AVG), (1, gen.POOL_MAX), (5, gen.POOL_AVG), (11, gen.POOL_AVG),
                                             (11, gen.POOL_MAX), (33, gen.POOL_AVG), (257, gen.POOL_MAX)])
