@@ -317,7 +317,12 @@ __device__ __forceinline__ bool f_wait(const ScoreParams& p, const FSmem& sm, ui
   return ok && wait_bar(&sm.tfull[g & (kSlots - 1)], (g / kSlots) & 1, p);
 }
 
-template <int kPhase>
+// kPart (phase 1): the rows end inside the last 64 of the 256 (G does not
+// divide 256).  In a kernel of its own: in the same one the extra unit cost
+// groups of 1 and 8 heads 1.5 %.  Every block of those rows in s2_unit_edge,
+// and now: seven layers of four groups of 3, 5, 6 and 7 heads, one prompt of
+// 3,000 tokens, the call 368, 541, 640 and 730 us, and 337, 487, 574 and 651.
+template <int kPhase, bool kPart>
 __device__ __forceinline__ void f_softmax(const ScoreParams& p, const FSmem& sm, uint32_t tmem_base, int wg) {
   const int warp = threadIdx.x >> 5;
   const int quarter = warp & 3;
@@ -382,9 +387,10 @@ __device__ __forceinline__ void f_softmax(const ScoreParams& p, const FSmem& sm,
       const int qb0 = key0 / p.Pb;
       const int r0 = 64 * wg;          // this warpgroup's rows of the block
       const int exist = p.R - r0, place0 = r0 % p.Pb;
-      // blocks [c0, c1) have no causal cut for this key super-tile and only rows that exist
-      const int c0 = (key0 + kSuperKeys - 1 + p.Pb - 1) / p.Pb - qb0;
-      const int c1 = exist >= 64 ? f.n / p.Pb - qb0 : 0;
+      // blocks [c0, cn) have no causal cut for this key super-tile and are whole
+      const int c0 = (key0 + kSuperKeys - 1 + p.Pb - 1) / p.Pb - qb0, cn = f.n / p.Pb - qb0;
+      const int c1 = exist >= 64 ? cn : 0;   // [c0, c1): and every row exists
+      const int c2 = kPart && exist >= 32 ? cn : 0;  // [c0, c2): and the first 32
       float sum0 = 0.f, sum1 = 0.f;    // the thread's key of either half
       for (int j = 0; j < ns; ++j) {
         const uint32_t lb = lq & 1;
@@ -405,8 +411,10 @@ __device__ __forceinline__ void f_softmax(const ScoreParams& p, const FSmem& sm,
           for (int hh = 0; hh < halves; ++hh) {
             ok = f_wait(p, sm, g, ok);
             // the row at place i sits at q0 + i: it exists below n and sees the keys up to there
-            const float e = s2_unit_edge(c, sm.tempty, taddr, g, nl, 64, exist, place0, p.Pb,
-                                         key0 + kTileKeys * hh + lrow - q0, f.n - q0);
+            const float e = kPart && j >= c0 && j < c2
+                                ? s2_unit_part(c, sm.tempty, taddr, g, nl, exist)
+                                : s2_unit_edge(c, sm.tempty, taddr, g, nl, 64, exist, place0, p.Pb,
+                                               key0 + kTileKeys * hh + lrow - q0, f.n - q0);
             if (hh == 0) sum0 += e; else sum1 += e;
             g += 2;
           }
@@ -430,7 +438,7 @@ __device__ __forceinline__ void f_softmax(const ScoreParams& p, const FSmem& sm,
   }
 }
 
-template <int D, int kPhase>
+template <int D, int kPhase, bool kPart>
 __global__ void __launch_bounds__(kScoreThreads, 1) h2o_full_kernel(const __grid_constant__ ScoreParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   if (smem_u32(smem_raw) & 1023u) {  // the 128-byte swizzle needs 1024-byte aligned buffers
@@ -474,7 +482,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) h2o_full_kernel(const __grid
     if (warp == 2 && kPhase == 1) f_lam(p, sm);
   } else {
     regs_alloc<kRegsSoftmax>();
-    f_softmax<kPhase>(p, sm, tmem_base, (warp - 4) >> 2);
+    f_softmax<kPhase, kPart>(p, sm, tmem_base, (warp - 4) >> 2);
   }
   tc_fence_before();
   __syncthreads();
@@ -520,23 +528,29 @@ int h2o_full_smem_bytes(int d) {
 
 namespace {
 using FullFn = void (*)(const ScoreParams);
-FullFn full_fn(int d, int phase) {
-  if (d == 64) return phase == 0 ? h2o_full_kernel<64, 0> : h2o_full_kernel<64, 1>;
-  return phase == 0 ? h2o_full_kernel<128, 0> : h2o_full_kernel<128, 1>;
+// The pass (0: rows, 1: keys; 2: keys of blocks of fewer than 256 rows) for head size d.
+FullFn full_fn(int d, int pass) {
+  if (pass == 0) return d == 64 ? h2o_full_kernel<64, 0, false> : h2o_full_kernel<128, 0, false>;
+  if (pass == 1) return d == 64 ? h2o_full_kernel<64, 1, false> : h2o_full_kernel<128, 1, false>;
+  return d == 64 ? h2o_full_kernel<64, 1, true> : h2o_full_kernel<128, 1, true>;
 }
+constexpr int kFullFns = 3;
 }  // namespace
 
-// The smaller of the two passes' register counts.
+// The smallest of the passes' register counts.
 int h2o_full_kernel_regs(int d) {
-  cudaFuncAttributes a = {}, b = {};
-  if (cudaFuncGetAttributes(&a, full_fn(d, 0)) != cudaSuccess || cudaFuncGetAttributes(&b, full_fn(d, 1)) != cudaSuccess)
-    return -1;
-  return a.numRegs < b.numRegs ? a.numRegs : b.numRegs;
+  int regs = 1 << 30;
+  for (int pass = 0; pass < kFullFns; ++pass) {
+    cudaFuncAttributes a = {};
+    if (cudaFuncGetAttributes(&a, full_fn(d, pass)) != cudaSuccess) return -1;
+    regs = a.numRegs < regs ? a.numRegs : regs;
+  }
+  return regs;
 }
 
 cudaError_t h2o_full_set_smem(int d, size_t smem) {
-  for (int phase = 0; phase < 2; ++phase) {
-    const cudaError_t e = cudaFuncSetAttribute(full_fn(d, phase), cudaFuncAttributeMaxDynamicSharedMemorySize,
+  for (int pass = 0; pass < kFullFns; ++pass) {
+    const cudaError_t e = cudaFuncSetAttribute(full_fn(d, pass), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                static_cast<int>(smem));
     if (e != cudaSuccess) return e;
   }
@@ -553,7 +567,7 @@ cudaError_t launch_lse_rows_fill(const ScoreParams& p, cudaStream_t s) {
 
 cudaError_t launch_h2o_full(const ScoreParams& p, int d, int grid, size_t smem, cudaStream_t s) {
   if (grid <= 0) return cudaSuccess;
-  full_fn(d, p.phase)<<<grid, kScoreThreads, smem, s>>>(p);
+  full_fn(d, p.phase == 1 && p.R < 256 ? 2 : p.phase)<<<grid, kScoreThreads, smem, s>>>(p);
   return cudaGetLastError();
 }
 

@@ -156,6 +156,24 @@ __device__ __forceinline__ float s2_unit32(float c, uint64_t* tempty, uint32_t t
   return sum4x2(a);
 }
 
+// The same for 64 columns of which only the first `exist` (32 or more) hold rows.
+__device__ __forceinline__ float s2_unit_part(float c, uint64_t* tempty, uint32_t taddr, uint32_t g, const float* nl,
+                                              int exist) {
+  uint32_t ra[32], rb[32];
+  tmem_ld64_async(taddr + (g & (kSlots - 1)) * kSlotCols, ra, rb);
+  tmem_wait64(ra, rb);
+  unit_release(tempty, g);
+  float2 a[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  s2_chunk_full(ra, c, nl, a);
+#pragma unroll
+  for (int q = 0; q < 32; ++q) {
+    const float x = fmaf(__uint_as_float(rb[q]), c, lds1(nl + 32 + q));
+    const float e = ex2_approx(32 + q < exist ? x : -INFINITY);
+    if (q & 1) a[(q >> 1) & 3].y += e; else a[(q >> 1) & 3].x += e;
+  }
+  return sum4x2(a);
+}
+
 // Sweep 2 at the edges: up to nrows (64 or 32) rows, of which the first `exist`
 // exist; their place in a period of `per` rows counts up from i0, and a row
 // counts for this thread's key when its place is in [th, lim).  Any other gets
