@@ -158,6 +158,15 @@ def test_h2o_full_prompt_block_edges(torch, H_q, H_kv, d, lens, supplied_lse):
     test_h2o_full_prompt_scores_and_selection(torch, H_q, H_kv, d, lens, supplied_lse)
 
 
+# Groups that do not divide 256 rows: 252 to 255 rows a block (the last warpgroup's
+# 64 rows end at 55 to 63), over prompts with blocks past the causal cut of most
+# key super-tiles.
+@pytest.mark.parametrize("H_q,H_kv,d,lens", [
+    (3, 1, 64, (700, 1024)), (10, 2, 128, (617,)), (6, 1, 128, (672, 1000)), (7, 1, 64, (756, 755)), (13, 1, 64, (690,))])
+def test_h2o_full_prompt_partial_blocks(torch, H_q, H_kv, d, lens):
+    test_h2o_full_prompt_scores_and_selection(torch, H_q, H_kv, d, lens, False)
+
+
 def _full_prompt_workload(n, seed):
     route = [gen.H2O, gen.SNAPKV, gen.H2O]
     return gen.Workload(name=f"h2o_full_{n}", L=3, H_q=32, H_kv=8, d=128, B=1, lens=np.asarray([n], np.int32),
