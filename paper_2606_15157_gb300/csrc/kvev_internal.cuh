@@ -179,6 +179,7 @@ struct DecLayer {
 };
 
 constexpr int kMaxDecCluster = 8;      // CTAs an H2O / TOVA unit's step may be split over
+constexpr int kMinSplitSlots = 512;    // least capacity of a unit that is split
 constexpr int kDecCtasPerSm = 4;       // resident CTAs per SM of the step kernel (64 registers)
 
 struct DecodeParams {

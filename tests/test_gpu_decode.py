@@ -196,13 +196,15 @@ def test_decode_lockstep_mixed_rules(env, d):
 
 @pytest.mark.parametrize("H_q,H_kv,d,budgets", [
     (4, 2, 64, (127, 96)),      # one CTA per unit
-    (4, 2, 128, (257, 128)),    # clusters of two: 17 tiles of 16 indices, and 9
+    (4, 2, 128, (257, 128)),    # the same: 17 tiles of 16 indices, and 9
+    (20, 20, 64, (511, 257)),   # the same, one slot short of a split
+    (20, 20, 64, (512, 257)),   # clusters of two (120 units): 33 tiles, and 17
     (2, 2, 64, (527, 640)),     # four
     (8, 1, 128, (1025, 33)),    # eight: three tiles for most CTAs, and none for some
     (8, 2, 128, (1039, 2000)),  # eight, with a layer that is not full at first
 ])
 def test_decode_split_units(env, H_q, H_kv, d, budgets):
-    # A unit's step is split over 1, 2, 4 or 8 CTAs by the largest capacity; units
+    # A unit's step is split over 1, 2, 4 or 8 CTAs by the units and the largest capacity; units
     # whose indices (slots and the new token) end at, one past and one short of
     # a tile, whose CTAs have no tile, and that are not full yet.
     torch, kvev, orc = env
