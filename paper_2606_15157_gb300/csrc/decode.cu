@@ -597,16 +597,20 @@ __global__ void __launch_bounds__(kDecodeThreads, kDecCtasPerSm) decode_step_ker
     const int a = kSplit ? (b - n_cheap_ctas) / p.cluster : b;
     prefetch_token<D, G>(p.layer[p.att_layer[a / per_layer]], a % per_layer, true, threadIdx.x, kDecodeThreads);
     pdl_wait();
-    pdl_trigger();
     step_attend<D, G, kSplit>(p, a, lg, sh);
   } else {
     const int i = (b - n_att_ctas) * kDecodeWarps + (threadIdx.x >> 5);
     if (i < p.n_cheap)
       prefetch_token<D, G>(p.layer[p.cheap_layer[i / per_layer]], i % per_layer, false, threadIdx.x & 31, 32);
     pdl_wait();
-    pdl_trigger();
     if (i < p.n_cheap) step_cheap_warp(p, i, D);
   }
+  // The next kernel's CTAs come in as this one's finish.  Let in at the start of
+  // the step they were placed beside CTAs with most of their work ahead, and
+  // stayed there: 16 steps of 256 units of 256 slots 169 us, from here 152 (164
+  // for one CTA per unit and launches in order); 168 units of 512 slots in
+  // clusters of two 271 and 255 (289); 256 units of 64 slots 105 and 110 (122).
+  pdl_trigger();
   // The last CTA of the step to finish advances every sequence by one token:
   // every other CTA has read lens before it counted itself done.
   __syncthreads();
