@@ -89,7 +89,6 @@ struct __align__(16) SelShared {
   int wsum[kSW];
   int wS[kSW];    // per warp segment: sure positions staged
   int wC[kSW];    // per warp segment: candidates
-  int wB[kSW];    // per warp segment: first entry of its candidate list
   int wgt[kSW];   // per warp segment: keys above T (general path) / candidates above T
   int weq[kSW];   // per warp segment: keys (candidates) equal to T
   int bcast[2];
@@ -487,7 +486,6 @@ __device__ void classify_pass(uint16_t* bins, int E, uint32_t d, int first, int 
   if (lane == 0) {
     sh.wS[warp] = ns;
     sh.wC[warp] = nc;
-    sh.wB[warp] = first;
     if (nc > room) sh.overflow = 1;
   }
 }
@@ -511,9 +509,9 @@ __device__ int count_candidates(const uint16_t* bins, int E, uint32_t d) {
 
 // The keys of each warp's listed candidates, from the scores.
 template <int NT>
-__device__ void candidate_keys(const Scalar& sk, SelShared<NT>& sh) {
+__device__ void candidate_keys(const Scalar& sk, int first, SelShared<NT>& sh) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nc = sh.wC[warp], first = sh.wB[warp];
+  const int nc = sh.wC[warp];
   for (int i = lane; i < nc; i += 32) sh.u.c.key[first + i] = sk.one(static_cast<int>(sh.u.c.pos[first + i]));
 }
 
@@ -538,8 +536,8 @@ __device__ void finish_few(const Scalar& sk, const uint16_t* bins, int E, int kk
   uint32_t pos = 0;
   int sure = 0;
   if (lane < nc) {
-    pos = sh.u.c.pos[sh.wB[warp] + lane];
-    sure = sh.u.c.sure[sh.wB[warp] + lane];
+    pos = sh.u.c.pos[warp * SelShared<NT>::kCandPerWarp + lane];
+    sure = sh.u.c.sure[warp * SelShared<NT>::kCandPerWarp + lane];
     sh.few[first + lane] = sk.one(static_cast<int>(pos));
   }
   __syncthreads();
@@ -569,14 +567,14 @@ __device__ void finish_few(const Scalar& sk, const uint16_t* bins, int E, int kk
 // equal to T to keep, by radix passes of up to 9 bits over key - (least
 // candidate key); then each warp counts its candidates above and equal to T.
 template <int NT>
-__device__ void select_candidates(int kk, SelShared<NT>& sh, uint32_t& T, int& need) {
+__device__ void select_candidates(int kk, int first, SelShared<NT>& sh, uint32_t& T, int& need) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
     sh.rlo = 0xFFFFFFFFu;
     sh.rhi = 0u;
   }
   __syncthreads();
-  const uint32_t* keys = sh.u.c.key + sh.wB[warp];
+  const uint32_t* keys = sh.u.c.key + first;
   const int nc = sh.wC[warp];
   uint32_t lo = 0xFFFFFFFFu, hi = 0u;
   for (int i = lane; i < nc; i += 32) {
@@ -633,7 +631,7 @@ __device__ void select_candidates(int kk, SelShared<NT>& sh, uint32_t& T, int& n
 // position j to base + j + (kept candidates with at most j sure positions
 // before them).
 template <int NT>
-__device__ void merge_write(const uint16_t* bins, int E, int k, int need, SelShared<NT>& sh, uint32_t T, int* out) {
+__device__ void merge_write(const uint16_t* bins, int E, int k, int need, int first, SelShared<NT>& sh, uint32_t T, int* out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t lt = (1u << lane) - 1u;
   int base = 0, eq_base = 0;
@@ -641,7 +639,7 @@ __device__ void merge_write(const uint16_t* bins, int E, int k, int need, SelSha
     base += sh.wS[w] + sh.wgt[w] + min(max(need - eq_base, 0), sh.weq[w]);
     eq_base += sh.weq[w];
   }
-  const int nc = sh.wC[warp], first = sh.wB[warp];
+  const int nc = sh.wC[warp];
   int* sure = sh.u.c.sure + first;
   int nk = 0;  // kept candidates so far; their sure counts are compacted into sure[0 .. nk)
   for (int i0 = 0; i0 < nc; i0 += 32) {
@@ -680,6 +678,18 @@ __device__ void merge_write(const uint16_t* bins, int E, int k, int need, SelSha
     }
     if (base + j + a < k) out[base + j + a] = pos;
   }
+}
+
+// Steps 3 and 4 from the candidate lists (this warp's starts at `first`).
+template <int NT>
+__device__ void finish_lists(const Scalar& sk, const uint16_t* bins, int E, int kk, int k, int first, SelShared<NT>& sh,
+                             int* out) {
+  candidate_keys(sk, first, sh);
+  __syncthreads();
+  uint32_t T;
+  int need;
+  select_candidates(kk, first, sh, T, need);
+  merge_write(bins, E, k, need, first, sh, T, out);
 }
 
 // The general path: four 8-bit radix passes over every key, then each warp
@@ -804,43 +814,37 @@ __device__ void select_unit(const Gen& gen, const Scalar& sk, uint32_t* row, int
   const int nd = sh.u.hist[d];
   __syncthreads();  // every thread has read it before the candidate lists overwrite the histogram
   // the end bins also hold keys outside the sampled range: not one prefix
-  bool fast = d > 0 && d < kBins0 - 1 && nd <= kCandidates && seg_len<NT>(E) <= 65536;
-  if (fast) {
-    constexpr int kCandPerWarp = SelShared<NT>::kCandPerWarp;
-    const int warp = threadIdx.x >> 5;
-    int first = warp * kCandPerWarp, room = kCandPerWarp;
-    if (NT > 256 && nd > kCandPerWarp) {
-      // The more warps, the shorter an equal share of the list (160 or 80
-      // entries; 320 for 256 threads), and crowded scores lie in few segments:
-      // the shares are counted out first.  200 equal scores in a run, 256 units
-      // of 8,192: the call 29.0 us, with equal shares (the general path) 37.6; with
-      // 256 threads their 320 entries hold them, 29.2.
-      room = count_candidates<NT>(bins, E, static_cast<uint32_t>(d));
-      if ((threadIdx.x & 31) == 0) sh.wC[warp] = room;
-      __syncthreads();
-      const int lane = threadIdx.x & 31;
-      first = warp_sum(lane < warp ? sh.wC[lane] : 0);
-    }
-    classify_pass(bins, E, static_cast<uint32_t>(d), first, room, sh);
+  constexpr int kShare = SelShared<NT>::kCandPerWarp;
+  const int warp = threadIdx.x >> 5;
+  const bool fast = d > 0 && d < kBins0 - 1 && nd <= kCandidates && seg_len<NT>(E) <= 65536;
+  if (fast && (NT == 256 || nd <= kShare)) {  // lists of an equal share each
+    const int first = warp * kShare;
+    classify_pass(bins, E, static_cast<uint32_t>(d), first, kShare, sh);
     __syncthreads();
-    fast = !sh.overflow;
     if (nd <= kFewCandidates) return finish_few(sk, bins, E, k - above, k, nd, sh, out);
-    if (fast) {
-      candidate_keys(sk, sh);
-      __syncthreads();
-    }
-  }
-  uint32_t T;
-  int need;
-  if (fast) {
-    select_candidates(k - above, sh, T, need);
-    merge_write(bins, E, k, need, sh, T, out);
-    return;
+    if (!sh.overflow) return finish_lists(sk, bins, E, k - above, k, first, sh, out);
+  } else if (fast) {
+    // The more warps, the shorter an equal share (160 or 80 entries; 320 for 256
+    // threads), and crowded scores lie in few segments: the lists are laid out
+    // by what each warp counts.  200 equal scores in a run, 256 units of 8,192:
+    // the call 29.0 us, with equal shares (the general path) 37.6; with 256
+    // threads, whose shares hold them, 29.2.  In the equal shares' way, instead of
+    // beside it, the counting cost every unit 0.6 us.
+    const int lane = threadIdx.x & 31;
+    const int mine = count_candidates<NT>(bins, E, static_cast<uint32_t>(d));
+    if (lane == 0) sh.wC[warp] = mine;
+    __syncthreads();
+    const int first = warp_sum(lane < warp ? sh.wC[lane] : 0);
+    classify_pass(bins, E, static_cast<uint32_t>(d), first, mine, sh);
+    __syncthreads();
+    return finish_lists(sk, bins, E, k - above, k, first, sh, out);
   }
   // the general path: many equal keys, or a sample that missed the k-th key:
   // the row holds bins, so the keys are built now
   build_row<NT>(gen, row, E);
   __syncthreads();
+  uint32_t T;
+  int need;
   select_all_keys(row, E, k, sh, T, need);
   write_kept(row, E, k, T, need, sh, out);
 }
