@@ -220,7 +220,9 @@ __device__ __forceinline__ void prefetch_row_l2(const float* src, int n) {
 // Key generators: eight consecutive keys of [0, E) from position i0 (a multiple
 // of eight, i0 < E), in two halves -- load() issues the reads, keys() computes
 // -- so that a pass can have the next block's reads in flight while it works
-// on the current one.  Keys past E are computed but never used.
+// on the current one.  Keys past E are computed but never used.  Plain loads,
+// not __ldg: the launch overlaps the kernels that write the scores, so they are
+// not constant while this grid exists, only from pdl_wait on.
 // ---------------------------------------------------------------------------
 constexpr int kGen = 8;
 
@@ -244,7 +246,7 @@ struct Pooled {
     for (int c = 0; c < 4; ++c) {
       const int st = i0 - 4 + 4 * c;
       r.c[c] = make_float4(kFill, kFill, kFill, kFill);
-      if (st >= 0 && st < E) r.c[c] = __ldg(reinterpret_cast<const float4*>(raw + st));  // neighbours': L1
+      if (st >= 0 && st < E) r.c[c] = *reinterpret_cast<const float4*>(raw + st);  // neighbours': L1
     }
   }
   __device__ __forceinline__ void keys(int i0, const Regs& r, uint32_t (&kq)[kGen]) const {
@@ -283,8 +285,8 @@ struct Raw {
     float4 v[2];
   };
   __device__ __forceinline__ void load(int i0, Regs& r) const {
-    r.v[0] = __ldg(reinterpret_cast<const float4*>(raw + i0));
-    r.v[1] = i0 + 4 < E ? __ldg(reinterpret_cast<const float4*>(raw + i0 + 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    r.v[0] = *reinterpret_cast<const float4*>(raw + i0);
+    r.v[1] = i0 + 4 < E ? *reinterpret_cast<const float4*>(raw + i0 + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
   __device__ __forceinline__ void keys(int, const Regs& r, uint32_t (&kq)[kGen]) const {
 #pragma unroll
