@@ -559,6 +559,7 @@ __device__ __forceinline__ void publisher(const ScoreParams& p, const Smem& sm, 
         __threadfence();
       }
       if (!__shfl_sync(0xffffffffu, last, 0)) continue;
+      __syncwarp();  // the other lanes read the group's records after lane 0's fence (a shuffle orders no memory)
       float2* g = p.part + static_cast<size_t>(it.cs + c0) * p.R_pad;
       for (int i = 0; i < nr; ++i) {
         float2 e[kMaxGroup];
