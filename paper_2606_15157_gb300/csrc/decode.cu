@@ -44,11 +44,11 @@ __device__ __forceinline__ int find_dec_layer(const DecodeParams& p, int u) {
   return lo;
 }
 
-// A CTA's eviction candidate (slot -1: none) and, from the CTA that holds the
-// new token's index, the new token's key.
+// A warp's or CTA's eviction candidate (DecChoice) and, from the CTA that holds
+// the new token's index, the new token's key.
 struct __align__(16) DecCandidate {
-  float key;
-  int pos, slot;
+  uint32_t hi, lo;
+  int aux;
   float new_key;
 };
 
@@ -99,8 +99,8 @@ __device__ __forceinline__ void st_cluster(uint32_t addr, float v) {
 }
 
 __device__ __forceinline__ void st_cluster(uint32_t addr, const DecCandidate& c) {
-  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(__float_as_int(c.key)),
-               "r"(c.pos), "r"(c.slot), "r"(__float_as_int(c.new_key))
+  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(c.hi), "r"(c.lo),
+               "r"(c.aux), "r"(__float_as_int(c.new_key))
                : "memory");
 }
 
@@ -113,38 +113,45 @@ __device__ __forceinline__ float over_warps(const float (&w)[kDecodeWarps]) {
               : ((((((a.x + a.y) + a.z) + a.w) + b.x) + b.y) + b.z) + b.w;
 }
 
-// Eviction order: smaller key first, then higher position first.
-__device__ __forceinline__ bool evict_before(float a, int pa, float b, int pb) {
-  return a < b || (a == b && pa > pb);
+// Eviction order: smaller key first, then higher position first; NaN before every
+// number, the lower slot first.  As two words whose lexicographic minimum is the
+// slot to evict the order is total, so that every lane, warp and CTA that merges
+// candidates ends with the same one: each thread writes its part of the new row
+// to the slot it found.
+struct DecChoice {
+  uint32_t hi, lo;  // hi 0: NaN; all ones: no candidate
+  int aux;          // the slot, or with a NaN key, whose slot is lo, the position
+  __device__ __forceinline__ int slot() const { return hi == 0 ? static_cast<int>(lo) : aux; }
+  __device__ __forceinline__ int pos() const { return hi == 0 ? aux : static_cast<int>(0x7FFFFFFFu - lo); }
+  __device__ __forceinline__ bool before(const DecChoice& o) const { return hi < o.hi || (hi == o.hi && lo < o.lo); }
+};
+constexpr DecChoice kNoChoice = {0xFFFFFFFFu, 0xFFFFFFFFu, -1};
+
+__device__ __forceinline__ DecChoice candidate(float key, int pos, int slot) {
+  const uint32_t u = __float_as_uint(key + 0.f);  // -0 as 0
+  if (key != key) return DecChoice{0u, static_cast<uint32_t>(slot), pos};
+  return DecChoice{u ^ (static_cast<uint32_t>(static_cast<int>(u) >> 31) | 0x80000000u),
+                   0x7FFFFFFFu - static_cast<uint32_t>(pos), slot};
 }
 
-// The first candidate in eviction order (candidates have pos >= 0) over lanes
-// that differ in the bits of `lanes` (a power of two, exclusive), in each.
-__device__ __forceinline__ void warp_evict_choice(float& a, int& pos, int& slot, int lanes) {
-  for (int o = lanes >> 1; o > 0; o >>= 1) {
-    const float a2 = __shfl_xor_sync(0xffffffffu, a, o);
-    const int p2 = __shfl_xor_sync(0xffffffffu, pos, o);
-    const int s2 = __shfl_xor_sync(0xffffffffu, slot, o);
-    if (p2 >= 0 && (pos < 0 || evict_before(a2, p2, a, pos))) {
-      a = a2;
-      pos = p2;
-      slot = s2;
-    }
-  }
+// The first candidate of the warp's lanes, in every lane.
+__device__ __forceinline__ DecChoice warp_evict_choice(const DecChoice& d) {
+  DecChoice r;
+  r.hi = __reduce_min_sync(0xffffffffu, d.hi);
+  r.lo = __reduce_min_sync(0xffffffffu, d.hi == r.hi ? d.lo : 0xFFFFFFFFu);
+  const uint32_t who = __ballot_sync(0xffffffffu, d.hi == r.hi && d.lo == r.lo);
+  r.aux = __shfl_sync(0xffffffffu, d.aux, __ffs(who) - 1);
+  return r;
 }
 
 // Block-wide first candidate, in every thread; slot -1 if there is none.
-__device__ __forceinline__ void block_evict_choice(float& a, int& pos, int& slot, DecCandidate (&wcand)[kDecodeWarps]) {
+__device__ __forceinline__ DecChoice block_evict_choice(const DecChoice& d, DecCandidate (&wcand)[kDecodeWarps]) {
   const int lane = threadIdx.x & 31;
-  warp_evict_choice(a, pos, slot, 32);
-  if (lane == 0) wcand[threadIdx.x >> 5] = DecCandidate{a, pos, slot, 0.f};
+  const DecChoice w = warp_evict_choice(d);
+  if (lane == 0) wcand[threadIdx.x >> 5] = DecCandidate{w.hi, w.lo, w.aux, 0.f};
   __syncthreads();
-  const DecCandidate d = wcand[lane & (kDecodeWarps - 1)];
-  a = d.key;
-  pos = d.pos;
-  slot = d.slot;
-  warp_evict_choice(a, pos, slot, kDecodeWarps);
-  if (pos < 0) slot = -1;
+  const DecCandidate e = wcand[lane & (kDecodeWarps - 1)];
+  return warp_evict_choice(DecChoice{e.hi, e.lo, e.aux});
 }
 
 // Copy one d-wide bf16 row (16-byte vectors) with the whole block.
@@ -358,8 +365,7 @@ __device__ void attend_unit(const DecodeParams& p, const DecLayer& ly, const Uni
   if (at != nullptr) at += base;
   const int limit = n + 1 - ly.r;  // positions >= limit are protected
   const int mc = c - base;         // the new token's local index
-  float ba = INFINITY;
-  int bp = -1, bs = -1;
+  DecChoice ev = kNoChoice;        // the slot to evict: of the thread's slots, then of all
   constexpr int kU = 4;  // slots per thread whose global loads are issued together
   for (int j0 = threadIdx.x; j0 < m; j0 += kU * kDecodeThreads) {
     float accv[kU], atv[kU];
@@ -385,42 +391,34 @@ __device__ void attend_unit(const DecodeParams& p, const DecLayer& ly, const Uni
       const float a = accv[q] + pj;
       lg[j] = a;
       const int pos = posv[q];
-      if (pos >= 0 && pos < limit && (bp < 0 || evict_before(a, pos, ba, bp))) {
-        ba = a;
-        bp = pos;
-        bs = base + j;
+      if (pos >= 0 && pos < limit) {
+        const DecChoice x = candidate(a, pos, base + j);
+        if (x.before(ev)) ev = x;
       }
     }
   }
   const bool full = c >= ly.b;
   float new_key = 0.f;
   if (full) {
-    block_evict_choice(ba, bp, bs, sh.wcand);  // bs = c: the new token; ends past a barrier: lg is complete
+    ev = block_evict_choice(ev, sh.wcand);  // slot c: the new token; ends past a barrier: lg is complete
     if (kSplit) {
       if (static_cast<int>(threadIdx.x) < C)
         st_cluster(cluster_addr(&sh.cand[rank], threadIdx.x),
-                   DecCandidate{ba, bp, bs, mc >= 0 && mc < m ? lg[mc] : 0.f});
+                   DecCandidate{ev.hi, ev.lo, ev.aux, mc >= 0 && mc < m ? lg[mc] : 0.f});
       __syncwarp();
       cluster_sync();
       const int k = threadIdx.x & 7;
-      bs = -1;
-      bp = -1;
-      if (k < C) {
-        const DecCandidate d = sh.cand[k];
-        ba = d.key;
-        bp = d.pos;
-        bs = d.slot;
-      }
-      warp_evict_choice(ba, bp, bs, 8);
+      ev = warp_evict_choice(k < C ? DecChoice{sh.cand[k].hi, sh.cand[k].lo, sh.cand[k].aux} : kNoChoice);
       new_key = sh.cand[(c / 16) / per].new_key;
     } else {
       new_key = lg[c];
     }
   } else {
-    bs = -1;
+    ev = kNoChoice;
     __syncthreads();
     if (mc >= 0 && mc < m) new_key = lg[mc];
   }
+  const int bs = ev.slot();
   for (int j = threadIdx.x; j < m; j += blockDim.x)
     if (j < mc && base + j != bs) p.acc[r.rows0 + base + j] = lg[j];
   const bool lead = rank == 0 && threadIdx.x == 0;
@@ -440,7 +438,7 @@ __device__ void attend_unit(const DecodeParams& p, const DecLayer& ly, const Uni
     if (bs < c && bs >= base && bs < base + m) place_new(p, ly, r, D, bs, n, new_key);
     if (lead) {
       p.count[r.u] = c;
-      p.evicted[r.u] = bp;  // the new token's own position when it is the one evicted
+      p.evicted[r.u] = ev.pos();  // the new token's own position when it is the one evicted
     }
   }
 }

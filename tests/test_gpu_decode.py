@@ -259,6 +259,65 @@ def test_decode_split_infinite_logits(env):
     assert plan.status() == kvev.OK
 
 
+@pytest.mark.parametrize("H_q,H_kv,d,budget,supplied", [
+    (4, 2, 64, 100, False), (4, 2, 64, 100, True),  # one CTA per unit
+    (20, 20, 64, 520, False),                       # clusters of two
+    (2, 1, 128, 1040, False), (8, 1, 64, 1100, False)])  # eight
+def test_decode_nan_attention(env, H_q, H_kv, d, budget, supplied):
+    # A NaN logit makes a unit's attention, and so its keys, NaN from then on (a
+    # supplied NaN only its slot's): the eviction is still one slot, chosen alike
+    # by every thread and CTA -- NaN before every number, the lower slot first --
+    # and every slot holds the row of the position it claims.
+    torch, kvev, orc = env
+    n, steps = budget + 60, 4
+    wl = gen.Workload(name="nan", L=2, H_q=H_q, H_kv=H_kv, d=d, B=1, lens=np.array([n], np.int32), S_cap=n, W=8,
+                      pool_kernel=5, pool_type=gen.POOL_AVG, route=np.array([gen.H2O, gen.H2O], np.int32),
+                      budget=np.array([budget, budget], np.int32), sink=4, seed=13, sink_tokens=4, sink_scale=4.0,
+                      route_decode=np.array([gen.H2O, gen.TOVA], np.int32), decode_steps=steps)
+    plan, bufs, arena = prefill_and_arena(torch, kvev, wl, 0)
+    g = Arena(torch, arena, wl)
+    rows = {}  # per unit: position -> K and V rows
+    for i in range(len(g.units)):
+        x = g.unit(i)
+        rows[i] = {int(p): (x["K"][j].copy(), x["V"][j].copy()) for j, p in enumerate(x["pos"])}
+    rng = np.random.default_rng(1)
+    for step in range(steps):
+        toks, k, v, q = step_tokens(wl, step, range(wl.L))
+        before = [g.unit(i) for i in range(len(g.units))]
+        if supplied:
+            attn = []
+            for l, (off, cap, u0) in enumerate(arena.layers):
+                x = rng.random((1, H_kv, cap + 1)).astype(np.float32)
+                x[:, :, rng.choice(cap, cap // 2, replace=False)] = np.nan
+                attn.append(torch.from_numpy(x).cuda())
+            arena.step_attn(k, v, attn)
+        else:
+            for x in q:
+                x[:, 0, 0] = float("nan")  # one head of the first group; the other groups' units stay finite
+            arena.step(k, v, q)
+        g.refresh(torch)
+        for i in range(len(g.units)):
+            l, s, h, u = g.units[i][:4]
+            kk, vv = (t.view(torch.int16).cpu().numpy().view(np.uint16)[s, h] for t in toks[l][:2])
+            rows[i][n + step] = (kk, vv)
+            x = g.unit(i)
+            assert x["count"] == budget and len(set(x["pos"].tolist())) == budget
+            for j, p in enumerate(x["pos"]):
+                assert np.array_equal(x["K"][j], rows[i][int(p)][0]), f"step {step} unit {i}: K row of position {p}"
+                assert np.array_equal(x["V"][j], rows[i][int(p)][1]), f"step {step} unit {i}: V row of position {p}"
+            limit = n + step + 1 - (budget // 2 if l == 0 else 0)
+            old = [int(p) for p in before[i]["pos"]] + [n + step]
+            ev = int(g.evicted[u])
+            assert ev in old and ev < limit and ev not in x["pos"]
+            if supplied:
+                w = attn[l][s, h].cpu().numpy()
+                nan = np.isnan(w + np.append(before[i]["acc"] if l == 0 else np.zeros(budget), 0.0))
+                assert ev == [p for p, x in zip(old, nan) if x and p < limit][0], f"step {step} unit {i}"
+            elif h == 0:
+                assert ev == [p for p in old if p < limit][0], f"step {step} unit {i}"
+    assert plan.status() == kvev.OK
+
+
 def _bf16_to_f64(u16):
     return (np.asarray(u16, np.uint32) << 16).view(np.float32).astype(np.float64)
 
