@@ -238,7 +238,7 @@ KVEV_API int kvev_plan_scores_offset(const kvev_plan *plan, int B, int S_cap, in
  *     positions plus the top (b_l - h2o_recent) scores before them.
  *   StreamingLLM: keep positions [0, sink) and the last `recent` positions.
  *   Any rule with b_l >= lens[s] keeps every position.
- * Top-k ties keep the lower position.
+ * Top-k ties keep the lower position; a NaN score counts as -inf.
  * EINVAL on null/misaligned pointers or B < 0, S_cap < 1; ENOMEM if the
  * workspace is smaller than kvev_plan_query() reports.  The workspace holds,
  * among the rest, 4 bytes per position per (scoring layer, sequence, KV head)

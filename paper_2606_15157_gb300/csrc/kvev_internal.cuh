@@ -568,10 +568,14 @@ __device__ __forceinline__ int ld_volatile(const int* p) {
   return *reinterpret_cast<const volatile int*>(p);
 }
 
-// Order-preserving map of an fp32 to uint32 (larger float -> larger key).
+// Order-preserving map of an fp32 to uint32 (larger float -> larger key).  NaN
+// counts as -inf.  (Said here, as the compiler turns sign-bit arithmetic on a
+// float's bits into floating-point operations where it sees the float, which may
+// change a NaN's bits: the same NaN had one key in some registers and another in
+// others.)
 __device__ __forceinline__ uint32_t float_key(float f) {
-  uint32_t u = __float_as_uint(f);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+  const uint32_t u = __float_as_uint(fmaxf(f, -INFINITY));
+  return u ^ (static_cast<uint32_t>(static_cast<int>(u) >> 31) | 0x80000000u);
 }
 
 }  // namespace kvev

@@ -483,6 +483,30 @@ def test_select_wide_pooling(torch, S_cap, pool, pool_type):
             assert np.array_equal(idx[1, s, h], np.concatenate([_top(pooled, b - W), np.arange(E, n)])), f"n={n}"
 
 
+@pytest.mark.parametrize("S_cap", [1032, 1031])
+@pytest.mark.parametrize("pool,pool_type", [(5, gen.POOL_AVG), (5, gen.POOL_MAX), (11, gen.POOL_AVG)])
+def test_select_nan_scores(torch, S_cap, pool, pool_type):
+    # NaN scores rank below every number, wherever in a row they are: from a few,
+    # which are never kept, to so many that the lowest positions among them are.
+    rng = np.random.default_rng(S_cap + pool)
+    b, W = 40, 8
+    lens = np.array([1031, 1030, 600, 129, 57], np.int32)
+    raw = rng.random((2, len(lens), 2, S_cap)).astype(np.float32) + np.float32(0.01)
+    raw[rng.random(raw.shape) < np.array([0.001, 0.1, 0.5, 0.9, 0.99])[None, :, None, None]] = np.nan
+    idx = _select_supplied(torch, raw, lens, b, W, pool, pool_type, S_cap)
+    is_max = pool_type == gen.POOL_MAX
+    for s, n in enumerate(lens):
+        for h in range(2):
+            assert np.array_equal(idx[0, s, h], _top(np.nan_to_num(raw[0, s, h, :n], nan=-np.inf), b)), f"H2O n={n}"
+            E = n - W
+            pad = np.pad(raw[1, s, h, :E], pool // 2, constant_values=-np.inf if is_max else 0)
+            pooled = pad[:E].copy()
+            for j in range(1, pool):  # a maximum over the numbers, a sum with any NaN is NaN
+                pooled = np.fmax(pooled, pad[j:j + E]) if is_max else pooled + pad[j:j + E]
+            keep = _top(np.where(np.isnan(pooled), -np.inf, pooled), b - W)
+            assert np.array_equal(idx[1, s, h], np.concatenate([keep, np.arange(E, n)])), f"SnapKV n={n}"
+
+
 def test_capacity_beyond_shared_memory(torch, orc):
     # Capacities past what one CTA's shared memory could hold as keys (53,504
     # positions at 4 bytes): the selection keeps them in the workspace at any
