@@ -408,7 +408,8 @@ KVEV_API int kvev_decode_init(kvev_plan *plan, int B, int growth, const void *pr
  *         softmax_j(q . k_j / sqrt(d)) over the retained slots and the new
  *         token; acc += p; once b slots are held, the slot with the smallest
  *         acc among positions < lens+1-r (r = h2o_recent, or floor(b/2)) is
- *         evicted (ties: the higher position) and the new token takes it.
+ *         evicted (ties: the higher position; a NaN acc comes after every
+ *         number, the lower slot first) and the new token takes it.
  *   TOVA: the same with acc = p (no accumulation) and r = 0, so the new token
  *         itself may be the one evicted.
  *   StreamingLLM: once sink + recent slots are held, the smallest position

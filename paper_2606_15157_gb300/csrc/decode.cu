@@ -113,23 +113,24 @@ __device__ __forceinline__ float over_warps(const float (&w)[kDecodeWarps]) {
               : ((((((a.x + a.y) + a.z) + a.w) + b.x) + b.y) + b.z) + b.w;
 }
 
-// Eviction order: smaller key first, then higher position first; NaN before every
+// Eviction order: smaller key first, then higher position first; NaN after every
 // number, the lower slot first.  As two words whose lexicographic minimum is the
 // slot to evict the order is total, so that every lane, warp and CTA that merges
 // candidates ends with the same one: each thread writes its part of the new row
 // to the slot it found.
 struct DecChoice {
-  uint32_t hi, lo;  // hi 0: NaN; all ones: no candidate
+  static constexpr uint32_t kNaN = 0xFFFFFFFEu;  // past +inf's
+  uint32_t hi, lo;  // all ones: no candidate
   int aux;          // the slot, or with a NaN key, whose slot is lo, the position
-  __device__ __forceinline__ int slot() const { return hi == 0 ? static_cast<int>(lo) : aux; }
-  __device__ __forceinline__ int pos() const { return hi == 0 ? aux : static_cast<int>(0x7FFFFFFFu - lo); }
+  __device__ __forceinline__ int slot() const { return hi == kNaN ? static_cast<int>(lo) : aux; }
+  __device__ __forceinline__ int pos() const { return hi == kNaN ? aux : static_cast<int>(0x7FFFFFFFu - lo); }
   __device__ __forceinline__ bool before(const DecChoice& o) const { return hi < o.hi || (hi == o.hi && lo < o.lo); }
 };
 constexpr DecChoice kNoChoice = {0xFFFFFFFFu, 0xFFFFFFFFu, -1};
 
 __device__ __forceinline__ DecChoice candidate(float key, int pos, int slot) {
   const uint32_t u = __float_as_uint(key + 0.f);  // -0 as 0
-  if (key != key) return DecChoice{0u, static_cast<uint32_t>(slot), pos};
+  if (key != key) return DecChoice{DecChoice::kNaN, static_cast<uint32_t>(slot), pos};
   return DecChoice{u ^ (static_cast<uint32_t>(static_cast<int>(u) >> 31) | 0x80000000u),
                    0x7FFFFFFFu - static_cast<uint32_t>(pos), slot};
 }

@@ -266,7 +266,7 @@ def test_decode_split_infinite_logits(env):
 def test_decode_nan_attention(env, H_q, H_kv, d, budget, supplied):
     # A NaN logit makes a unit's attention, and so its keys, NaN from then on (a
     # supplied NaN only its slot's): the eviction is still one slot, chosen alike
-    # by every thread and CTA -- NaN before every number, the lower slot first --
+    # by every thread and CTA -- NaN after every number, the lower slot first --
     # and every slot holds the row of the position it claims.
     torch, kvev, orc = env
     n, steps = budget + 60, 4
@@ -311,8 +311,9 @@ def test_decode_nan_attention(env, H_q, H_kv, d, budget, supplied):
             assert ev in old and ev < limit and ev not in x["pos"]
             if supplied:
                 w = attn[l][s, h].cpu().numpy()
-                nan = np.isnan(w + np.append(before[i]["acc"] if l == 0 else np.zeros(budget), 0.0))
-                assert ev == [p for p, x in zip(old, nan) if x and p < limit][0], f"step {step} unit {i}"
+                key = np.append(before[i]["acc"] if l == 0 else np.zeros(budget), 0.0).astype(np.float32) + w
+                best = [(np.isnan(a), j if np.isnan(a) else a, -p) for j, (a, p) in enumerate(zip(key, old)) if p < limit]
+                assert ev == -min(best)[2], f"step {step} unit {i}"
             elif h == 0:
                 assert ev == [p for p in old if p < limit][0], f"step {step} unit {i}"
     assert plan.status() == kvev.OK
