@@ -306,7 +306,6 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
-// Same, with an L2 cache-eviction policy (from createpolicy).
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z,
                                             uint64_t* bar) {
   asm volatile(
@@ -316,6 +315,7 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
+// The 2-D load with an L2 cache-eviction policy (from createpolicy).
 __device__ __forceinline__ void tma_load_2d_hint(void* dst, const CUtensorMap* map, int x, int y,
                                                  uint64_t* bar, uint64_t policy) {
   asm volatile(
@@ -335,10 +335,6 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
   uint64_t p;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
   return p;
-}
-
-__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
-  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
 // ---- programmatic dependent launch ---------------------------------------------
@@ -372,19 +368,9 @@ __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// D(tmem) (+)= A(smem) * B(smem)^T, bf16 inputs, fp32 accumulate, one CTA.
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                          uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// The same MMA issued from a whole converged warp: one elected lane issues, so
-// the warp-uniform operands can stay in uniform registers.
+// D(tmem) (+)= A(smem) * B(smem)^T, bf16 inputs, fp32 accumulate, one CTA, issued
+// from a whole converged warp: one elected lane issues, so the warp-uniform
+// operands can stay in uniform registers.
 __device__ __forceinline__ void umma_bf16_elect(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
                                                 uint32_t idesc, uint32_t accumulate) {
   asm volatile(
@@ -396,8 +382,9 @@ __device__ __forceinline__ void umma_bf16_elect(uint32_t d_tmem, uint64_t a_desc
       : "memory");
 }
 
-// tcgen05.commit from the lane that elect.sync picks in a converged warp (the
-// same lane that issued the MMAs through umma_bf16_elect).
+// Arrive on `bar` once the tcgen05 operations issued so far complete, from the
+// lane that elect.sync picks in a converged warp (the same lane that issued the
+// MMAs through umma_bf16_elect).
 __device__ __forceinline__ void umma_commit_elect(uint64_t* bar) {
   asm volatile(
       "{\n\t.reg .pred e;\n\t"
@@ -407,20 +394,6 @@ __device__ __forceinline__ void umma_commit_elect(uint64_t* bar) {
       : "memory");
 }
 
-// Arrive on `bar` once every tcgen05 operation issued so far by this thread completes.
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-          smem_u32(bar))
-      : "memory");
-}
-
-__device__ __forceinline__ void tmem_wait_ld() {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// Issue a load of 32 consecutive fp32 columns of this thread's TMEM lane; the
-// registers are valid only after tmem_wait32() on the same array.
 // 64 consecutive fp32 columns of this thread's TMEM lane in one load: columns
 // [0, 32) into r0 and [32, 64) into r1; valid only after tmem_wait64().
 __device__ __forceinline__ void tmem_ld64_async(uint32_t taddr, uint32_t (&r0)[32], uint32_t (&r1)[32]) {
@@ -439,6 +412,7 @@ __device__ __forceinline__ void tmem_wait64(uint32_t (&r0)[32], uint32_t (&r1)[3
       : "memory");
 }
 
+// 32 consecutive fp32 columns; valid only after tmem_wait32() on the same array.
 __device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
