@@ -114,22 +114,25 @@ def _ptr_array(ptrs, n: int):
     ones NULL.  The caller keeps it until the library call returns.  (A ctypes array of 32 pointers
     takes 2.7 us to make, this 0.6; a decode step passes three.  Lists with anything but ints, and
     iterators, which can be read once only, go the ctypes way.)"""
-    if isinstance(ptrs, (list, tuple)):
+    if type(ptrs) is list or type(ptrs) is tuple:
         try:
             a = array("Q", ptrs)
         except (TypeError, OverflowError):
-            return (C.c_void_p * n)(*ptrs)
-        if len(a) > n:
-            raise IndexError(f"{len(a)} pointers for {n} layers")
-        a.extend([0] * (n - len(a)))
-        return a
-    return (C.c_void_p * n)(*ptrs)
+            pass
+        else:
+            if len(a) == n:
+                return a
+            if len(a) > n:
+                raise IndexError(f"{len(a)} pointers for {n} layers")
+            a.extend([0] * (n - len(a)))
+            return a
+    a = array("Q")
+    a.frombytes(bytes((C.c_void_p * n)(*ptrs)))
+    return a
 
 
 def _addr(a):
-    if a is None:
-        return None
-    return a.buffer_info()[0] if isinstance(a, array) else C.addressof(a)
+    return None if a is None else a.buffer_info()[0]
 
 
 def _data_ptrs(tensors):

@@ -301,11 +301,11 @@ def test_binding_argtypes_match_header(kv):
     lambda: [3], lambda: [], lambda: [3, 4, 5], lambda: [1.5, 2], lambda: "ab", lambda: b"ab", lambda: None])
 def test_pointer_lists_convert_as_ctypes_does(kv, make):
     # the pointer-level functions take what an array of void pointers takes, and refuse what it refuses
-    def words(f):
+    def words(convert, address):
         try:
-            a = f()
+            a = convert()
         except Exception as e:
             return type(e)
-        return list((C.c_uint64 * 2).from_address(kv._addr(a)))
-    assert words(lambda: kv._ptr_array(make(), 2)) == words(lambda: (C.c_void_p * 2)(*make()))
+        return list((C.c_uint64 * 2).from_address(address(a)))
+    assert words(lambda: kv._ptr_array(make(), 2), kv._addr) == words(lambda: (C.c_void_p * 2)(*make()), C.addressof)
     assert kv._addr(None) is None
