@@ -670,7 +670,7 @@ int evict_impl(kvev_plan& P, DevCtx& D, const void* const* K, const void* const*
 
   // ---- prologue: validated lengths, work items, flag reset -------------
   const int n_slayers = static_cast<int>(P.score_layers.size());
-  // chunk size: at least kMinChunkTiles tiles, and few enough chunks per unit
+  // chunk size: at least min_chunk_tiles tiles, and few enough chunks per unit
   // that a unit never spans more than two rounds of the persistent grid
   const int grid = D.num_sms;
   const int tiles_max = (S_cap + kTileKeys - 1) / kTileKeys;
@@ -1141,7 +1141,9 @@ extern "C" int kvev_decode_init(kvev_plan* plan, int B, int growth, const void* 
   dp.h2o_state = h2o_state;
   dp.lens_in = lens_dev;
   // eight CTAs per SM keep enough of the copy in flight: few units are split
-  // over several, each of at least 64 slots
+  // over several, each of at least 64 slots in the layers of the largest
+  // capacity (all are split alike; 32 layers of which one has 2,048 slots and 31
+  // have 64, init and a step: batch 1 66 us before the split, 24 now)
   int cap = 0;
   for (int l = 0; l < P.L; ++l) cap = std::max(cap, d.cap[l]);
   dp.init_split = std::max(1, std::min((8 * P.ctx.num_sms + d.units - 1) / d.units, cap / 64));

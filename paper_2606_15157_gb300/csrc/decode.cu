@@ -587,7 +587,8 @@ __global__ void __launch_bounds__(kDecodeThreads, kDecCtasPerSm) decode_step_ker
   extern __shared__ float lg[];
   __shared__ DecShared<kSplit> sh;
   // the H2O / TOVA units, and eight cheap units per CTA: after the others, or,
-  // split, before them (every CTA is resident at once, and those end first)
+  // split, before them (those end first and leave their places; as a rule all
+  // CTAs are resident at once, nothing depends on it)
   const int n_cheap_ctas = kSplit ? static_cast<int>(gridDim.x) - p.n_att * p.cluster : 0;
   const int n_att_ctas = kSplit ? 0 : p.n_att;
   const int b = static_cast<int>(blockIdx.x);

@@ -22,11 +22,20 @@ constexpr int kScoreNoH2O = 1;     // SnapKV layers only (H2O layers are scored 
 // work item (chunk), by how many items sweep 2 of an item runs behind its sweep
 // 1, and of how many chunks the records are merged into one before they are
 // published (when a unit has more).
-//   R_pad <= 128: the sweeps move a tile faster than HBM delivers it, so K has
-//     to be in L2 still when sweep 2 reads it again: 2 x 152 x 320 KB are
-//     between the reads.  One 8,192-token prompt, 32 SnapKV layers: 10 tiles and
-//     lag 1 140 us, 12 and 1 159, 8 and 1 171, 16 and 1 173, 10 and 2 166, 8 and
-//     2 183, 16 and 2 175 (8 tiles leave the normaliser too little time).
+//   R_pad <= 128: the sweeps move a tile faster than HBM delivers it, so K
+//     should be in L2 still when sweep 2 reads it again, and the smaller the
+//     items, the more evenly the CTAs are dealt; but the normaliser needs its
+//     time.  32 SnapKV layers, 32-row window, us a call with 10 tiles and lag 1,
+//     16 and 2, 12 and 1, 8 and 1, 10 and 2:
+//       prompts x length     10/1  16/2  12/1   8/1  10/2
+//       1 x  2,048             89    88    96    95    94
+//       1 x  4,096            122   136   127   127   129
+//       1 x  8,192            179   212   197   202   204
+//       1 x 16,384            321   376   341   334   363
+//       1 x 32,768            574   678   624   586   676
+//       8 x  2,048            444   493   485   454   497
+//       8 x  8,192          1,156 1,433 1,266 1,295 1,396
+//       4 x 16,384          1,123 1,362 1,223 1,171 1,331
 //   R_pad > 128: the softmax warps are the pace and an item reloads 64 KB of Q:
 //     eight prompts of 16K-32K, 16 tiles and lag 2 3.98 ms, 16 and 1 4.06, 12
 //     and 1 4.10, 20 and 1 4.09, 12 and 2 4.25; groups of 8 4.01, of 32 4.16
@@ -339,10 +348,12 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
 
 // ---- programmatic dependent launch ---------------------------------------------
 // A kernel launched with the programmatic attribute may start while the kernels
-// before it on the stream still run: it waits (pdl_wait) before it touches any
-// memory, so that only its launch and its parameter reads overlap them.  A
-// kernel lets its successor start as soon as all of its own CTAs have
-// (pdl_trigger), which saves most of the 2-3 us between two launches.
+// before it on the stream still run, which may be writing whatever it reads: up
+// to pdl_wait only its parameters are read and lines sent to L2 (prefetches into
+// L2, which read nothing into the SM; never loads or prefetches into L1).  A
+// kernel lets its successor in once all of its own CTAs have called pdl_trigger
+// or ended: at its start, which saves most of the 2-3 us between two launches,
+// or at its end (the decode step), where the successor's CTAs would get in its way.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -348,7 +348,7 @@ __device__ __forceinline__ bool slot_wait(const ScoreParams& p, const Smem& sm, 
 // and after: one 8,192-token prompt, 32 rows x 4 heads 239 and 173 us (4.5 and
 // 6.2 TB/s of K for the two sweeps); one 30,011-token prompt, 64 x 4 627 and
 // 576 us; eight of 16K-32K 4.25 and 4.01 ms; with the normalisers supplied,
-// four of them 1.02 and 0.90 ms (6.1 TB/s, 0.91 of the measured copy rate).
+// four of them 1.02 and 0.90 ms (5.3 TB/s, 0.78 of the measured copy rate).
 
 // NH: 128-row groups of the window rows (R_pad <= 128 NH).  Sweep 2 units hold
 // one 128-key tile x up to 256 rows (NH = 2), of which warpgroup w takes rows
@@ -393,7 +393,8 @@ __device__ __forceinline__ void softmax_wg(const ScoreParams& p, const Smem& sm,
       // One unit per (256-key super-tile, 128-row group): this warpgroup's 64
       // keys of the super-tile, for the thread's row of the group.  Rows that
       // do not exist (tr < 0) are computed like the others and dropped when
-      // the warpgroup publishes; a warp without rows only releases the unit.
+      // the warpgroup publishes; in the loop without checks a warp without rows
+      // only releases the unit.
       const int nst = (it.ntiles + 1) / 2;
       // the super-tiles whose every key is visible to every row come first
       const int nfull = min(nst, max(0, it.n - p.W + 1 - it.key0) / kSuperKeys);

@@ -51,7 +51,7 @@
 //      at most 32 candidates are ranked with shuffles instead;
 //   4. every warp merges its staged positions and its kept candidates into
 //      its share of the output, after the shares of the warps before it.
-// An end bin, or a candidate list that overflows (many equal keys), takes the
+// An end bin, or more candidates than the lists hold (many equal keys), takes the
 // general path instead: the full keys are written to the row (transposed
 // 128-key blocks), four 8-bit radix passes over every key fix T, and one
 // ordered pass writes the kept positions.
@@ -1007,6 +1007,9 @@ cudaError_t launch_select(const SelectParams& p, int grid, int num_sms, cudaStre
   // passes are chains of L2 round trips and barriers, which more threads
   // shorten while the SMs have room.  One 8,192-token prompt (256 units): 18.5
   // us with 256 threads, 15.2 with 512, 28 with 1,024 (two rounds of units).
+  // Up to one unit per SM 1,024 threads gain over 512 only on long rows (16
+  // units, the call: 16,384 keys 18.8 and 19.5 us, 8,192 16.6 and 16.7, 300 to
+  // 4,096 the same within the clock's 2 us, or 2 behind).
   if (grid <= num_sms)
     return launch_overlapped(select_kernel<1024>, p, grid, 1024, 0, s);
   if (grid <= 2 * num_sms) return launch_overlapped(select_kernel<512>, p, grid, 512, 0, s);
