@@ -1007,9 +1007,9 @@ cudaError_t launch_select(const SelectParams& p, int grid, int num_sms, cudaStre
   // passes are chains of L2 round trips and barriers, which more threads
   // shorten while the SMs have room.  One 8,192-token prompt (256 units): 18.5
   // us with 256 threads, 15.2 with 512, 28 with 1,024 (two rounds of units).
-  // Up to one unit per SM 1,024 threads gain over 512 only on long rows (16
-  // units, the call: 16,384 keys 18.8 and 19.5 us, 8,192 16.6 and 16.7, 300 to
-  // 4,096 the same within the clock's 2 us, or 2 behind).
+  // Up to one unit per SM 1,024 threads gain over 512 only on long rows: the
+  // call replayed, 8 units of 16,384 keys 18.8 and 19.5 us, of 300 to 8,192
+  // 14.6-16.6 and 14.5-14.8; 128 units of 300 to 8,192 16.8-18.6 and 16.5-17.2.
   if (grid <= num_sms)
     return launch_overlapped(select_kernel<1024>, p, grid, 1024, 0, s);
   if (grid <= 2 * num_sms) return launch_overlapped(select_kernel<512>, p, grid, 512, 0, s);
