@@ -1043,15 +1043,15 @@ int dec_att_cap(const kvev_plan& P, const DecLayout& d) {
 // load round trips for one CTA (16 slots per warp and trip), so while the units
 // leave CTA slots of the GPU empty each is split, as long as every warp still
 // has a tile of 16 slots.  Per step, 32 layers of which 7 are H2O with 2,048
-// slots, 8 KV heads, one CTA per unit and split: batch 1 24.5 and 13.0 us (eight
-// CTAs), batch 2 26.4 and 18.5 (four), batch 4 31.6 and 28.5 (two).
-// Below kMinSplitSlots the cluster's barriers cost what the split gains, for any
-// group, head size and number of units (16 steps, batch 1, groups of four, one
-// CTA and the split that was taken: 256 slots 131 and 146 us, 384 156 and 159,
-// 512 182 and 174, 1,024 274 and 213; batch 3, 256 slots, 188 and 205).
+// slots, 8 KV heads, one CTA per unit and split: batch 1 22.7 and 12.3 us (eight
+// CTAs), batch 2 24.4 and 17.8 (four), batch 4 29.9 and 27.5 (two).
+// Below kMinSplitSlots the cluster's barriers cost what the split gains (16
+// steps, batch 1, groups of four, one CTA and split: 256 slots 123 and 132 us,
+// 384 150 and 145, 512 177 and 159, 1,024 270 and 206; groups of one, 256 slots,
+// batch 1 with d = 64 90 and 109, batch 3 157 and 174).
 // At most three CTAs per SM of the four that fit leaves room for the
 // StreamingLLM and append-only units' CTAs; four measured the same or better
-// (144 units of 1,024 slots, two and four CTAs each, 280 and 265 us).
+// (144 units of 1,024 slots, two and four CTAs each, 272 and 254 us).
 // Not with the attention supplied: a unit is then a few loads per thread
 // (batch 1, 512 slots: one CTA 5.8 us, split 6.4).
 int dec_cluster(int n_att, int cap, int num_sms) {

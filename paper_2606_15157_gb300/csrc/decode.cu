@@ -562,7 +562,7 @@ __device__ void step_cheap_warp(const DecodeParams& p, int i, int D) {
 // are read at the end of the step's chain of round trips, and from HBM when the
 // caller wrote them some time ago.  Measured with 32 steps' tokens laid out
 // beforehand, 2,048 slots: batch 1 13.4 and 13.0 us a step, batch 16 91.6 and
-// 90.6; 512 slots with the attention supplied, batch 8: 8.2 and 7.5.
+// 90.6; with the attention supplied, batch 8: 8.2 and 7.5.
 __device__ __forceinline__ void prefetch_l2(const void* base, size_t bytes, size_t at) {
   if (at < bytes) asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const char*>(base) + at));
 }
@@ -607,9 +607,9 @@ __global__ void __launch_bounds__(kDecodeThreads, kDecCtasPerSm) decode_step_ker
   }
   // The next kernel's CTAs come in as this one's finish.  Let in at the start of
   // the step they were placed beside CTAs with most of their work ahead, and
-  // stayed there: 16 steps of 256 units of 256 slots 169 us, from here 152 (164
-  // for one CTA per unit and launches in order); 168 units of 512 slots in
-  // clusters of two 271 and 255 (289); 256 units of 64 slots 105 and 110 (122).
+  // stayed there: 16 steps of 256 units of 256 slots 166 us, from here 147; 168
+  // units of 512 slots in clusters of two 263 and 247; 256 units of 64 slots 99
+  // and 105.
   pdl_trigger();
   // The last CTA of the step to finish advances every sequence by one token:
   // every other CTA has read lens before it counted itself done.
